@@ -173,7 +173,9 @@ lbm_status lbm_cde_set_velocity(lbm_cde_t h, int32_t kind, const float* a_dev,
  * and resets the step counter to 0. */
 lbm_status lbm_cde_set_phi(lbm_cde_t h, const float* phi_dev);
 
-/* Advances nsteps time steps (asynchronous; one kernel launch per step). */
+/* Advances nsteps time steps (asynchronous; one kernel launch per step, or per
+ * several D2Q9 steps with the default launch shape, see lbm_cde_set_launch:
+ * the state after nsteps does not depend on how they are grouped). */
 lbm_status lbm_cde_step(lbm_cde_t h, int64_t nsteps);
 
 /* Sets the launch shape of the step kernel: block threads per CTA along x
@@ -195,9 +197,14 @@ lbm_status lbm_cde_step(lbm_cde_t h, int64_t nsteps);
  * planes z - 1 .. z + 1 and the offsets each step pulls staged in shared
  * memory by asynchronous copies; needs nx % 64 == 0, ny a multiple of
  * block / 32, 18 ncell < 2^31 and 16-byte aligned offsets, phi and velocity
- * fields. A shape
+ * fields. vec 10 with block 128 selects the fused steps of D2Q9 (any storage,
+ * walls on any face; 12 ncell < 2^31), which are also what a handle starts with:
+ * a launch takes up to eight steps, on tiles in shared memory (alone: vec 12),
+ * or on large grids four steps by warps that walk down strips of the grid
+ * (alone: vec 11); a single step and what does not qualify run one node per
+ * thread. Their states equal those of vec 1 bit for bit. A shape
  * whose field does not meet these runs the one-node kernel, and so does every
- * shape when the x or z faces carry walls.
+ * other shape when the x or z faces carry walls.
  * Results do not depend on the shape beyond FP32 rounding order. Errors:
  * LBM_E_ARG. */
 lbm_status lbm_cde_set_launch(lbm_cde_t h, int32_t block, int32_t vec);

@@ -64,7 +64,9 @@ struct lbm_cde_s {
     int* status_dev = nullptr;
     long long wait_limit = 4000000000LL;   // SM cycles per bounded device wait (about 2 s)
     int zwalk = 0;                         // z-walk kernel: planes per CTA (0: automatic)
-    int sms = 152;                         // multiprocessors of the device (adjoint grid)
+    int sms = 152;                         // multiprocessors of the device (adjoint grid, fused steps)
+    lbm::FusePlan plan{0, 0};              // fused steps of a long run (fuse_plan) for plan_kinds
+    int plan_kinds = 0;
     // per-phase device time of the last backward sweep (lbm_cde_set_profiling)
     bool prof = false;
     double prof_ms[3] = {0, 0, 0};
@@ -281,6 +283,34 @@ static int ukind_internal(int k)
     return k == LBM_U_FIELD ? lbm::U_FIELD : (k == LBM_U_ROW_PROFILE ? lbm::U_ROW : lbm::U_NONE);
 }
 
+static bool fused_ok(lbm_cde_t h)
+{
+    return lbm::fused_ok(h->q, h->ncell);
+}
+
+// How the next of `left` steps run. Launch vec 0 (the default) and 10: the plan
+// of the grid's size; 11: the walk kernel; 12: the tile kernel; the others take
+// one step a launch.
+static lbm::FusePlan fuse_plan(lbm_cde_t h, int64_t left)
+{
+    const int v = h->cfg.vec;
+    if (!fused_ok(h) || left < 2 || !(v == 0 || (v >= 10 && v <= 12))) return {1, 0};
+    const int kinds = v == 11 ? lbm::FUSE_WALK : (v == 12 ? lbm::FUSE_TILE : lbm::FUSE_ANY);
+    if (left < lbm::TILE_T) return lbm::plan_fused(h->d.storage, (int)h->d.nx, (int)h->d.ny, h->sms, left, kinds);
+    if (h->plan_kinds != kinds) {   // the plan of a long run is kept
+        h->plan = lbm::plan_fused(h->d.storage, (int)h->d.nx, (int)h->d.ny, h->sms, lbm::TILE_T, kinds);
+        h->plan_kinds = kinds;
+    }
+    return h->plan;
+}
+
+static cudaError_t launch_fused(lbm_cde_t h, lbm::FusePlan p, int uk, const StepArgs& a, void* const* mid,
+                                cudaStream_t st)
+{
+    return p.rows > 0 ? lbm::launch_tile(h->d.storage, uk, p.T, p.rows, a, mid, st)
+                      : lbm::launch_walk(h->d.storage, uk, p.T, a, mid, st);
+}
+
 // ---------------------------------------------------------------------------
 // C ABI
 // ---------------------------------------------------------------------------
@@ -416,7 +446,7 @@ lbm_status lbm_cde_create(const lbm_cde_desc* desc, lbm_cde_t* out)
     }
     // launch shape: 256 threads along x, cells per thread chosen for the row length
     h->cfg.block = d.nx >= 256 ? 256 : (d.nx >= 128 ? 128 : 64);
-    h->cfg.vec = 1;
+    h->cfg.vec = 0;   // fused steps where they apply, else one node per thread
     *out = h;
     return LBM_OK;
 }
@@ -525,12 +555,21 @@ lbm_status lbm_cde_step(lbm_cde_t h, int64_t nsteps)
         const lbm_status ts = ensure_tma_maps(h);
         if (ts != LBM_OK) return ts;
     }
-    for (int64_t n = 0; n < nsteps; ++n) {
+    for (int64_t n = 0; n < nsteps;) {
         StepArgs a = make_args(h, h->cur);
+        const lbm::FusePlan plan = fuse_plan(h, nsteps - n);
+        if (plan.T > 1) {
+            CK(h, launch_fused(h, plan, uk, a, nullptr, h->st));
+            h->cur ^= 1;
+            h->t += plan.T;
+            n += plan.T;
+            continue;
+        }
         if (tma) a.tma = &h->tmaps[h->cur];
         CK(h, lbm::launch_step(h->q, h->d.storage, uk, walls, h->cfg, a, h->st));
         h->cur ^= 1;
         h->t += 1;
+        ++n;
     }
     return LBM_OK;
 }
@@ -568,6 +607,13 @@ lbm_status lbm_cde_set_launch(lbm_cde_t h, int32_t block, int32_t vec)
         if (block != 128 || !tma)
             return fail(h, LBM_E_ARG, "vec 7 / 8 (TMA-staged D2Q9 16-bit kernel) needs block 128, "
                                       "nx % 256 == 0 and 12 ncell < 2^31");
+        h->cfg.block = block;
+        h->cfg.vec = vec;
+        return LBM_OK;
+    }
+    if (vec >= 10 && vec <= 12) {
+        if (block != 128 || !fused_ok(h))
+            return fail(h, LBM_E_ARG, "vec 10 / 11 / 12 (fused steps) needs D2Q9, block 128 and 12 ncell < 2^31");
         h->cfg.block = block;
         h->cfg.vec = vec;
         return LBM_OK;
@@ -683,6 +729,7 @@ lbm_status lbm_cde_autotune(lbm_cde_t h, int64_t steps, int32_t* block_out, int3
         cand.push_back(LaunchCfg{128, 7});
         cand.push_back(LaunchCfg{128, 8});
     }
+    if (fused_ok(h)) cand.push_back(LaunchCfg{128, 10});   // fused steps
     for (size_t ci = 0; ci < cand.size() && s == LBM_OK; ++ci) {
         h->cfg = cand[ci];
         s = lbm_cde_set_state(h, save, t0);
@@ -981,10 +1028,12 @@ lbm_status lbm_cde_forward_ckpt(lbm_cde_t h, const float* phi0_dev, int64_t nste
     s = lbm_cde_set_phi(h, phi0_dev);
     if (s != LBM_OK) return s;
     CK(h, cudaMemcpyAsync(h->ck[0], h->state[h->cur], sb, cudaMemcpyDeviceToDevice, h->st));
-    for (int64_t k = 1; k <= nsteps; ++k) {
-        s = lbm_cde_step(h, 1);
+    for (int64_t k = 0; k < nsteps;) {
+        const int64_t n = std::min(every, nsteps - k);
+        s = lbm_cde_step(h, n);
         if (s != LBM_OK) return s;
-        if (k % every == 0 && k < nsteps)
+        k += n;
+        if (k < nsteps)
             CK(h, cudaMemcpyAsync(h->ck[k / every], h->state[h->cur], sb, cudaMemcpyDeviceToDevice, h->st));
     }
     if (phiN_dev) {
@@ -1066,12 +1115,20 @@ lbm_status lbm_cde_backward(lbm_cde_t h, const float* dL_dphiN_dev, float* dL_dp
     // recompute B_{jK+1} .. B_{end-1} of segment j from its checkpoint, on stream rs
     auto recompute = [&](int64_t j, cudaStream_t rs) -> lbm_status {
         const int64_t start = j * K, end = std::min(start + K, Nst);
-        for (int64_t t = 1; t < end - start; ++t) {
+        for (int64_t t = 1; t < end - start;) {
+            const lbm::FusePlan plan = fuse_plan(h, end - start - t);
             StepArgs a = make_args(h, 0);
             a.src = seg_state(j, t - 1);
-            a.dst = seg_state(j, t);
+            a.dst = seg_state(j, t + plan.T - 1);
             set_step(a, start + t);
-            CK(h, lbm::launch_step(h->q, LBM_STORE_F32, uk, walls, h->cfg, a, rs));
+            if (plan.T > 1) {
+                void* mid[lbm::TILE_T];
+                for (int f = 0; f < plan.T - 1; ++f) mid[f] = seg_state(j, t + f);
+                CK(h, launch_fused(h, plan, uk, a, mid, rs));
+            } else {
+                CK(h, lbm::launch_step(h->q, LBM_STORE_F32, uk, walls, h->cfg, a, rs));
+            }
+            t += plan.T;
         }
         return LBM_OK;
     };

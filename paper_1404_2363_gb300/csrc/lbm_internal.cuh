@@ -102,6 +102,47 @@ struct StepArgs {
     int zwalk;            // D3Q15 z-walk kernel: planes per CTA (0: chosen by the launcher)
 };
 
+// Several fused D2Q9 steps (lbm_walk_d2q9.cuh).
+struct WalkArgs {
+    StepArgs a;          // src: state k - 1; dst: state k - 1 + T
+    int srow[5];         // schedule rows of u(k - 1) .. u(k - 1 + T), or -1
+    void* mid[3];        // SAVE: the states k .. k + T - 2 (FP32)
+    int strips, ranges;  // strips of walk_cols(T) columns x ranges of rows
+    int vec;             // pairs are stored as one word (nx even, aligned planes)
+    int wide;            // rows are staged by 16-byte copies (nx a multiple of 4, or 8 for 16-bit planes; aligned)
+};
+
+// Steps of the D2Q9 model on tiles in shared memory (lbm_tile_d2q9.cuh).
+constexpr int TILE_T = 8;        // most steps of one launch
+constexpr int TILE_ROWS = 64;    // most rows of a tile
+struct TileArgs {
+    StepArgs a;              // src: state k - 1; dst: state k - 1 + T
+    int srow[TILE_T + 1];    // schedule rows of u(k - 1) .. u(k - 1 + T), or -1
+    void* mid[TILE_T - 1];   // FP32: where the states between go, or NULL
+    int T;                   // steps
+    int rows;                // tile: 64 columns x rows, the halo of T on each side included
+    int field;               // a.ua is a field (else a row profile, or NULL)
+};
+
+// The fused D2Q9 steps need int offsets.
+inline bool fused_ok(int q, long long ncell) { return q == 9 && 12LL * ncell < (1LL << 31); }
+
+constexpr int WALK_HALO = 4;     // columns of a warp's 64 lost on each side: at least T, and a multiple of 4 so
+                                 // that strips start on 16-byte boundaries
+constexpr int WALK_COLS = 64 - 2 * WALK_HALO;
+
+// Ranges of rows of the walk kernel for at most `warps` resident warps per SM,
+// and its time of one launch in us (cost, may be NULL). Measured on GB300: a row
+// takes about 0.45 us + 0.47 us k at T = 4 with k >= 1 warps per scheduler
+// (1024^2: 0.92, 1.33, 1.87 us at k = 1, 2, 3); a range of R rows walks R + 2 T.
+int walk_ranges(int strips, int ny, int T, int sms, int warps, double* cost);
+
+// How the next of `left` D2Q9 steps run: T steps by one launch of the one-step
+// kernel (T = 1), of the walk kernel (rows = 0) or of the tile kernel (rows of a tile).
+struct FusePlan { int T, rows; };
+enum { FUSE_WALK = 1, FUSE_TILE = 2, FUSE_ANY = 3 };   // kernels the plan may take (one: at least two steps by it)
+FusePlan plan_fused(int store, int nx, int ny, int sms, long long left, int kinds = FUSE_ANY);
+
 // One reverse-time step (lbm_adjoint.cu).
 struct AdjArgs {
     const float* mu_in;   // adjoint of the post-collision state B_k [q][ncell]
@@ -189,6 +230,11 @@ struct LaunchCfg {
 // Kernel launchers (lbm_kernels.cu). Each returns the cudaError_t of the launch.
 cudaError_t launch_step(int q, int store, int ukind, bool walls, LaunchCfg cfg,
                         const StepArgs& a, cudaStream_t st);
+// T (2 or 4) fused D2Q9 steps from a.src to a.dst; mid: the T - 1 states between
+// (FP32 storage), or nullptr
+cudaError_t launch_walk(int store, int ukind, int T, const StepArgs& a, void* const* mid, cudaStream_t st);
+// T (1 .. TILE_T) D2Q9 steps on tiles of the given rows in shared memory, likewise
+cudaError_t launch_tile(int store, int ukind, int T, int rows, const StepArgs& a, void* const* mid, cudaStream_t st);
 cudaError_t launch_init(int q, int store, int ukind, const float* phi0, const StepArgs& a,
                         cudaStream_t st);
 cudaError_t launch_phi(int q, int store, const StepArgs& a, float* phi_out, cudaStream_t st);

@@ -1,0 +1,105 @@
+"""The kernels that take several D2Q9 steps per launch (launch vec 10, 11, 12 and
+the default) against the one-step kernel, bit for bit: they run the same
+operations in the same order, so the whole state has to be equal, at the edges
+of their strips, tiles and row ranges, for every wall kind, velocity kind,
+storage form and alignment."""
+import numpy as np
+import pytest
+import torch
+
+from _common import Case, assert_parity, run_oracle
+from paper_1404_2363_gb300.solver import Solver
+
+pytestmark = pytest.mark.gpu
+
+# nx: below, at and past the 56 columns of a strip and the 48 .. 60 of a tile; multiples of 8, 4 and 2, and odd
+# (16-byte copies, paired stores, neither). ny: fewer rows than the halo of eight, tile remainders, several ranges
+SIZES = [(5, 3), (8, 9), (56, 129), (57, 21), (64, 40), (127, 18), (300, 37), (114, 70)]
+Y = [("periodic", "periodic"), ("noflux", "bounceback"), ("bounceback", "noflux"), ("dirichlet", "bounceback"),
+     ("noflux", "dirichlet")]
+X = [("periodic", "periodic"), ("noflux", "bounceback"), ("bounceback", "noflux")]
+
+
+def state(case, shape, steps):
+    s = Solver(nx=case.nx, ny=case.ny, storage=case.storage, bc=case.bc, bc_x=case.bc_x, phi_w=case.phi_w,
+               model=case.model)
+    if shape is not None:
+        s.set_launch(*shape)
+    s.set_D(case.D)
+    phi0, a, sched = case.inputs()
+    if a is not None:
+        s.set_velocity(torch.from_numpy(a).cuda(), None if sched is None else torch.from_numpy(sched).cuda(),
+                       kind="row" if case.ukind == "row" else "field")
+    s.set_phi(torch.from_numpy(phi0).cuda())
+    for n in steps:
+        s.step(n)
+    g, t = s.get_state()
+    g = g.cpu().numpy()
+    s.close()
+    assert t == sum(steps)
+    return g
+
+
+@pytest.mark.parametrize("storage", ["f32", "f16", "bf16"])
+@pytest.mark.parametrize("nx,ny", SIZES)
+def test_fused_steps_equal_single_steps(storage, nx, ny):
+    for j, (bc, bx) in enumerate((bc, bx) for bc in Y for bx in X):
+        uk = ("field", "row", "none")[j % 3] if bx[0] == "periodic" else "field"
+        model = ("A", "B1", "B3")[j % 3] if storage == "f32" and "dirichlet" not in bc else "A"
+        case = Case(nx=nx, ny=ny, storage=storage, bc=bc, bc_x=bx, ukind=uk, phi_w=(0.7, 0.3), model=model, umax=0.02)
+        ref = state(case, (128, 1), [15])      # 8 + 7, 4 x 3 + 2 + 1
+        for shape in ((128, 11), (128, 12), None):
+            got = state(case, shape, [15])
+            assert np.array_equal(got, ref), (shape, bc, bx, uk, model)
+
+
+@pytest.mark.parametrize("storage", ["f32", "bf16"])
+def test_fused_steps_do_not_depend_on_their_grouping(storage):
+    case = Case(nx=200, ny=61, storage=storage)
+    ref = state(case, (128, 1), [41])
+    for shape in ((128, 11), (128, 12), (128, 10), None):
+        for steps in ([41], [1] * 5 + [2, 3, 4, 5, 6, 7, 9], [40, 1], [8, 33]):
+            assert np.array_equal(state(case, shape, steps), ref), (shape, steps)
+
+
+@pytest.mark.parametrize("shape", [(128, 11), (128, 12)])
+def test_fused_steps_match_oracle(O, shape):
+    case = Case(nx=181, ny=53, steps=120, bc=("noflux", "bounceback"), bc_x=("bounceback", "noflux"))
+    phi0, a, sched = case.inputs()
+    g = state(case, shape, [case.steps]).view(np.float32).reshape(9, case.ny, case.nx)
+    assert_parity(g.astype(np.float64).sum(0), run_oracle(O, case, phi0, a, sched), 1e-5)
+
+
+def test_fused_steps_on_an_unaligned_velocity_field():
+    """A velocity field that starts 4 bytes past a 16-byte boundary: no 16-byte copies, the same state."""
+    nx, ny = 112, 40
+    case = Case(nx=nx, ny=ny, sched=False)
+    phi0, a, _ = case.inputs()
+    buf = torch.zeros(2 * nx * ny + 1, device="cuda")
+    buf[1:] = torch.from_numpy(a).cuda().reshape(-1)
+    out = []
+    for shape in ((128, 1), (128, 11), (128, 12)):
+        s = Solver(nx=nx, ny=ny)
+        s.set_launch(*shape)
+        s.set_D(case.D)
+        s.set_velocity(buf[1:].reshape(2, ny, nx))
+        s.set_phi(torch.from_numpy(phi0).cuda())
+        s.step(14)
+        out.append(s.get_state()[0].cpu().numpy())
+        s.close()
+    assert np.array_equal(out[0], out[1]) and np.array_equal(out[0], out[2])
+
+
+def test_fused_launch_shapes_are_checked():
+    from paper_1404_2363_gb300 import _native as N
+
+    s = Solver(lattice=15, nx=16, ny=16, nz=4)
+    for vec in (10, 11, 12):
+        with pytest.raises(N.LbmError):
+            s.set_launch(128, vec)
+    s.close()
+    s = Solver(nx=16, ny=16)
+    for block, vec in ((256, 10), (128, 0), (128, 13)):
+        with pytest.raises(N.LbmError):
+            s.set_launch(block, vec)
+    s.close()
