@@ -29,7 +29,7 @@
 
 #include "../../include/lbm_cde.h"
 #include "lbm_device.cuh"
-#include "lbm_pair.cuh"
+#include "lbm_walk_d2q9.cuh"
 
 namespace lbm {
 
@@ -416,6 +416,189 @@ __global__ void __launch_bounds__(256) k_batch_cells(const __grid_constant__ Cel
     if (threadIdx.x < 32) tile_column_sum(cs, a.strip + (long long)(a.tile_base + t) * 32);
 }
 
+// PER_STEP mode, several steps per launch (the walk of lbm_walk_d2q9.cuh): a
+// warp owns 64 columns of a channel, 56 of them kept, and walks down its rows
+// through T = 4 levels whose states stay in registers. A row enters through a ring
+// in shared memory, three rows in flight. Every level forms the 32 x 16 cell tiles'
+// column sums in the order of k_batch_cells (the rows r and r + 8 first, then the
+// eight pairs in row order), so that fields and moments have its bits; the eight
+// sums' first halves wait in shared memory.
+// One step a launch is bound by HBM (72 B a node and step); a range is a whole
+// channel's height where there are enough warps (walls need no halo rows), else a
+// multiple of 16 rows.
+struct BatchTask {
+    int inst;          // instance within the launch
+    int strip0;        // first of the CTA's WALK_WARPS strips
+    int ya, yb;        // rows [ya, yb)
+};
+
+struct BatchWalkArgs {
+    CellArgs c;                  // koff: steps before this launch; strip: the sums of its first step
+    const BatchTask* tasks;
+    long long strip_step;        // floats from one step's sums to the next
+    int second;                  // of the two launches of eight steps
+};
+
+constexpr int BWALK_T = 4;
+constexpr int BWALK_ROW = 9 * 256;                                                // bytes of a staged row
+constexpr int BWALK_WARP = WALK_ROWS * BWALK_ROW + BWALK_T * 8 * 256;             // and the waiting row sums
+
+__global__ void __launch_bounds__(32 * WALK_WARPS, 3) k_batch_walk(const __grid_constant__ BatchWalkArgs p)
+{
+    constexpr int T = BWALK_T, HALO = WALK_HALO;
+    extern __shared__ __align__(16) unsigned char bwalk_sm[];
+    grid_dep_launch();
+    grid_dep_wait();
+    const BatchTask tk = p.tasks[blockIdx.x];
+    const InstK& I = p.c.inst[tk.inst];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int nx = I.nx, ny = I.ny, N = (int)p.c.ncat;
+    const int strip = tk.strip0 + warp;
+    if (strip * WALK_COLS >= nx) return;
+    const int from = (int)((*p.c.kdev + p.c.koff) & 1) ^ p.second;   // B_{k-1} in buf[(k-1) & 1] after every second launch
+    const float* const src = p.c.buf[from] + I.off;
+    float* const dst = p.c.buf[1 - from] + I.off;
+    const int x0 = strip * WALK_COLS - HALO + 2 * lane;
+    int c0 = x0 % nx;
+    c0 = c0 < 0 ? c0 + nx : c0;
+    const int c1 = c0 + 1 == nx ? 0 : c0 + 1;
+    const bool mine = lane >= HALO / 2 && lane < 32 - HALO / 2 && x0 < nx;
+    const bool ywall = I.bc_lo != BC_PERIODIC;
+    const int ya = tk.ya, yb = tk.yb;
+    const int rs = ywall ? max(ya - T, 0) : ya - T, re = yb - 1 + T;
+    const bool even = (I.off & 1) == 0 && (N & 1) == 0;   // rows of even offset have aligned pairs
+    unsigned char* const sm = bwalk_sm + warp * BWALK_WARP + 8 * lane;
+    unsigned char* const held = sm + WALK_ROWS * BWALK_ROW;
+    auto wrap = [&](int y) {
+        if (ywall) return min(max(y, 0), ny - 1);
+        return ((y % ny) + ny) % ny;
+    };
+    auto issue = [&](int r) {
+        if (r <= re) {
+            const int row = wrap(r) * nx;
+            const bool v8 = even && ((row + c0) & 1) == 0 && c1 != 0;
+            unsigned char* st = sm + (r & (WALK_ROWS - 1)) * BWALK_ROW;
+#pragma unroll
+            for (int i = 0; i < 9; ++i) {
+                const float* q = src + i * N + row;
+                if (v8) walk_copy<8>(st + 256 * i, q + c0);
+                else {
+                    walk_copy<4>(st + 256 * i, q + c0);
+                    walk_copy<4>(st + 256 * i + 4, q + c1);
+                }
+            }
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    WalkLevel lv[T];
+    float ux[T + 1], uy[T + 1];   // velocities of the rows r .. r - T
+    float2 acc[T];
+#pragma unroll
+    for (int s = 0; s < T; ++s) {
+        acc[s] = sp2(0.f);
+#pragma unroll
+        for (int j = 0; j < 3; ++j) lv[s].c0[j] = lv[s].pa[j] = lv[s].pb[j] = sp2(0.f);
+    }
+#pragma unroll
+    for (int s = 0; s <= T; ++s) ux[s] = uy[s] = 0.f;
+#pragma unroll 1
+    for (int j = 0; j < WALK_AHEAD; ++j) issue(rs + j);
+
+    auto row_step = [&](int r, auto par) {
+        constexpr bool ODD = decltype(par)::value != 0;
+        float2 n[9];
+        asm volatile("cp.async.wait_group %0;" ::"n"(WALK_AHEAD - 1) : "memory");
+        const unsigned char* st = sm + (r & (WALK_ROWS - 1)) * BWALK_ROW;
+#pragma unroll
+        for (int i = 0; i < 9; ++i) n[i] = *reinterpret_cast<const float2*>(st + 256 * i);
+        issue(r + WALK_AHEAD);
+#pragma unroll
+        for (int s = T; s > 0; --s) ux[s] = ux[s - 1], uy[s] = uy[s - 1];
+        if (I.urow) {
+            const int y = wrap(r);
+            ux[0] = __ldg(I.urow + y);
+            uy[0] = __ldg(I.urow + ny + y);
+        }
+#pragma unroll
+        for (int s = 1; s <= T; ++s) {
+            WalkLevel& lw = lv[s - 1];
+            float2(&p1)[3] = ODD ? lw.pb : lw.pa;
+            float2(&p2)[3] = ODD ? lw.pa : lw.pb;
+            const int y = r - s;
+            float2 f[9];
+            f[0] = lw.c0[0];
+            f[1] = walk_from_left(lw.c0[1]);
+            f[3] = walk_from_right(lw.c0[2]);
+            f[2] = p2[0];
+            f[5] = walk_from_left(p2[1]);
+            f[6] = walk_from_right(p2[2]);
+            f[4] = n[4];
+            f[7] = walk_from_right(n[7]);
+            f[8] = walk_from_left(n[8]);
+            const bool lo = ywall && y == 0, hi = ywall && y == ny - 1;
+            if (lo || hi) {
+                const int kind = lo ? I.bc_lo : I.bc_hi;
+                if (kind == BC_BOUNCE) {
+                    if (lo) f[2] = p2[0], f[5] = p2[1], f[6] = p2[2];   // stashed when row 0 came in
+                    else f[4] = p1[0], f[7] = p1[1], f[8] = p1[2];
+                } else {
+                    if (lo) f[2] = f[4], f[5] = f[8], f[6] = f[7];
+                    else f[4] = f[2], f[8] = f[5], f[7] = f[6];
+                }
+            }
+            p2[0] = n[2], p2[1] = n[5], p2[2] = n[6];
+            lw.c0[0] = n[0], lw.c0[1] = n[1], lw.c0[2] = n[3];
+            if (ywall && y == -1 && I.bc_lo == BC_BOUNCE) p1[0] = n[4], p1[1] = n[7], p1[2] = n[8];
+            const float2 phi = collide_pair_f32(f, sp2(ux[s]), sp2(uy[s]), I.c);
+#pragma unroll
+            for (int i = 0; i < 9; ++i) n[i] = f[i];
+            if (y < ya || y >= yb) continue;
+            // column sums of the cell tiles
+            const float2 wp = lo || hi ? make_float2(__fmul_rn(0.5f, phi.x), __fmul_rn(0.5f, phi.y)) : phi;
+            const int q = y & 15;
+            auto hold = [&](int j) -> float2& { return *reinterpret_cast<float2*>(held + ((s - 1) * 8 + j) * 256); };
+            if (q < 8) hold(q) = wp;
+            else {
+                const float2 h = hold(q - 8);
+                const float2 v = make_float2(__fadd_rn(h.x, wp.x), __fadd_rn(h.y, wp.y));
+                acc[s - 1] = q == 8 ? v : make_float2(__fadd_rn(acc[s - 1].x, v.x), __fadd_rn(acc[s - 1].y, v.y));
+            }
+            if (q == 15 || y == ny - 1) {
+                float2 sum = acc[s - 1];
+                for (int j = q < 8 ? 0 : q - 7; j < (q < 8 ? q + 1 : 8); ++j) {   // rows without a partner
+                    const float2 h = hold(j);
+                    sum = j == 0 ? h : make_float2(__fadd_rn(sum.x, h.x), __fadd_rn(sum.y, h.y));
+                }
+                if (mine) {
+                    const long long tile = p.c.tile_base + I.tile0 + (long long)(y >> 4) * I.tx + (x0 >> 5);
+                    float* o = p.c.strip + (s - 1) * p.strip_step + tile * 32 + (x0 & 31);
+                    o[0] = sum.x;
+                    if (x0 + 1 < nx) o[1] = sum.y;
+                }
+            }
+            if (s == T && mine) {
+                float* o = dst + y * nx + x0;
+                if (even && ((y * nx) & 1) == 0 && x0 + 1 < nx) {
+#pragma unroll
+                    for (int i = 0; i < 9; ++i) *reinterpret_cast<float2*>(o + i * N) = f[i];
+                } else {
+                    const bool two = x0 + 1 < nx;
+#pragma unroll
+                    for (int i = 0; i < 9; ++i) {
+                        o[i * N] = f[i].x;
+                        if (two) o[i * N + 1] = f[i].y;
+                    }
+                }
+            }
+        }
+    };
+#pragma unroll 1
+    for (int r = rs; r <= re; r += 2) {
+        row_step(r, std::integral_constant<int, 0>{});
+        row_step(r + 1, std::integral_constant<int, 1>{});
+    }
+}
+
 // Eq. 47 moments of step k for PER_STEP mode, two deterministic passes.
 // Pass 1: one thread per column x of an instance (256-column blocks, each
 // within one instance): phi-bar(x) = FP64 sum of the column's tile sums, then
@@ -458,9 +641,11 @@ __device__ __forceinline__ void col_moments(const BatchArgs& a, long long k, int
 
 __global__ void __launch_bounds__(256) k_batch_col_moments(const BatchArgs a, const float* __restrict__ strip,
                                                            const int* __restrict__ cblk_inst,
-                                                           double* __restrict__ cpart, int koff)
+                                                           double* __restrict__ cpart, int koff, long long strip_step)
 {
-    col_moments(a, *a.kdev + 1 + koff, blockIdx.x, strip, cblk_inst, cpart);
+    // step koff + blockIdx.y of the launch, its sums strip_step floats after the last one's
+    col_moments(a, *a.kdev + 1 + koff + blockIdx.y, blockIdx.x, strip + blockIdx.y * strip_step, cblk_inst,
+                cpart + 3LL * gridDim.x * blockIdx.y);
 }
 
 // Pass 2 for instance i (one warp): block partials added in index order with a
@@ -490,11 +675,11 @@ __device__ __forceinline__ void inst_moments(const BatchArgs& a, long long k, in
 }
 
 __global__ void __launch_bounds__(256) k_batch_inst_moments(const BatchArgs a, const double* __restrict__ cpart,
-                                                            int koff)
+                                                            int ncblk, int koff)
 {
     const int i = (int)((blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5);
     if (i >= a.ninst) return;
-    inst_moments(a, *a.kdev + 1 + koff, i, cpart);
+    inst_moments(a, *a.kdev + 1 + koff + blockIdx.y, i, cpart + 3LL * ncblk * blockIdx.y);
 }
 
 // PERSISTENT mode on cell tiles (tile height 0): one cooperative launch runs
@@ -636,6 +821,11 @@ struct StepStreams {
     cudaEvent_t cells_done;       // recorded after the cell launches of a step
     cudaEvent_t moments_done[2];  // after the moment passes of a step, by step parity
     float* strip2;                // the column sums of the odd steps
+    // the walk launches (none: one step a launch)
+    const BatchTask* tasks;       // of every launch of a step, one after the other
+    const int* ntasks;            // CTAs of each
+    float* wstrip[2];             // [BWALK_T][cell tiles][32] column sums, by launch parity
+    double* wcpart[2];            // [BWALK_T][ncblk][3]
 };
 
 // rows > 0: PERSISTENT on warp tiles of that height; rows == 0: on cell tiles
@@ -682,11 +872,30 @@ static cudaError_t launch_mode(int mode, int rows, const BatchArgs& a, const Ins
     // writes its column sums to the strip buffer of its parity, and leaves its two
     // moment passes to st2, so that they overlap the cells of step s + 1; the
     // cells of step s + 2 wait for the moment passes of step s (the strip buffer).
+    // Two walk launches take eight steps (B_t stays in buf[t & 1]); the rest run one
+    // by one. `u` counts the units launched: a unit's moment passes use the buffers of its parity.
     cudaError_t e = cudaSuccess;
-    for (int s = 0; s < a.nsteps && e == cudaSuccess; ++s) {
-        float* sb = (s & 1) ? ss.strip2 : strip;
-        if (s >= 2) e = cudaStreamWaitEvent(st, ss.moments_done[s & 1], 0);
+    int u = 0;
+    for (int s = 0; s < a.nsteps && e == cudaSuccess; ++u) {
+        const bool walk = ss.tasks != nullptr && i32 && s < (a.nsteps & ~7);
+        const int n = walk ? BWALK_T : 1;
+        float* sb = walk ? ss.wstrip[u & 1] : ((u & 1) ? ss.strip2 : strip);
+        double* cp = walk ? ss.wcpart[u & 1] : cpart + ((u & 1) ? 3LL * ncblk : 0);
+        if (u >= 2) e = cudaStreamWaitEvent(st, ss.moments_done[u & 1], 0);
+        const BatchTask* tasks = ss.tasks;
         for (size_t g = 0; g < cells.size() && e == cudaSuccess; ++g) {
+            if (walk) {
+                BatchWalkArgs w{};
+                w.c = cells[g];
+                w.c.strip = sb;
+                w.c.koff = s;
+                w.tasks = tasks;
+                w.strip_step = 32LL * nctiles;
+                w.second = (s & 7) == 4;
+                e = launch_dependent(k_batch_walk, dim3((unsigned)ss.ntasks[g]), 32 * WALK_WARPS, WALK_WARPS * BWALK_WARP, st, w);
+                tasks += ss.ntasks[g];
+                continue;
+            }
             CellArgs ca = cells[g];
             ca.strip = sb;
             ca.koff = s;
@@ -697,14 +906,15 @@ static cudaError_t launch_mode(int mode, int rows, const BatchArgs& a, const Ins
         if (e == cudaSuccess) e = cudaEventRecord(ss.cells_done, st);
         if (e == cudaSuccess) e = cudaStreamWaitEvent(ss.st2, ss.cells_done, 0);
         if (e != cudaSuccess) break;
-        k_batch_col_moments<<<(unsigned)ncblk, 256, 0, ss.st2>>>(a, sb, cblk_inst, cpart, s);
-        k_batch_inst_moments<<<(unsigned)((a.ninst + 7) / 8), 256, 0, ss.st2>>>(a, cpart, s);
+        k_batch_col_moments<<<dim3((unsigned)ncblk, (unsigned)n), 256, 0, ss.st2>>>(a, sb, cblk_inst, cp, s, 32LL * nctiles);
+        k_batch_inst_moments<<<dim3((unsigned)((a.ninst + 7) / 8), (unsigned)n), 256, 0, ss.st2>>>(a, cp, ncblk, s);
         e = cudaGetLastError();
-        if (e == cudaSuccess) e = cudaEventRecord(ss.moments_done[s & 1], ss.st2);
+        if (e == cudaSuccess) e = cudaEventRecord(ss.moments_done[u & 1], ss.st2);
+        s += n;
     }
     if (e != cudaSuccess) return e;
     // the last moment passes (and with them every earlier one) before the advance
-    if (a.nsteps > 0) e = cudaStreamWaitEvent(st, ss.moments_done[(a.nsteps - 1) & 1], 0);
+    if (u > 0) e = cudaStreamWaitEvent(st, ss.moments_done[(u - 1) & 1], 0);
     if (e != cudaSuccess) return e;
     k_batch_advance<<<1, 1, 0, st>>>(kdev, a.nsteps);
     return cudaGetLastError();
@@ -745,6 +955,8 @@ struct lbm_cde_batch_s {
     std::vector<int> cell_tiles;        // cell tiles of each launch
     float* strip = nullptr;             // [cell tiles][32] column sums (even steps in PER_STEP mode)
     lbm::StepStreams ss{};              // PER_STEP: moment stream, events, odd-step column sums
+    lbm::BatchTask* tasks = nullptr;    // walk launches: the CTAs' tasks, group by group
+    std::vector<int> ntasks;
     int* cblk_inst = nullptr;           // instance of each 256-column block of the moment pass
     int ncblk = 0;
     double* cpart = nullptr;            // [2][ncblk][3] moment partials (PER_STEP uses the first)
@@ -925,6 +1137,75 @@ static lbm_status rebuild_tiles(lbm_cde_batch_t b)
     return LBM_OK;
 }
 
+// Tasks and buffers of the walk launches, where they pay: the time of four steps
+// by the walk's rule (walk_ranges: a row takes 0.45 + 0.47 k us at k warps per
+// scheduler, at most three) against that of four one-step launches (4.1 us each,
+// or 72 bytes a node at 6 TB/s).
+static lbm_status setup_walk(lbm_cde_batch_t b)
+{
+    if (9LL * b->ncat >= (1LL << 31)) return LBM_OK;
+    int dev = 0, sms = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1) {
+        cudaGetLastError();
+        return LBM_OK;
+    }
+    const int T = lbm::BWALK_T;
+    auto strips = [&](const lbm::InstDev& I) { return (I.nx + lbm::WALK_COLS - 1) / lbm::WALK_COLS; };
+    long long warps = 0;
+    for (const lbm::InstDev& I : b->inst) warps += strips(I);
+    // ranges of a channel: enough for two warps per scheduler, at least 16 rows each
+    const long long want = 8LL * sms;
+    const int split = (int)std::max<long long>(1, (want + warps - 1) / warps);
+    std::vector<lbm::BatchTask> all;
+    double rows = 0, longest = 0, used = 0;
+    b->ntasks.clear();
+    for (int g0 = 0; g0 < b->n; g0 += lbm::CELL_INST) {
+        std::vector<lbm::BatchTask> t;
+        for (int j = 0; j < std::min(lbm::CELL_INST, b->n - g0); ++j) {
+            const lbm::InstDev& I = b->inst[g0 + j];
+            const int blocks = (I.ny + 15) / 16, nr = std::min(split, blocks);
+            for (int q = 0; q < nr; ++q) {
+                const int ya = 16 * (blocks * q / nr), yb = std::min(16 * (blocks * (q + 1) / nr), I.ny);
+                for (int s0 = 0; s0 < strips(I); s0 += lbm::WALK_WARPS) t.push_back({j, s0, ya, yb});
+                rows += (double)strips(I) * (yb - ya + 2 * T);
+                longest = std::max(longest, (double)(yb - ya + 2 * T));
+                used += strips(I);
+            }
+        }
+        std::stable_sort(t.begin(), t.end(), [](const lbm::BatchTask& x, const lbm::BatchTask& y) {
+            return x.yb - x.ya > y.yb - y.ya;   // long walks first
+        });
+        b->ntasks.push_back((int)t.size());
+        all.insert(all.end(), t.begin(), t.end());
+    }
+    const double slots = 4.0 * sms, k = std::min(3.0, std::max(1.0, used / slots));
+    const double walk = std::max(rows / (slots * k), longest) * (0.45 + 0.47 * k) + 1.5;
+    const double single = T * std::max(4.1, b->ncat * 72 / 6.0e6);
+    if (walk >= single) {
+        b->ntasks.clear();
+        return LBM_OK;
+    }
+    b->tasks = static_cast<lbm::BatchTask*>(balloc(b, sizeof(lbm::BatchTask) * all.size()));
+    bool ok = b->tasks != nullptr;
+    for (int p = 0; p < 2 && ok; ++p) {
+        b->ss.wstrip[p] = static_cast<float*>(balloc(b, sizeof(float) * 32 * (size_t)b->nctiles * T));
+        b->ss.wcpart[p] = static_cast<double*>(balloc(b, sizeof(double) * 3 * (size_t)b->ncblk * T));
+        ok = b->ss.wstrip[p] && b->ss.wcpart[p];
+    }
+    if (!ok) return LBM_E_OOM;
+    if (cudaFuncSetAttribute(lbm::k_batch_walk, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             lbm::WALK_WARPS * lbm::BWALK_WARP) != cudaSuccess)
+        return LBM_E_CUDA;
+    if (cudaMemcpyAsync(b->tasks, all.data(), sizeof(lbm::BatchTask) * all.size(), cudaMemcpyHostToDevice, b->st) !=
+            cudaSuccess ||
+        cudaStreamSynchronize(b->st) != cudaSuccess)
+        return LBM_E_CUDA;
+    b->ss.tasks = b->tasks;
+    b->ss.ntasks = b->ntasks.data();
+    return LBM_OK;
+}
+
 extern "C" {
 
 lbm_status lbm_cde_batch_opts_init(lbm_cde_batch_opts* o)
@@ -1102,6 +1383,10 @@ lbm_status lbm_cde_batch_create(const lbm_cde_channel_desc* descs, int32_t n, co
         cudaMemcpyAsync(b->tile_inst, ti.data(), sizeof(int) * ti.size(), cudaMemcpyHostToDevice, b->st);
         cudaStreamSynchronize(b->st);
     }
+    if (lbm_status ws = setup_walk(b); ws != LBM_OK) {
+        lbm_cde_batch_destroy(b);
+        return bfail(nullptr, ws, "walk setup failed");
+    }
     cudaMemsetAsync(b->sync, 0, 64, b->st);
     lbm_status s = rebuild_tiles(b);
     if (s != LBM_OK) {
@@ -1127,6 +1412,11 @@ lbm_status lbm_cde_batch_destroy(lbm_cde_batch_t b)
     bfree(b, b->moments);
     bfree(b, b->strip);
     bfree(b, b->ss.strip2);
+    bfree(b, b->tasks);
+    for (int p = 0; p < 2; ++p) {
+        bfree(b, b->ss.wstrip[p]);
+        bfree(b, b->ss.wcpart[p]);
+    }
     if (b->ss.st2) {
         cudaStreamSynchronize(b->ss.st2);
         cudaStreamDestroy(b->ss.st2);

@@ -103,3 +103,31 @@ def test_fused_launch_shapes_are_checked():
         with pytest.raises(N.LbmError):
             s.set_launch(block, vec)
     s.close()
+
+
+def test_batch_walk_equals_one_step_launches():
+    """Several batch steps per launch (PER_STEP mode on batches large enough for it) against the persistent
+    cell tiles, which take one step at a time: fields and moments bit for bit, over odd and even row lengths,
+    heights off the 16-row tiles, every wall pair and model, with and without a velocity; 21 steps are two
+    groups of eight and five single ones, in chunks of 16."""
+    from paper_1404_2363_gb300.batch import Batch, poiseuille_row
+
+    g = np.random.default_rng(5)
+    walls = [("noflux", "noflux"), ("bounceback", "bounceback"), ("periodic", "periodic"), ("noflux", "bounceback"),
+             ("bounceback", "noflux")]
+    chs, phis = [], []
+    for i in range(48):
+        nx, ny = int(g.integers(1500, 2600)), int(g.integers(30, 90))
+        chs.append({"nx": nx, "ny": ny, "bc": walls[i % 5], "D": [[0.03, 0.004], [0.004, 0.05]],
+                    "u_row": poiseuille_row(ny, 0.08) if i % 7 else None, "x_ref0": float(round(0.2 * nx)),
+                    "x_ref_velocity": 0.05, "model": ("A", "B1", "B2", "B3")[i % 4]})
+        phis.append((0.05 + g.random((ny, nx))).astype(np.float32))
+    out = []
+    for mode in ("persistent", "per_step"):
+        b = Batch(chs, mode=mode, tile_rows=0, graph_steps=16)
+        b.set_phi(phis)
+        m = b.run(21)
+        out.append((m, torch.cat([p.reshape(-1) for p in b.get_phi()])))
+        b.close()
+    assert np.array_equal(out[0][0], out[1][0])
+    assert torch.equal(out[0][1], out[1][1])
