@@ -57,9 +57,28 @@ constexpr int ADJ_ROWS = 8;
 
 int adjoint_rows(long long nx, long long ny, long long nz, int sms)
 {
+    const AdjBlock b = adjoint_block(nx);
     int rows = ADJ_ROWS;
-    while (rows > 1 && ((nx + 255) / 256) * ((ny + rows - 1) / rows) * nz < (long long)sms * 3) rows /= 2;
+    while (rows > 1 && ((nx + b.w - 1) / b.w) * ((ny + rows * b.h - 1) / (rows * b.h)) * nz < (long long)sms * 3) rows /= 2;
     return rows;
+}
+
+// Block shape: w columns (a multiple of 32, so that a warp stays in one row) x h
+// rows, at most 256 threads, with the fewest columns past the row's end, the
+// widest of those: 97 columns take 128 x 2 threads (D3Q15 97 x 80 x 66 with dL/da: 62 us
+// a step with 256 columns a block, 38 % of them in the row).
+AdjBlock adjoint_block(long long nx)
+{
+    AdjBlock best{256, 1};
+    long long waste = (nx + 255) / 256 * 256 - nx;
+    for (int w = 224; w >= 32; w -= 32) {
+        const long long r = (nx + w - 1) / w * w - nx;
+        if (r < waste) {
+            waste = r;
+            best = {w, 256 / w};
+        }
+    }
+    return best;
 }
 
 // DA: the velocity-field gradient is accumulated (UK == U_FIELD only); its
@@ -90,6 +109,7 @@ __global__ void __launch_bounds__(256, (L::Q == 9 && !DA && WM < 2) ? 4 : 3) k_a
     const int nx = a.nx, ny = a.ny, nz = a.nz;
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     const int z = blockIdx.z;
+    const int tid = threadIdx.y * blockDim.x + threadIdx.x;
     const IX N = (IX)a.ncell;
     const bool live = x < nx;
     const int xc = live ? x : nx - 1;
@@ -103,9 +123,9 @@ __global__ void __launch_bounds__(256, (L::Q == 9 && !DA && WM < 2) ? 4 : 3) k_a
 #pragma unroll
     for (int j = 0; j < NG; ++j) g[j] = 0.f;
 
-    const int y0 = blockIdx.y * a.rows;
+    const int y0 = blockIdx.y * a.rows * blockDim.y;   // the block's rows, blockDim.y at a time
 #pragma unroll 1
-    for (int y = y0; y < y0 + a.rows && y < ny; ++y) {
+    for (int y = y0 + threadIdx.y; y < y0 + a.rows * (int)blockDim.y && y < ny; y += blockDim.y) {
         const int ys[3] = {y + 1 == ny ? 0 : y + 1, y, y == 0 ? ny - 1 : y - 1};
         // row offsets of the source rows (y - e_y, z - e_z)
         IX roff[3][3];
@@ -384,11 +404,15 @@ __global__ void __launch_bounds__(256, (L::Q == 9 && !DA && WM < 2) ? 4 : 3) k_a
     // a shuffle tree over NG values)
     __shared__ float red[NG][256];
     __shared__ float seg[NG][8];
+    const int nt = blockDim.x * blockDim.y;
 #pragma unroll
-    for (int j = 0; j < NG; ++j) red[j][threadIdx.x] = g[j];
+    for (int j = 0; j < NG; ++j) {
+        red[j][tid] = g[j];
+        if (tid + nt < 256) red[j][tid + nt] = 0.f;   // at least 128 threads
+    }
     __syncthreads();
-    if ((int)threadIdx.x < 8 * NG) {
-        const int j = threadIdx.x >> 3, sg = threadIdx.x & 7;
+    for (int t = tid; t < 8 * NG; t += nt) {
+        const int j = t >> 3, sg = t & 7;
         const float* r = &red[j][sg * 32];
         float s = 0.f;
 #pragma unroll 8
@@ -396,13 +420,13 @@ __global__ void __launch_bounds__(256, (L::Q == 9 && !DA && WM < 2) ? 4 : 3) k_a
         seg[j][sg] = s;
     }
     __syncthreads();
-    if ((int)threadIdx.x < NG) {
+    if (tid < NG) {
         float s = 0.f;
 #pragma unroll
-        for (int sg = 0; sg < 8; ++sg) s += seg[threadIdx.x][sg];
+        for (int sg = 0; sg < 8; ++sg) s += seg[tid][sg];
         const long long blk = blockIdx.x + (long long)gridDim.x * (blockIdx.y + (long long)gridDim.y * blockIdx.z);
         const long long nb = (long long)gridDim.x * gridDim.y * gridDim.z;
-        a.partials[threadIdx.x * nb + blk] = s;   // [NG][nblocks]: coalesced in the reduction
+        a.partials[tid * nb + blk] = s;   // [NG][nblocks]: coalesced in the reduction
     }
 }
 
@@ -506,9 +530,10 @@ __global__ void k_adjoint_seed(const float* __restrict__ g, float* __restrict__ 
     }
 }
 
-static long long adj_blocks(const AdjArgs& a)
+static long long adj_blocks(long long nx, long long ny, long long nz, int rows)
 {
-    return (long long)((a.nx + 255) / 256) * ((a.ny + a.rows - 1) / a.rows) * a.nz;
+    const AdjBlock b = adjoint_block(nx);
+    return ((nx + b.w - 1) / b.w) * ((ny + rows * b.h - 1) / (rows * b.h)) * nz;
 }
 
 // grad_acc += the per-block partials of nslice slices starting at base, summed in a fixed order
@@ -516,7 +541,7 @@ template <class L>
 static cudaError_t grad_reduce(const AdjArgs& a, float* base, int nslice, long long slice, cudaStream_t st)
 {
     constexpr int NG = ngrad<L>();
-    const long long nb = adj_blocks(a);
+    const long long nb = adj_blocks(a.nx, a.ny, a.nz, a.rows);
     float2* p2 = reinterpret_cast<float2*>(base + (long long)ADJ_SLICES * slice);   // slice is even
     k_grad_sum2<<<dim3(GRAD_CHUNKS, NG), 256, 0, st>>>(base, nb, slice, NG, nslice, p2);
     k_grad_sum3<<<1, 64, 0, st>>>(p2, NG, a.grad_acc);
@@ -526,22 +551,25 @@ static cudaError_t grad_reduce(const AdjArgs& a, float* base, int nslice, long l
 template <class L, int UK, typename IX, int WM>
 static cudaError_t adj_wm(const AdjArgs& a, cudaStream_t st, bool reduce)
 {
-    dim3 grid((unsigned)((a.nx + 255) / 256), (unsigned)((a.ny + a.rows - 1) / a.rows), (unsigned)a.nz);
+    const AdjBlock bl = adjoint_block(a.nx);
+    const int rows = a.rows * bl.h;
+    dim3 grid((unsigned)((a.nx + bl.w - 1) / bl.w), (unsigned)((a.ny + rows - 1) / rows), (unsigned)a.nz);
+    const dim3 block((unsigned)bl.w, (unsigned)bl.h);
     // the u^2 terms of MRT-B1/B2 (zero coefficients for the other models; with no
     // velocity they vanish)
     constexpr bool QOK = L::Q == 9 && UK != U_NONE;
     const bool quad = QOK && (a.c.b1 != 0.f || a.c.g7 != 0.f);
     if constexpr (UK == U_FIELD) {
         if (a.du_acc != nullptr) {
-            if (quad) k_adjoint<L, UK, WM, true, IX, QOK><<<grid, 256, 0, st>>>(a);
-            else k_adjoint<L, UK, WM, true, IX, false><<<grid, 256, 0, st>>>(a);
+            if (quad) k_adjoint<L, UK, WM, true, IX, QOK><<<grid, block, 0, st>>>(a);
+            else k_adjoint<L, UK, WM, true, IX, false><<<grid, block, 0, st>>>(a);
             cudaError_t e = cudaGetLastError();
             if (e != cudaSuccess || !reduce) return e;
             return grad_reduce<L>(a, a.partials, 1, 0, st);
         }
     }
-    if (quad) k_adjoint<L, UK, WM, false, IX, QOK><<<grid, 256, 0, st>>>(a);
-    else k_adjoint<L, UK, WM, false, IX, false><<<grid, 256, 0, st>>>(a);
+    if (quad) k_adjoint<L, UK, WM, false, IX, QOK><<<grid, block, 0, st>>>(a);
+    else k_adjoint<L, UK, WM, false, IX, false><<<grid, block, 0, st>>>(a);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess || !reduce) return e;
     return grad_reduce<L>(a, a.partials, 1, 0, st);
@@ -588,7 +616,7 @@ cudaError_t launch_grad_reduce(int q, const AdjArgs& a, float* base, int nslice,
 long long adjoint_slice_size(int q, long long nx, long long ny, long long nz, int sms)
 {
     const int rows = adjoint_rows(nx, ny, nz, sms);
-    const long long nb = ((nx + 255) / 256) * ((ny + rows - 1) / rows) * nz;
+    const long long nb = adj_blocks(nx, ny, nz, rows);
     const long long f = nb * (q == 9 ? ngrad<D2Q9>() : ngrad<D3Q15>());
     return (f + 1) & ~1LL;
 }

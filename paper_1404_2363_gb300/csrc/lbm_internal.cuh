@@ -254,6 +254,8 @@ cudaError_t launch_adjoint_init(int q, int ukind, const AdjArgs& a, const float*
                                 cudaStream_t st);
 cudaError_t launch_adjoint_seed(const float* g, float* mu, long long ncell, int q, cudaStream_t st);
 long long adjoint_partials_size(int q, long long nx, long long ny, long long nz, int sms);   // in floats
+struct AdjBlock { int w, h; };   // threads of a block: columns x rows
+AdjBlock adjoint_block(long long nx);
 int adjoint_rows(long long nx, long long ny, long long nz, int sms);
 int adjoint_ngrad(int q);
 
