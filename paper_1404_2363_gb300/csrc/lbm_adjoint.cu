@@ -103,6 +103,8 @@ AdjBlock adjoint_block(long long nx)
 template <class L, int UK, int WM, bool DA, typename IX, bool QUAD>
 __global__ void __launch_bounds__(256, (L::Q == 9 && !DA && WM < 2) ? 4 : 3) k_adjoint(const AdjArgs a)
 {
+    grid_dep_launch();
+    grid_dep_wait();
     static_assert(!QUAD || (L::Q == 9 && UK != U_NONE), "u^2 terms only for D2Q9 with a velocity");
     constexpr bool WALLS = WM == 1, BOX = WM == 2;
     constexpr int Q = L::Q, DIM = L::DIM, NG = ngrad<L>();
@@ -561,16 +563,14 @@ static cudaError_t adj_wm(const AdjArgs& a, cudaStream_t st, bool reduce)
     const bool quad = QOK && (a.c.b1 != 0.f || a.c.g7 != 0.f);
     if constexpr (UK == U_FIELD) {
         if (a.du_acc != nullptr) {
-            if (quad) k_adjoint<L, UK, WM, true, IX, QOK><<<grid, block, 0, st>>>(a);
-            else k_adjoint<L, UK, WM, true, IX, false><<<grid, block, 0, st>>>(a);
-            cudaError_t e = cudaGetLastError();
+            const cudaError_t e = launch_dependent(quad ? k_adjoint<L, UK, WM, true, IX, QOK> : k_adjoint<L, UK, WM, true, IX, false>,
+                                                   grid, block, 0, st, a);
             if (e != cudaSuccess || !reduce) return e;
             return grad_reduce<L>(a, a.partials, 1, 0, st);
         }
     }
-    if (quad) k_adjoint<L, UK, WM, false, IX, QOK><<<grid, block, 0, st>>>(a);
-    else k_adjoint<L, UK, WM, false, IX, false><<<grid, block, 0, st>>>(a);
-    cudaError_t e = cudaGetLastError();
+    const cudaError_t e = launch_dependent(quad ? k_adjoint<L, UK, WM, false, IX, QOK> : k_adjoint<L, UK, WM, false, IX, false>,
+                                           grid, block, 0, st, a);
     if (e != cudaSuccess || !reduce) return e;
     return grad_reduce<L>(a, a.partials, 1, 0, st);
 }

@@ -892,7 +892,7 @@ static cudaError_t launch_mode(int mode, int rows, const BatchArgs& a, const Ins
                 w.tasks = tasks;
                 w.strip_step = 32LL * nctiles;
                 w.second = (s & 7) == 4;
-                e = launch_dependent(k_batch_walk, dim3((unsigned)ss.ntasks[g]), 32 * WALK_WARPS, WALK_WARPS * BWALK_WARP, st, w);
+                e = launch_dependent(k_batch_walk, dim3((unsigned)ss.ntasks[g]), dim3(32 * WALK_WARPS), WALK_WARPS * BWALK_WARP, st, w);
                 tasks += ss.ntasks[g];
                 continue;
             }

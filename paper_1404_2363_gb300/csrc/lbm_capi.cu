@@ -444,8 +444,10 @@ lbm_status lbm_cde_create(const lbm_cde_desc* desc, lbm_cde_t* out)
             h->sms = n;
         cudaGetLastError();
     }
-    // launch shape: 256 threads along x, cells per thread chosen for the row length
-    h->cfg.block = d.nx >= 256 ? 256 : (d.nx >= 128 ? 128 : 64);
+    // launch shape: threads along x, from 64 to 256, with the fewest past the row's end, the most of those
+    h->cfg.block = 256;
+    for (int w = 224; w >= 64; w -= 32)
+        if ((d.nx + w - 1) / w * w < (d.nx + h->cfg.block - 1) / h->cfg.block * h->cfg.block) h->cfg.block = w;
     h->cfg.vec = 0;   // fused steps where they apply, else one node per thread
     *out = h;
     return LBM_OK;

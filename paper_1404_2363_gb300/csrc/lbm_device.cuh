@@ -468,6 +468,8 @@ __device__ __forceinline__ void vel_ix(const StepArgs& a, IX N, IX cell, int y, 
 template <class L, int STORE, int UK, bool WALLS, int VEC, typename IX>
 __global__ void __launch_bounds__(256) k_step(const StepArgs a)
 {
+    grid_dep_launch();
+    grid_dep_wait();
     using T = typename StT<STORE>::T;
     constexpr int Q = L::Q;
     constexpr bool NEQ = (STORE != ST_F32);
@@ -588,6 +590,8 @@ __device__ __forceinline__ int reflect_mask(int i, int mask)
 template <class L, int STORE, int UK, typename IX>
 __global__ void __launch_bounds__(256) k_step_box(const StepArgs a)
 {
+    grid_dep_launch();
+    grid_dep_wait();
     using T = typename StT<STORE>::T;
     constexpr int Q = L::Q;
     constexpr bool NEQ = (STORE != ST_F32);

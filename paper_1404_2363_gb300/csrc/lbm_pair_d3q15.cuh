@@ -50,6 +50,8 @@ __device__ __forceinline__ float2 feq_unit_pair15(float w0, float wa, float wd, 
 template <int STORE, int UK, bool WALLS>
 __global__ void __launch_bounds__(256) k_step_pair_d3q15(const StepArgs a)
 {
+    grid_dep_launch();
+    grid_dep_wait();
     using P = Pair<STORE>;
     using T2 = typename P::T2;
     using L = D3Q15;

@@ -15,9 +15,9 @@ static cudaError_t step_vec(LaunchCfg cfg, const StepArgs& a, cudaStream_t st)
     if (a.bcx_lo != BC_PERIODIC || a.bcz_lo != BC_PERIODIC) {
         // walls on the x or z faces: the general one-node kernel, whatever the launch shape
         dim3 grid((unsigned)((a.nx + 255) / 256), (unsigned)a.ny, (unsigned)a.nz);
-        if ((long long)(L::Q + 3) * a.ncell < (1LL << 31)) k_step_box<L, STORE, UK, int><<<grid, 256, 0, st>>>(a);
-        else k_step_box<L, STORE, UK, long long><<<grid, 256, 0, st>>>(a);
-        return cudaGetLastError();
+        if ((long long)(L::Q + 3) * a.ncell < (1LL << 31))
+            return launch_dependent(k_step_box<L, STORE, UK, int>, grid, dim3(256), 0, st, a);
+        return launch_dependent(k_step_box<L, STORE, UK, long long>, grid, dim3(256), 0, st, a);
     }
     if constexpr (L::Q == 9) {
         if (cfg.vec == 6 && quad_ok(a, UK)) {
@@ -36,8 +36,7 @@ static cudaError_t step_vec(LaunchCfg cfg, const StepArgs& a, cudaStream_t st)
             // node-pair variant (paired FP32 arithmetic, two adjacent nodes per thread)
             const int per = 2 * cfg.block;
             dim3 grid((unsigned)((a.nx + per - 1) / per), (unsigned)a.ny, (unsigned)a.nz);
-            k_step_pair_d3q15<STORE, UK, WALLS><<<grid, cfg.block, 0, st>>>(a);
-            return cudaGetLastError();
+            return launch_dependent(k_step_pair_d3q15<STORE, UK, WALLS>, grid, dim3((unsigned)cfg.block), 0, st, a);
         }
     }
     if constexpr (L::Q == 9 && STORE != ST_F32) {
@@ -58,14 +57,11 @@ static cudaError_t step_vec(LaunchCfg cfg, const StepArgs& a, cudaStream_t st)
     dim3 block((unsigned)cfg.block);
     // 32-bit offsets when every plane and velocity offset fits
     const bool idx32 = (long long)(L::Q + 3) * a.ncell < (1LL << 31);
-    if (idx32) {
-        if (vec == 2) k_step<L, STORE, UK, WALLS, 2, int><<<grid, block, 0, st>>>(a);
-        else k_step<L, STORE, UK, WALLS, 1, int><<<grid, block, 0, st>>>(a);
-    } else {
-        if (vec == 2) k_step<L, STORE, UK, WALLS, 2, long long><<<grid, block, 0, st>>>(a);
-        else k_step<L, STORE, UK, WALLS, 1, long long><<<grid, block, 0, st>>>(a);
-    }
-    return cudaGetLastError();
+    if (idx32)
+        return vec == 2 ? launch_dependent(k_step<L, STORE, UK, WALLS, 2, int>, grid, block, 0, st, a)
+                        : launch_dependent(k_step<L, STORE, UK, WALLS, 1, int>, grid, block, 0, st, a);
+    return vec == 2 ? launch_dependent(k_step<L, STORE, UK, WALLS, 2, long long>, grid, block, 0, st, a)
+                    : launch_dependent(k_step<L, STORE, UK, WALLS, 1, long long>, grid, block, 0, st, a);
 }
 
 template <class L, int STORE, int UK>

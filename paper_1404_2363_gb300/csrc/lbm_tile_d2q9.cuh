@@ -287,7 +287,7 @@ cudaError_t tile_d2q9(const TileArgs& p, cudaStream_t st)
     }
     const dim3 grid((unsigned)((p.a.nx + 64 - 2 * p.T - 1) / (64 - 2 * p.T)),
                     (unsigned)((p.a.ny + p.rows - 2 * p.T - 1) / (p.rows - 2 * p.T)));
-    return launch_dependent(k_tile_d2q9<STORE, WALLS>, grid, TILE_THREADS, tile_smem(p.rows), st, p);
+    return launch_dependent(k_tile_d2q9<STORE, WALLS>, grid, dim3(TILE_THREADS), tile_smem(p.rows), st, p);
 }
 
 }  // namespace lbm

@@ -141,29 +141,6 @@ __device__ __forceinline__ void walk_feq(const Coef& c, float2 ux, float2 uy, fl
     e[6] = fma2(sp2(-c.kd), d, sp2(c.wd));
 }
 
-// Waits for the kernels this launch depends on (programmatic dependent launch),
-// and lets the next one start its prologue.
-__device__ __forceinline__ void grid_dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-__device__ __forceinline__ void grid_dep_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-
-// A launch that may start while the stream's previous kernel drains: it waits
-// in grid_dep_wait() before it reads anything.
-template <class A>
-cudaError_t launch_dependent(void (*kernel)(A), dim3 grid, int threads, int smem, cudaStream_t st, const A& args)
-{
-    cudaLaunchConfig_t cfg{};
-    cfg.gridDim = grid;
-    cfg.blockDim = dim3((unsigned)threads);
-    cfg.dynamicSmemBytes = (size_t)smem;
-    cfg.stream = st;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kernel, args);
-}
-
 constexpr int WALK_WARPS = 4;    // independent warps per CTA
 __host__ __device__ constexpr int walk_minb(int T) { return T <= 2 ? 4 : 3; }   // 128 / 168 registers
 
@@ -541,7 +518,7 @@ cudaError_t walk_d2q9(WalkArgs& p, cudaStream_t st)
     p.strips = (p.a.nx + WALK_COLS - 1) / WALK_COLS;
     p.ranges = walk_ranges(p.strips, p.a.ny, T, sms[dev], per_sm[dev] * WALK_WARPS, nullptr);
     const int ctas = (p.strips * p.ranges + WALK_WARPS - 1) / WALK_WARPS;
-    return launch_dependent(k_walk_d2q9<STORE, FIELD, WALLS, T, SAVE>, dim3((unsigned)ctas), 32 * WALK_WARPS, smem, st, p);
+    return launch_dependent(k_walk_d2q9<STORE, FIELD, WALLS, T, SAVE>, dim3((unsigned)ctas), dim3(32 * WALK_WARPS), smem, st, p);
 }
 
 template <int STORE, bool FIELD, int T, bool SAVE>

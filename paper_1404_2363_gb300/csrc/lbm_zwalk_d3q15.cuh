@@ -93,6 +93,8 @@ __device__ __forceinline__ void zw_issue_g(const uint16_t* __restrict__ g, uint1
 template <int STORE, int UK, bool WALLS, int TY>
 __global__ void __launch_bounds__(32 * TY, TY == 8 ? 3 : 6) k_step_zw_d3q15(const StepArgs a)
 {
+    grid_dep_launch();
+    grid_dep_wait();
     using Gm = ZwGeom<TY>;
     constexpr int PLANE = Gm::PLANE, CHUNKS = Gm::CHUNKS, GPOS = Gm::GPOS;
     using P = Pair<STORE>;
@@ -334,9 +336,8 @@ cudaError_t launch_zw_d3q15(const StepArgs& a, cudaStream_t st)
             }
         }
     }
-    k_step_zw_d3q15<STORE, UK, WALLS, TY>
-        <<<dim3((unsigned)(a.nx / ZW_TX), (unsigned)(a.ny / TY), (unsigned)nb), threads, smem, st>>>(a);
-    return cudaGetLastError();
+    return launch_dependent(k_step_zw_d3q15<STORE, UK, WALLS, TY>,
+                            dim3((unsigned)(a.nx / ZW_TX), (unsigned)(a.ny / TY), (unsigned)nb), dim3(threads), smem, st, a);
 }
 
 }  // namespace lbm
