@@ -101,10 +101,15 @@ AdjBlock adjoint_block(long long nx)
 // a compile-time choice: behind a run-time test the kernel executed 7 % more
 // instructions for the other models, which never take them.
 template <class L, int UK, int WM, bool DA, typename IX, bool QUAD>
-__global__ void __launch_bounds__(256, (L::Q == 9 && !DA && WM < 2) ? 4 : 3) k_adjoint(const AdjArgs a)
+__global__ void __launch_bounds__(256, (L::Q == 9 && !DA && WM < 2) ? 4 : 3) k_adjoint(const AdjArgs args)
 {
+    AdjArgs a = args;
     grid_dep_launch();
     grid_dep_wait();
+    a.mu_in = after_dep(a.mu_in);
+    a.fprev = after_dep(a.fprev);
+    a.ua = after_dep(a.ua);
+    a.sched = after_dep(a.sched);
     static_assert(!QUAD || (L::Q == 9 && UK != U_NONE), "u^2 terms only for D2Q9 with a velocity");
     constexpr bool WALLS = WM == 1, BOX = WM == 2;
     constexpr int Q = L::Q, DIM = L::DIM, NG = ngrad<L>();

@@ -449,13 +449,14 @@ __global__ void __launch_bounds__(32 * WALK_WARPS, 3) k_batch_walk(const __grid_
     extern __shared__ __align__(16) unsigned char bwalk_sm[];
     grid_dep_launch();
     grid_dep_wait();
-    const BatchTask tk = p.tasks[blockIdx.x];
+    const BatchTask tk = after_dep(p.tasks)[blockIdx.x];
     const InstK& I = p.c.inst[tk.inst];
+    const float* const urow = after_dep(I.urow);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int nx = I.nx, ny = I.ny, N = (int)p.c.ncat;
     const int strip = tk.strip0 + warp;
     if (strip * WALK_COLS >= nx) return;
-    const int from = (int)((*p.c.kdev + p.c.koff) & 1) ^ p.second;   // B_{k-1} in buf[(k-1) & 1] after every second launch
+    const int from = (int)((*after_dep(p.c.kdev) + p.c.koff) & 1) ^ p.second;   // B_{k-1} in buf[(k-1) & 1] after every second launch
     const float* const src = p.c.buf[from] + I.off;
     float* const dst = p.c.buf[1 - from] + I.off;
     const int x0 = strip * WALK_COLS - HALO + 2 * lane;
@@ -514,10 +515,10 @@ __global__ void __launch_bounds__(32 * WALK_WARPS, 3) k_batch_walk(const __grid_
         issue(r + WALK_AHEAD);
 #pragma unroll
         for (int s = T; s > 0; --s) ux[s] = ux[s - 1], uy[s] = uy[s - 1];
-        if (I.urow) {
+        if (urow) {
             const int y = wrap(r);
-            ux[0] = __ldg(I.urow + y);
-            uy[0] = __ldg(I.urow + ny + y);
+            ux[0] = __ldg(urow + y);
+            uy[0] = __ldg(urow + ny + y);
         }
 #pragma unroll
         for (int s = 1; s <= T; ++s) {

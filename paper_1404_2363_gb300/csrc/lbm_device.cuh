@@ -275,6 +275,23 @@ __device__ __forceinline__ float populations(const float (&a)[L::Q], float (&v)[
     }
 }
 
+// v_1 .. v_8 of D2Q9 from the isotropic parts A (axis) and B (diagonal), these with
+// the stress rows added and taken (AP, AM, BP, BM), and the flux parts of the axis
+// (X, Y) and diagonal (Xd, Yd) populations; v_1 + ... + v_8 = 4 (A + B).
+__device__ __forceinline__ void populations9(float (&v)[9], float AP, float AM, float BP, float BM, float X,
+                                             float Xd, float Y, float Yd)
+{
+    const float XY = Xd + Yd, XmY = Xd - Yd;
+    v[1] = AP + X;
+    v[3] = AP - X;
+    v[2] = AM + Y;
+    v[4] = AM - Y;
+    v[5] = BP + XY;
+    v[7] = BP - XY;
+    v[6] = BM - XmY;
+    v[8] = BM + XmY;
+}
+
 // ---------------------------------------------------------------------------
 // Collision in moment space for one node (Eq. 11, 13 with Eq. 31 / A.5, 14).
 // On return f holds the post-collision populations f' (OFFSET = false) or
@@ -288,60 +305,53 @@ __device__ __forceinline__ float collide(float (&f)[L::Q], float ux, float uy, f
 {
     constexpr int Q = L::Q;
     if constexpr (L::Q == 15) return collide_d3q15<float, OFFSET>(f, ux, uy, uz, c);   // MRT-A only
-    float m[Q];
-    moments<L>(f, m);
-    const float phi = m[0];
     if constexpr (OFFSET && L::Q == 9) {
         // offsets of the 16-bit forms (linear equilibria only): with dl = m - m^eq,
         // a = diag(1/|M_k|^2) (I - S) dl, the rates and scales folded in c.ro, c.fr
+        float m[9];
+        moments<L>(f, m);
+        const float phi = m[0];
         const float dl1 = fmaf(-c.meq1, phi, m[1]), dl2 = fmaf(-c.meq2, phi, m[2]);
         const float dl3 = fmaf(-phi, ux, m[3]), dl4 = fmaf(phi, ux, m[4]);
         const float dl5 = fmaf(-phi, uy, m[5]), dl6 = fmaf(phi, uy, m[6]);
-        float a[9];
-        a[0] = 0.f;
-        a[1] = __fmul_rn(dl1, c.ro[1]);
-        a[2] = __fmul_rn(dl2, c.ro[2]);
-        a[4] = __fmul_rn(dl4, c.ro[4]);
-        a[6] = __fmul_rn(dl6, c.ro[6]);
-        a[7] = __fmul_rn(m[7], c.ro[7]);
-        a[8] = __fmul_rn(m[8], c.ro[8]);
-        a[3] = fmaf(c.fr[0], dl3, fmaf(c.fr[1], dl4, fmaf(c.fr[2], dl5, __fmul_rn(c.fr[3], dl6))));
-        a[5] = fmaf(c.fr[4], dl3, fmaf(c.fr[5], dl4, fmaf(c.fr[6], dl5, __fmul_rn(c.fr[7], dl6))));
-        f[0] = fmaf(-c.eps0, phi, -populations<L, true, false>(a, f));
+        const float a1 = __fmul_rn(dl1, c.ro[1]), a2 = __fmul_rn(dl2, c.ro[2]);
+        const float a4 = __fmul_rn(dl4, c.ro[4]), a6 = __fmul_rn(dl6, c.ro[6]);
+        const float a3 = fmaf(c.fr[0], dl3, fmaf(c.fr[1], dl4, fmaf(c.fr[2], dl5, __fmul_rn(c.fr[3], dl6))));
+        const float a5 = fmaf(c.fr[4], dl3, fmaf(c.fr[5], dl4, fmaf(c.fr[6], dl5, __fmul_rn(c.fr[7], dl6))));
+        const float A = fmaf(-2.f, a2, -a1), B = fmaf(2.f, a1, a2);
+        populations9(f, fmaf(c.ro[7], m[7], A), fmaf(-c.ro[7], m[7], A), fmaf(c.ro[8], m[8], B),
+                     fmaf(-c.ro[8], m[8], B), fmaf(-2.f, a4, a3), fmaf(c.ro[4], dl4, a3), fmaf(-2.f, a6, a5),
+                     fmaf(c.ro[6], dl6, a5));
+        // sum_i g_i = -phi eps0 balances the FP32 weights of the decode, which sum
+        // to 1 + eps0 (else the mass would drift by phi eps0 per step)
+        f[0] = fmaf(-c.eps0, phi, -__fmul_rn(4.f, A + B));
         return phi;
     }
-    const float u[3] = {ux, uy, uz};
-    // dl = m - m^eq_lin (Eq. 15 / A.3 with c1 = 1, c2 from Eq. 16 / A.4: linear in u);
-    // d = dl - (u^2 terms of the MRT-B1/B2 equilibria, zero otherwise)
-    float dl[Q], d[Q];
-    dl[0] = d[0] = 0.f;
-    dl[1] = fmaf(-c.meq1, phi, m[1]);
-    dl[2] = fmaf(-c.meq2, phi, m[2]);
-    d[1] = dl[1];
-    d[2] = dl[2];
+    // f' = M^-1 (m - S (m - m^eq))
+    float m[Q], d[Q];
+    moments<L>(f, m);
+    const float phi = m[0], u[3] = {ux, uy, uz};
+    d[0] = 0.f;
+    d[1] = fmaf(-c.meq1, phi, m[1]);
+    d[2] = fmaf(-c.meq2, phi, m[2]);
 #pragma unroll
     for (int a = 0; a < L::DIM; ++a) {
-        d[3 + 2 * a] = dl[3 + 2 * a] = fmaf(-phi, u[a], m[3 + 2 * a]);
-        d[4 + 2 * a] = dl[4 + 2 * a] = fmaf(phi, u[a], m[4 + 2 * a]);
+        d[3 + 2 * a] = fmaf(-phi, u[a], m[3 + 2 * a]);
+        d[4 + 2 * a] = fmaf(phi, u[a], m[4 + 2 * a]);
     }
 #pragma unroll
-    for (int k = 3 + 2 * L::DIM; k < Q; ++k) d[k] = dl[k] = m[k];
+    for (int k = 3 + 2 * L::DIM; k < Q; ++k) d[k] = m[k];
     if (c.b1 != 0.f || c.b2 != 0.f || c.g7 != 0.f || c.g8 != 0.f) {   // MRT-B1/B2 only
-        float u2 = fmaf(ux, ux, __fmul_rn(uy, uy));
-        if (L::DIM == 3) u2 = fmaf(uz, uz, u2);
-        d[1] = fmaf(__fmul_rn(-c.b1, u2), phi, dl[1]);
-        d[2] = fmaf(__fmul_rn(-c.b2, u2), phi, dl[2]);
-        if (L::Q == 9) {
-            d[7] = fmaf(__fmul_rn(-c.g7, fmaf(ux, ux, -__fmul_rn(uy, uy))), phi, dl[7]);
-            d[8] = fmaf(__fmul_rn(-c.g8, __fmul_rn(ux, uy)), phi, dl[8]);
-        }
+        const float u2 = fmaf(ux, ux, __fmul_rn(uy, uy));
+        d[1] = fmaf(__fmul_rn(-c.b1, u2), phi, d[1]);
+        d[2] = fmaf(__fmul_rn(-c.b2, u2), phi, d[2]);
+        d[7] = fmaf(__fmul_rn(-c.g7, fmaf(ux, ux, -__fmul_rn(uy, uy))), phi, d[7]);
+        d[8] = fmaf(__fmul_rn(-c.g8, __fmul_rn(ux, uy)), phi, d[8]);
     }
-    // relaxation m' = m - S d; the offset form keeps m' - m^eq_lin = dl - S d
-    const float (&base)[Q] = OFFSET ? dl : m;
     float mp[Q];
-    mp[0] = OFFSET ? 0.f : phi;
-    mp[1] = fmaf(-c.s[1], d[1], base[1]);
-    mp[2] = fmaf(-c.s[2], d[2], base[2]);
+    mp[0] = phi;
+    mp[1] = fmaf(-c.s[1], d[1], m[1]);
+    mp[2] = fmaf(-c.s[2], d[2], m[2]);
 #pragma unroll
     for (int a = 0; a < L::DIM; ++a) {
         float r = 0.f;
@@ -350,22 +360,18 @@ __device__ __forceinline__ float collide(float (&f)[L::Q], float ux, float uy, f
             r = fmaf(c.A[a * L::DIM + b], d[3 + 2 * b], r);
             r = fmaf(c.C[a * L::DIM + b], d[4 + 2 * b], r);
         }
-        mp[3 + 2 * a] = base[3 + 2 * a] - r;
-        mp[4 + 2 * a] = fmaf(-c.s[4 + 2 * a], d[4 + 2 * a], base[4 + 2 * a]);
+        mp[3 + 2 * a] = m[3 + 2 * a] - r;
+        mp[4 + 2 * a] = fmaf(-c.s[4 + 2 * a], d[4 + 2 * a], m[4 + 2 * a]);
     }
 #pragma unroll
-    for (int k = 3 + 2 * L::DIM; k < Q; ++k) mp[k] = fmaf(-c.s[k], d[k], base[k]);
+    for (int k = 3 + 2 * L::DIM; k < Q; ++k) mp[k] = fmaf(-c.s[k], d[k], m[k]);
     // f' = M^T diag(1 / |row|^2) m'
 #pragma unroll
     for (int k = 0; k < Q; ++k) mp[k] = __fmul_rn(mp[k], 1.0f / (float)row_norm2<L>(k));
-    const float moving = populations<L, OFFSET, false>(mp, f);
     // The rest population closes the mass balance: sum_i f'_i = m'_0 = phi
     // (row 0 of M^-1 m'). Taking it from the moving populations keeps FP32
-    // rounding of the 1/|M_0|^2 factor from biasing the total mass. For the
-    // offsets, sum_i g_i = -phi eps0 balances the FP32 weights of the decode,
-    // which sum to 1 + eps0 (else the mass would drift by phi eps0 per step).
-    if constexpr (OFFSET) f[0] = fmaf(-c.eps0, phi, -moving);   // see Coef::eps0
-    else f[0] = phi - moving;
+    // rounding of the 1/|M_0|^2 factor from biasing the total mass.
+    f[0] = phi - populations<L, false, false>(mp, f);
     return phi;
 }
 
@@ -466,10 +472,10 @@ __device__ __forceinline__ void vel_ix(const StepArgs& a, IX N, IX cell, int y, 
 }
 
 template <class L, int STORE, int UK, bool WALLS, int VEC, typename IX>
-__global__ void __launch_bounds__(256) k_step(const StepArgs a)
+__global__ void __launch_bounds__(256) k_step(const StepArgs args)
 {
-    grid_dep_launch();
-    grid_dep_wait();
+    StepArgs a = args;
+    step_after_dep(a);
     using T = typename StT<STORE>::T;
     constexpr int Q = L::Q;
     constexpr bool NEQ = (STORE != ST_F32);
@@ -588,10 +594,10 @@ __device__ __forceinline__ int reflect_mask(int i, int mask)
 }
 
 template <class L, int STORE, int UK, typename IX>
-__global__ void __launch_bounds__(256) k_step_box(const StepArgs a)
+__global__ void __launch_bounds__(256) k_step_box(const StepArgs args)
 {
-    grid_dep_launch();
-    grid_dep_wait();
+    StepArgs a = args;
+    step_after_dep(a);
     using T = typename StT<STORE>::T;
     constexpr int Q = L::Q;
     constexpr bool NEQ = (STORE != ST_F32);

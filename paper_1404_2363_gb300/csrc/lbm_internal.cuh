@@ -230,7 +230,26 @@ struct LaunchCfg {
 // Waits for the kernels this launch depends on (programmatic dependent launch),
 // and lets the next one start its prologue.
 __device__ __forceinline__ void grid_dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+// A pointer whose loads stay behind grid_dep_wait(): read-only loads (__ldg) may
+// otherwise be moved ahead of it, where the previous kernel may not have written yet.
+template <class P>
+__device__ __forceinline__ P after_dep(P p)
+{
+    unsigned long long v = reinterpret_cast<unsigned long long>(p);
+    asm volatile("" : "+l"(v)::"memory");
+    return reinterpret_cast<P>(v);
+}
 __device__ __forceinline__ void grid_dep_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+__device__ __forceinline__ void step_after_dep(StepArgs& a)
+{
+    grid_dep_launch();
+    grid_dep_wait();
+    a.src = after_dep(a.src);
+    a.phi_src = after_dep(a.phi_src);
+    a.ua = after_dep(a.ua);
+    a.sched = after_dep(a.sched);
+}
 
 // A launch that may start while the stream's previous kernel drains: it waits
 // in grid_dep_wait() before it reads anything. From launch to launch of dependent

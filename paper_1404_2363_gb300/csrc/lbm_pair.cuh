@@ -46,16 +46,15 @@ __device__ __forceinline__ float2 collide_pair(float2 (&v)[9], float2 ux, float2
     const float2 dl5 = fma2(neg2(phi), uy, m5), dl6 = fma2(phi, uy, m6);
     const float2 a1 = mul2(dl1, sp2(c.ro[1])), a2 = mul2(dl2, sp2(c.ro[2]));
     const float2 a4 = mul2(dl4, sp2(c.ro[4])), a6 = mul2(dl6, sp2(c.ro[6]));
-    const float2 a7 = mul2(m7, sp2(c.ro[7])), a8 = mul2(m8, sp2(c.ro[8]));
     const float2 a3 = fma2(sp2(c.fr[0]), dl3, fma2(sp2(c.fr[1]), dl4, fma2(sp2(c.fr[2]), dl5, mul2(sp2(c.fr[3]), dl6))));
     const float2 a5 = fma2(sp2(c.fr[4]), dl3, fma2(sp2(c.fr[5]), dl4, fma2(sp2(c.fr[6]), dl5, mul2(sp2(c.fr[7]), dl6))));
     // v = M^T a (populations<D2Q9, true, false>)
     const float2 A = fma2(sp2(-2.f), a2, neg2(a1));
     const float2 B = fma2(sp2(2.f), a1, a2);
     const float2 X = fma2(sp2(-2.f), a4, a3), Y = fma2(sp2(-2.f), a6, a5);
-    const float2 Xd = add2(a3, a4), Yd = add2(a5, a6);
-    const float2 AP = add2(A, a7), AM = sub2(A, a7);
-    const float2 BP = add2(B, a8), BM = sub2(B, a8);
+    const float2 Xd = fma2(sp2(c.ro[4]), dl4, a3), Yd = fma2(sp2(c.ro[6]), dl6, a5);
+    const float2 AP = fma2(sp2(c.ro[7]), m7, A), AM = fma2(sp2(-c.ro[7]), m7, A);
+    const float2 BP = fma2(sp2(c.ro[8]), m8, B), BM = fma2(sp2(-c.ro[8]), m8, B);
     const float2 XY = add2(Xd, Yd), XmY = sub2(Xd, Yd);
     v[1] = add2(AP, X);
     v[3] = sub2(AP, X);

@@ -48,10 +48,10 @@ __device__ __forceinline__ float2 feq_unit_pair15(float w0, float wa, float wd, 
 
 // Needs nx even and 18 ncell < 2^31 (int offsets; checked by the launcher).
 template <int STORE, int UK, bool WALLS>
-__global__ void __launch_bounds__(256) k_step_pair_d3q15(const StepArgs a)
+__global__ void __launch_bounds__(256) k_step_pair_d3q15(const StepArgs args)
 {
-    grid_dep_launch();
-    grid_dep_wait();
+    StepArgs a = args;
+    step_after_dep(a);
     using P = Pair<STORE>;
     using T2 = typename P::T2;
     using L = D3Q15;

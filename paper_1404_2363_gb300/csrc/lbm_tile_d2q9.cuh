@@ -48,9 +48,12 @@ __global__ void __launch_bounds__(TILE_THREADS, 1) k_tile_d2q9(const __grid_cons
     const bool xwall = WALLS && a.bcx_lo != BC_PERIODIC, ywall = WALLS && a.bc_lo != BC_PERIODIC;
     grid_dep_launch();
     grid_dep_wait();
+    const void* const asrc = after_dep(a.src);
+    const float* const aua = after_dep(a.ua);
+    const float* const aphi = after_dep(a.phi_src);
     if (threadIdx.x <= T) {
         float s[3];
-        sched_row_at(a.sched, p.srow[threadIdx.x], 2, s);
+        sched_row_at(after_dep(a.sched), p.srow[threadIdx.x], 2, s);
         sched[threadIdx.x][0] = s[0];
         sched[threadIdx.x][1] = s[1];
     }
@@ -82,18 +85,18 @@ __global__ void __launch_bounds__(TILE_THREADS, 1) k_tile_d2q9(const __grid_cons
         if constexpr (NEQ) {
             float2 ax = sp2(0.f), ay = sp2(0.f);
             if (p.field) {
-                ax = make_float2(__ldg(a.ua + x[0]), __ldg(a.ua + x[1]));
-                ay = make_float2(__ldg(a.ua + N + x[0]), __ldg(a.ua + N + x[1]));
-            } else if (a.ua != nullptr) {
-                ax = sp2(__ldg(a.ua + y));
-                ay = sp2(__ldg(a.ua + ny + y));
+                ax = make_float2(__ldg(aua + x[0]), __ldg(aua + x[1]));
+                ay = make_float2(__ldg(aua + N + x[0]), __ldg(aua + N + x[1]));
+            } else if (aua != nullptr) {
+                ax = sp2(__ldg(aua + y));
+                ay = sp2(__ldg(aua + ny + y));
             }
-            const unsigned short* q = static_cast<const unsigned short*>(a.src);
+            const unsigned short* q = static_cast<const unsigned short*>(asrc);
             unsigned g[9];
 #pragma unroll
             for (int i = 0; i < 9; ++i)
                 g[i] = (unsigned)__ldg(q + i * N + x[0]) | (unsigned)__ldg(q + i * N + x[1]) << 16;
-            const float2 phi = xmul2(make_float2(__ldg(a.phi_src + x[0]), __ldg(a.phi_src + x[1])), sp2(SC));
+            const float2 phi = xmul2(make_float2(__ldg(aphi + x[0]), __ldg(aphi + x[1])), sp2(SC));
             float2 e[9];
             walk_feq(c, xmul2(ax, sp2(sched[0][0])), xmul2(ay, sp2(sched[0][1])), e);
 #pragma unroll
@@ -104,7 +107,7 @@ __global__ void __launch_bounds__(TILE_THREADS, 1) k_tile_d2q9(const __grid_cons
             d[9 * plane] = ax.x, d[9 * plane + 32] = ax.y;
             d[10 * plane] = ay.x, d[10 * plane + 32] = ay.y;
         } else {
-            const float* q = static_cast<const float*>(a.src);
+            const float* q = static_cast<const float*>(asrc);
 #pragma unroll
             for (int i = 0; i < 9; ++i) {
                 walk_copy<4>(d + i * plane, q + i * N + x[0]);
@@ -114,10 +117,10 @@ __global__ void __launch_bounds__(TILE_THREADS, 1) k_tile_d2q9(const __grid_cons
             for (int k = 0; k < 2; ++k) {
                 float* du = d + (9 + k) * plane;
                 if (p.field) {
-                    walk_copy<4>(du, a.ua + k * N + x[0]);
-                    walk_copy<4>(du + 32, a.ua + k * N + x[1]);
+                    walk_copy<4>(du, aua + k * N + x[0]);
+                    walk_copy<4>(du + 32, aua + k * N + x[1]);
                 } else {
-                    const float v = a.ua != nullptr ? __ldg(a.ua + k * ny + y) : 0.f;
+                    const float v = aua != nullptr ? __ldg(aua + k * ny + y) : 0.f;
                     du[0] = v, du[32] = v;
                 }
             }
@@ -131,7 +134,7 @@ __global__ void __launch_bounds__(TILE_THREADS, 1) k_tile_d2q9(const __grid_cons
     // population opp(i) that streams to y. The even step takes its populations
     // from the node's own slots and leaves f'_i(x) in slot (i, x). The last step
     // goes to global memory.
-    auto row_step = [&](int s, int ty, auto odd) {
+    auto row_step = [&](int s, int ty, auto odd, auto slow) {   // slow: a row or a tile with a wall
         constexpr bool gather = decltype(odd)::value;
         const int y = yv - T + ty;
         float* const d = sm + ty * P + lane;
@@ -145,7 +148,7 @@ __global__ void __launch_bounds__(TILE_THREADS, 1) k_tile_d2q9(const __grid_cons
             f[i] = make_float2(q[0], q[32]);
         }
         bool in0 = true, in1 = true;   // the lane's nodes inside the domain (x walls)
-        if (WALLS) {
+        if constexpr (decltype(slow)::value) {
             const int x = xv - T + lane;
             in0 = !xwall || (x >= 0 && x < nx);
             in1 = !xwall || (x + 32 >= 0 && x + 32 < nx);
@@ -204,7 +207,8 @@ __global__ void __launch_bounds__(TILE_THREADS, 1) k_tile_d2q9(const __grid_cons
                 }
             }
         }
-        const float2 ux = xmul2(uax, sp2(sched[s][0])), uy = xmul2(uay, sp2(sched[s][1]));
+        const float2 ux = NEQ ? xmul2(uax, sp2(sched[s][0])) : mul2(uax, sp2(sched[s][0]));
+        const float2 uy = NEQ ? xmul2(uay, sp2(sched[s][1])) : mul2(uay, sp2(sched[s][1]));
         const float2 phi = walk_collide<NEQ>(f, ux, uy, c);
         const int x = xv - T + lane;
         const bool keep = y >= yv && y < ye;
@@ -256,6 +260,7 @@ __global__ void __launch_bounds__(TILE_THREADS, 1) k_tile_d2q9(const __grid_cons
             if (in1) q[32] = v.y;
         }
     };
+    const bool xedge = xwall && (xv - T <= 0 || xv + 64 - T >= nx);   // the tile has columns at or past an x wall
     auto step = [&](int t, auto odd) {
         __syncthreads();
 #pragma unroll 1
@@ -263,7 +268,8 @@ __global__ void __launch_bounds__(TILE_THREADS, 1) k_tile_d2q9(const __grid_cons
             const int y = yv - T + ty;
             // the rows that later steps still need, inside the domain
             if (y < yv - (T - t) || y >= ye + (T - t) || (ywall && (y < 0 || y >= ny))) continue;
-            row_step(t, ty, odd);
+            if (WALLS && (xedge || (ywall && (y == 0 || y == ny - 1)))) row_step(t, ty, odd, std::integral_constant<bool, WALLS>{});
+            else row_step(t, ty, odd, std::false_type{});
         }
     };
 #pragma unroll 1

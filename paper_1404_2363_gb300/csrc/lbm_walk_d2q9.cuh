@@ -25,32 +25,13 @@
 
 namespace lbm {
 
-// Products that feed an addition: rounded on their own in every build, so that
-// the fused steps give the bits of k_step (which uses __fmul_rn; the paired
-// product may be fused into a paired addition that follows it).
+// A product that feeds an addition, rounded on its own in every build, so that
+// the fused steps give the bits of k_step (which uses __fmul_rn): a paired
+// product may be fused into a paired addition that follows it, with any rounding
+// suffix.
 __device__ __forceinline__ float2 xmul2(float2 a, float2 b)
 {
     return make_float2(__fmul_rn(a.x, b.x), __fmul_rn(a.y, b.y));
-}
-
-// m = M v for a node pair, in the order of operations of moments<D2Q9>
-__device__ __forceinline__ void walk_moments(const float2 (&v)[9], float2 (&m)[9])
-{
-    const float2 sx = add2(v[1], v[3]), ax = sub2(v[1], v[3]);
-    const float2 sy = add2(v[2], v[4]), ay = sub2(v[2], v[4]);
-    const float2 p57 = add2(v[5], v[7]), d57 = sub2(v[5], v[7]);
-    const float2 p68 = add2(v[6], v[8]), d68 = sub2(v[6], v[8]);
-    const float2 sa = add2(sx, sy), sd = add2(p57, p68);
-    const float2 jx = sub2(d57, d68), jy = add2(d57, d68);
-    m[0] = add2(add2(v[0], sa), sd);
-    m[1] = fma2(sp2(2.f), sd, fma2(sp2(-4.f), v[0], neg2(sa)));
-    m[2] = fma2(sp2(-2.f), sa, fma2(sp2(4.f), v[0], sd));
-    m[3] = add2(ax, jx);
-    m[4] = fma2(sp2(-2.f), ax, jx);
-    m[5] = add2(ay, jy);
-    m[6] = fma2(sp2(-2.f), ay, jy);
-    m[7] = sub2(sx, sy);
-    m[8] = sub2(p57, p68);
 }
 
 // collide<D2Q9, OFFSET> for a node pair, bit for bit: post-collision
@@ -58,27 +39,39 @@ __device__ __forceinline__ void walk_moments(const float2 (&v)[9], float2 (&m)[9
 template <bool OFFSET>
 __device__ __forceinline__ float2 walk_collide(float2 (&v)[9], float2 ux, float2 uy, const Coef& c)
 {
-    float2 m[9];
-    walk_moments(v, m);
-    const float2 phi = m[0];
-    float2 d1 = fma2(sp2(-c.meq1), phi, m[1]), d2 = fma2(sp2(-c.meq2), phi, m[2]);
-    const float2 d3 = fma2(neg2(phi), ux, m[3]), d4 = fma2(phi, ux, m[4]);
-    const float2 d5 = fma2(neg2(phi), uy, m[5]), d6 = fma2(phi, uy, m[6]);
-    float2 a1, a2, a3, a4, a5, a6, A, B, AP, AM, BP, BM;
+    const float2 sx = add2(v[1], v[3]), ax = sub2(v[1], v[3]);
+    const float2 sy = add2(v[2], v[4]), ay = sub2(v[2], v[4]);
+    const float2 p57 = add2(v[5], v[7]), d57 = sub2(v[5], v[7]);
+    const float2 p68 = add2(v[6], v[8]), d68 = sub2(v[6], v[8]);
+    const float2 sa = add2(sx, sy), sd = add2(p57, p68);
+    const float2 dx = sub2(d57, d68), dy = add2(d57, d68);
+    const float2 phi = add2(add2(v[0], sa), sd);
+    const float2 m7 = sub2(sx, sy), m8 = sub2(p57, p68);
+    float2 A, B, AP, AM, BP, BM, X, Xd, Y, Yd;
     if constexpr (OFFSET) {
-        a1 = xmul2(d1, sp2(c.ro[1]));
-        a2 = xmul2(d2, sp2(c.ro[2]));
-        a4 = xmul2(d4, sp2(c.ro[4]));
-        a6 = xmul2(d6, sp2(c.ro[6]));
-        const float2 a7 = xmul2(m[7], sp2(c.ro[7])), a8 = xmul2(m[8], sp2(c.ro[8]));
-        a3 = fma2(sp2(c.fr[0]), d3, fma2(sp2(c.fr[1]), d4, fma2(sp2(c.fr[2]), d5, xmul2(sp2(c.fr[3]), d6))));
-        a5 = fma2(sp2(c.fr[4]), d3, fma2(sp2(c.fr[5]), d4, fma2(sp2(c.fr[6]), d5, xmul2(sp2(c.fr[7]), d6))));
+        const float2 d1 = fma2(sp2(-c.meq1), phi, fma2(sp2(2.f), sd, fma2(sp2(-4.f), v[0], neg2(sa))));
+        const float2 d2 = fma2(sp2(-c.meq2), phi, fma2(sp2(-2.f), sa, fma2(sp2(4.f), v[0], sd)));
+        const float2 d3 = fma2(neg2(phi), ux, add2(ax, dx)), d4 = fma2(phi, ux, fma2(sp2(-2.f), ax, dx));
+        const float2 d5 = fma2(neg2(phi), uy, add2(ay, dy)), d6 = fma2(phi, uy, fma2(sp2(-2.f), ay, dy));
+        const float2 a1 = mul2(d1, sp2(c.ro[1])), a2 = mul2(d2, sp2(c.ro[2]));
+        const float2 a4 = mul2(d4, sp2(c.ro[4])), a6 = mul2(d6, sp2(c.ro[6]));
+        const float2 a3 = fma2(sp2(c.fr[0]), d3, fma2(sp2(c.fr[1]), d4, fma2(sp2(c.fr[2]), d5, mul2(sp2(c.fr[3]), d6))));
+        const float2 a5 = fma2(sp2(c.fr[4]), d3, fma2(sp2(c.fr[5]), d4, fma2(sp2(c.fr[6]), d5, mul2(sp2(c.fr[7]), d6))));
         A = fma2(sp2(-2.f), a2, neg2(a1));
         B = fma2(sp2(2.f), a1, a2);
-        AP = add2(A, a7), AM = sub2(A, a7);
-        BP = add2(B, a8), BM = sub2(B, a8);
+        AP = fma2(sp2(c.ro[7]), m7, A), AM = fma2(sp2(-c.ro[7]), m7, A);
+        BP = fma2(sp2(c.ro[8]), m8, B), BM = fma2(sp2(-c.ro[8]), m8, B);
+        X = fma2(sp2(-2.f), a4, a3), Xd = fma2(sp2(c.ro[4]), d4, a3);
+        Y = fma2(sp2(-2.f), a6, a5), Yd = fma2(sp2(c.ro[6]), d6, a5);
     } else {
-        float2 d7 = m[7], d8 = m[8];
+        const float2 m1 = fma2(sp2(2.f), sd, fma2(sp2(-4.f), v[0], neg2(sa)));
+        const float2 m2 = fma2(sp2(-2.f), sa, fma2(sp2(4.f), v[0], sd));
+        const float2 m3 = add2(ax, dx), m4 = fma2(sp2(-2.f), ax, dx);
+        const float2 m5 = add2(ay, dy), m6 = fma2(sp2(-2.f), ay, dy);
+        float2 d1 = fma2(sp2(-c.meq1), phi, m1), d2 = fma2(sp2(-c.meq2), phi, m2);
+        const float2 d3 = fma2(neg2(phi), ux, m3), d4 = fma2(phi, ux, m4);
+        const float2 d5 = fma2(neg2(phi), uy, m5), d6 = fma2(phi, uy, m6);
+        float2 d7 = m7, d8 = m8;
         if (c.b1 != 0.f || c.b2 != 0.f || c.g7 != 0.f || c.g8 != 0.f) {   // MRT-B1/B2 only
             const float2 uyy = xmul2(uy, uy);
             const float2 u2 = fma2(ux, ux, uyy);
@@ -96,21 +89,21 @@ __device__ __forceinline__ float2 walk_collide(float2 (&v)[9], float2 ux, float2
         r1 = fma2(sp2(c.A[3]), d5, r1);
         r1 = fma2(sp2(c.C[3]), d6, r1);
         const float2 a0 = xmul2(phi, sp2(1.f / 9.f));
-        a1 = xmul2(fma2(sp2(-c.s[1]), d1, m[1]), sp2(1.f / 36.f));
-        a2 = xmul2(fma2(sp2(-c.s[2]), d2, m[2]), sp2(1.f / 36.f));
-        a3 = xmul2(sub2(m[3], r0), sp2(1.f / 6.f));
-        a4 = xmul2(fma2(sp2(-c.s[4]), d4, m[4]), sp2(1.f / 12.f));
-        a5 = xmul2(sub2(m[5], r1), sp2(1.f / 6.f));
-        a6 = xmul2(fma2(sp2(-c.s[6]), d6, m[6]), sp2(1.f / 12.f));
+        const float2 a1 = xmul2(fma2(sp2(-c.s[1]), d1, m1), sp2(1.f / 36.f));
+        const float2 a2 = xmul2(fma2(sp2(-c.s[2]), d2, m2), sp2(1.f / 36.f));
+        const float2 a3 = xmul2(sub2(m3, r0), sp2(1.f / 6.f));
+        const float2 a4 = xmul2(fma2(sp2(-c.s[4]), d4, m4), sp2(1.f / 12.f));
+        const float2 a5 = xmul2(sub2(m5, r1), sp2(1.f / 6.f));
+        const float2 a6 = xmul2(fma2(sp2(-c.s[6]), d6, m6), sp2(1.f / 12.f));
         // 1/|M_7|^2 = 1/|M_8|^2 = 1/4: exact products, so fused below
-        const float2 q7 = fma2(sp2(-c.s[7]), d7, m[7]), q8 = fma2(sp2(-c.s[8]), d8, m[8]);
+        const float2 q7 = fma2(sp2(-c.s[7]), d7, m7), q8 = fma2(sp2(-c.s[8]), d8, m8);
         A = fma2(sp2(-2.f), a2, sub2(a0, a1));
         B = fma2(sp2(2.f), a1, add2(a0, a2));
         AP = fma2(sp2(0.25f), q7, A), AM = fma2(sp2(-0.25f), q7, A);
         BP = fma2(sp2(0.25f), q8, B), BM = fma2(sp2(-0.25f), q8, B);
+        X = fma2(sp2(-2.f), a4, a3), Xd = add2(a3, a4);
+        Y = fma2(sp2(-2.f), a6, a5), Yd = add2(a5, a6);
     }
-    const float2 X = fma2(sp2(-2.f), a4, a3), Y = fma2(sp2(-2.f), a6, a5);
-    const float2 Xd = add2(a3, a4), Yd = add2(a5, a6);
     const float2 XY = add2(Xd, Yd), XmY = sub2(Xd, Yd);
     v[1] = add2(AP, X);
     v[3] = sub2(AP, X);
@@ -121,7 +114,7 @@ __device__ __forceinline__ float2 walk_collide(float2 (&v)[9], float2 ux, float2
     v[6] = sub2(BM, XmY);
     v[8] = add2(BM, XmY);
     const float2 AB = add2(A, B);
-    if constexpr (OFFSET) v[0] = fma2(sp2(-c.eps0), phi, xmul2(sp2(-4.f), AB));   // Coef::eps0
+    if constexpr (OFFSET) v[0] = fma2(sp2(-c.eps0), phi, mul2(sp2(-4.f), AB));   // Coef::eps0
     else v[0] = fma2(sp2(-4.f), AB, phi);                                         // 4 x exact
     return phi;
 }
@@ -142,7 +135,10 @@ __device__ __forceinline__ void walk_feq(const Coef& c, float2 ux, float2 uy, fl
 }
 
 constexpr int WALK_WARPS = 4;    // independent warps per CTA
-__host__ __device__ constexpr int walk_minb(int T) { return T <= 2 ? 4 : 3; }   // 128 / 168 registers
+#ifndef WALK_WB
+#define WALK_WB 2
+#endif
+__host__ __device__ constexpr int walk_minb(int T, bool walls) { return T <= 2 ? 4 : (walls ? WALK_WB : 3); }   // 128 / 168 registers
 
 // What a level keeps of its last two rows for the rows that still pull from
 // them, unshifted: the e_y = 0 populations {0, 1, 3} of the last row and the
@@ -191,7 +187,7 @@ __device__ __forceinline__ void walk_copy(void* dst, const void* src)   // async
 // SAVE: the FP32 states between are stored too (p.mid), for the reverse sweep.
 // At T = 4 the levels need 168 registers: 12 warps per SM.
 template <int STORE, bool FIELD, bool WALLS, int T, bool SAVE>
-__global__ void __launch_bounds__(32 * WALK_WARPS, walk_minb(T)) k_walk_d2q9(const __grid_constant__ WalkArgs p)
+__global__ void __launch_bounds__(32 * WALK_WARPS, walk_minb(T, WALLS)) k_walk_d2q9(const __grid_constant__ WalkArgs p)
 {
     using L = D2Q9;
     constexpr bool NEQ = STORE != ST_F32;
@@ -208,9 +204,11 @@ __global__ void __launch_bounds__(32 * WALK_WARPS, walk_minb(T)) k_walk_d2q9(con
     __shared__ float sched[T + 1][2];
     grid_dep_launch();
     grid_dep_wait();
+    const void* const asrc = after_dep(a.src);
+    const float* const aua = after_dep(a.ua);
     if (threadIdx.x <= T) {
         float s[3];
-        sched_row_at(a.sched, p.srow[threadIdx.x], 2, s);
+        sched_row_at(after_dep(a.sched), p.srow[threadIdx.x], 2, s);
         sched[threadIdx.x][0] = s[0];
         sched[threadIdx.x][1] = s[1];
     }
@@ -236,6 +234,7 @@ __global__ void __launch_bounds__(32 * WALK_WARPS, walk_minb(T)) k_walk_d2q9(con
     const bool left = xwall && x0 == 0;
     const bool rx = xwall && x0 == nx - 1, ry = xwall && x0 + 1 == nx - 1;
     const bool edge = WALLS && __any_sync(0xffffffffu, left || rx || ry);
+    const bool lb = left && a.bcx_lo == BC_BOUNCE, ln = left && a.bcx_lo == BC_NOFLUX, hb = a.bcx_hi == BC_BOUNCE;
     const bool ywall = WALLS && a.bc_lo != BC_PERIODIC;
     const int rs = ywall ? max(ya - T, 0) : ya - T, re = yb - 1 + T;
 
@@ -266,10 +265,10 @@ __global__ void __launch_bounds__(32 * WALK_WARPS, walk_minb(T)) k_walk_d2q9(con
             col %= nx;
             if (col < 0) col += nx;
         }
-        const float* fp = NEQ ? a.phi_src : static_cast<const float*>(a.src);
-        if (FIELD && ch >= Slot::schunks) fp = a.ua + (ch >= Slot::schunks + 16 ? N : 0);
+        const float* fp = NEQ ? a.phi_src : static_cast<const float*>(asrc);
+        if (FIELD && ch >= Slot::schunks) fp = aua + (ch >= Slot::schunks + 16 ? N : 0);
         else if (!NEQ) fp += plane * N;
-        from[k] = g16 ? reinterpret_cast<const unsigned char*>(static_cast<const unsigned short*>(a.src) + plane * N + col)
+        from[k] = g16 ? reinterpret_cast<const unsigned char*>(static_cast<const unsigned short*>(asrc) + plane * N + col)
                       : reinterpret_cast<const unsigned char*>(fp + col);
     }
     auto issue = [&](int r) {   // stage walk row r
@@ -292,7 +291,7 @@ __global__ void __launch_bounds__(32 * WALK_WARPS, walk_minb(T)) k_walk_d2q9(con
                     walk_copy<4>(d + 4, q + row + c1);
                 };
                 if constexpr (NEQ) {   // no 4-byte copy can start at an odd 16-bit word
-                    const unsigned short* q = static_cast<const unsigned short*>(a.src);
+                    const unsigned short* q = static_cast<const unsigned short*>(asrc);
                     unsigned g[9];
 #pragma unroll
                     for (int i = 0; i < 9; ++i)
@@ -304,28 +303,27 @@ __global__ void __launch_bounds__(32 * WALK_WARPS, walk_minb(T)) k_walk_d2q9(con
                 } else {
 #pragma unroll
                     for (int i = 0; i < 9; ++i)
-                        copy_pair(st + Slot::plane * i + 8 * lane, static_cast<const float*>(a.src) + i * N);
+                        copy_pair(st + Slot::plane * i + 8 * lane, static_cast<const float*>(asrc) + i * N);
                 }
                 if (FIELD) {
-                    copy_pair(su + 8 * lane, a.ua);
-                    copy_pair(su + 256 + 8 * lane, a.ua + N);
+                    copy_pair(su + 8 * lane, aua);
+                    copy_pair(su + 256 + 8 * lane, aua + N);
                 }
             }
         }
         asm volatile("cp.async.commit_group;" ::: "memory");
     };
-    auto velocity = [&](int y, float2& ux, float2& uy) {   // velocity factors of walk row y
-        if (FIELD) {
+    float rux[T + 1], ruy[T + 1];   // row profile: the velocity factors of the rows r .. r - T
+#pragma unroll
+    for (int s = 0; s <= T; ++s) rux[s] = ruy[s] = 0.f;
+    auto velocity = [&](int y, int s, float2& ux, float2& uy) {   // velocity factors of walk row y = r - s
+        if (!FIELD) {
+            ux = sp2(rux[s]);
+            uy = sp2(ruy[s]);
+        } else {
             const unsigned char* su = smu + (y & (WALK_UROWS - 1)) * 512 + 8 * lane;
             ux = *reinterpret_cast<const float2*>(su);
             uy = *reinterpret_cast<const float2*>(su + 256);
-        } else {
-            ux = uy = sp2(0.f);
-            if (a.ua != nullptr) {
-                const int yy = wrap(y);
-                ux = sp2(__ldg(a.ua + yy));
-                uy = sp2(__ldg(a.ua + ny + yy));
-            }
         }
     };
 
@@ -340,10 +338,21 @@ __global__ void __launch_bounds__(32 * WALK_WARPS, walk_minb(T)) k_walk_d2q9(con
 #pragma unroll 1
     for (int j = 0; j < WALK_AHEAD; ++j) issue(rs + j);
 
-    auto row_step = [&](int r, auto par) {
+    // Rows next to a y wall, and the strips with an x wall, run their own instances: the branches of the wall
+    // rules between the levels cost all other rows their overlap (4096^2 between Neumann walls: 125 us a
+    // step with them in place, 77 without)
+    auto row_step = [&](int r, auto par, auto rule) {   // rule: 0 none, 1 x walls, 2 y walls (x walls if edge)
+        constexpr bool SLOW = decltype(rule)::value == 2, EDGE = WALLS && decltype(rule)::value > 0;
         constexpr bool ODD = decltype(par)::value != 0;
         float2 n[9];
         asm volatile("cp.async.wait_group %0;" ::"n"(WALK_AHEAD - 1) : "memory");
+        if (!FIELD && aua != nullptr) {
+#pragma unroll
+            for (int s = T; s > 0; --s) rux[s] = rux[s - 1], ruy[s] = ruy[s - 1];
+            const int y = wrap(r);
+            rux[0] = __ldg(aua + y);
+            ruy[0] = __ldg(aua + ny + y);
+        }
         __syncwarp();   // row r has landed for every lane, and every lane is done with row r - 1
         {
             const unsigned char* st = sm + (r & (WALK_ROWS - 1)) * Slot::state;
@@ -351,7 +360,7 @@ __global__ void __launch_bounds__(32 * WALK_WARPS, walk_minb(T)) k_walk_d2q9(con
                 using P = Pair<STORE>;
                 using Q = QuadH<STORE>;
                 float2 ax, ay, e[9];
-                velocity(r, ax, ay);
+                velocity(r, 0, ax, ay);
                 walk_feq(c, xmul2(ax, sp2(sched[0][0])), xmul2(ay, sp2(sched[0][1])), e);
                 const float2 phi = xmul2(*reinterpret_cast<const float2*>(st + 9 * Slot::plane + 8 * lane), sp2(SC));
 #pragma unroll
@@ -371,7 +380,7 @@ __global__ void __launch_bounds__(32 * WALK_WARPS, walk_minb(T)) k_walk_d2q9(con
             float2(&p2)[3] = ODD ? lw.pa : lw.pb;
             const int y = r - s;
             float2 ax, ay;
-            velocity(y, ax, ay);
+            velocity(y, s, ax, ay);
             float2 f[9];
             f[0] = lw.c0[0];
             f[1] = walk_from_left(lw.c0[1]);
@@ -382,10 +391,10 @@ __global__ void __launch_bounds__(32 * WALK_WARPS, walk_minb(T)) k_walk_d2q9(con
             f[4] = n[4];
             f[7] = walk_from_right(n[7]);
             f[8] = walk_from_left(n[8]);
-            if (WALLS) {
+            if constexpr (SLOW || EDGE) {
                 // the rules of k_step_box, in its order of precedence: bounce-back on y, on x, then the
                 // mirror rule on x, on y, then Dirichlet
-                const bool lo = ywall && y == 0, hi = ywall && y == ny - 1;
+                const bool lo = SLOW && ywall && y == 0, hi = SLOW && ywall && y == ny - 1;
                 const int kind = lo ? a.bc_lo : a.bc_hi;
                 if ((lo || hi) && kind == BC_BOUNCE) {
                     if (lo) {      // stashed when row 0 came in
@@ -398,19 +407,14 @@ __global__ void __launch_bounds__(32 * WALK_WARPS, walk_minb(T)) k_walk_d2q9(con
                         f[8] = p1[2];
                     }
                 }
-                if (edge) {
-                    if (a.bcx_lo == BC_BOUNCE) {
-                        if (left) f[1].x = lw.c0[2].x, f[5].x = lw.sb, f[8].x = p1[2].x;
-                    } else {
-                        if (left) f[1].x = f[3].x, f[5].x = f[6].x, f[8].x = f[7].x;
-                    }
-                    if (a.bcx_hi == BC_BOUNCE) {
-                        if (rx) f[3].x = lw.c0[1].x, f[6].x = lw.sb, f[7].x = p1[1].x;
-                        if (ry) f[3].y = lw.c0[1].y, f[6].y = lw.sb, f[7].y = p1[1].y;
-                    } else {
-                        if (rx) f[3].x = f[1].x, f[6].x = f[5].x, f[7].x = f[8].x;
-                        if (ry) f[3].y = f[1].y, f[6].y = f[5].y, f[7].y = f[8].y;
-                    }
+                if (EDGE) {   // selects, no branches
+                    f[1].x = lb ? lw.c0[2].x : (ln ? f[3].x : f[1].x);
+                    f[5].x = lb ? lw.sb : (ln ? f[6].x : f[5].x);
+                    f[8].x = lb ? p1[2].x : (ln ? f[7].x : f[8].x);
+                    const float3 rv = rx ? make_float3(hb ? lw.c0[1].x : f[1].x, hb ? lw.sb : f[5].x, hb ? p1[1].x : f[8].x)
+                                         : make_float3(hb ? lw.c0[1].y : f[1].y, hb ? lw.sb : f[5].y, hb ? p1[1].y : f[8].y);
+                    f[3].x = rx ? rv.x : f[3].x, f[6].x = rx ? rv.y : f[6].x, f[7].x = rx ? rv.z : f[7].x;
+                    f[3].y = ry ? rv.x : f[3].y, f[6].y = ry ? rv.y : f[6].y, f[7].y = ry ? rv.z : f[7].y;
                     lw.sb = left ? n[7].x : (rx ? n[8].x : n[8].y);
                 }
                 if (lo || hi) {
@@ -437,9 +441,11 @@ __global__ void __launch_bounds__(32 * WALK_WARPS, walk_minb(T)) k_walk_d2q9(con
             }
             p2[0] = n[2], p2[1] = n[5], p2[2] = n[6];   // the next row's p1
             lw.c0[0] = n[0], lw.c0[1] = n[1], lw.c0[2] = n[3];
-            if (WALLS && ywall && y == -1 && a.bc_lo == BC_BOUNCE) p1[0] = n[4], p1[1] = n[7], p1[2] = n[8];
+            if (SLOW && ywall && y == -1 && a.bc_lo == BC_BOUNCE) p1[0] = n[4], p1[1] = n[7], p1[2] = n[8];
 
-            const float2 ux = xmul2(ax, sp2(sched[s][0])), uy = xmul2(ay, sp2(sched[s][1]));
+            // a product that only feeds products may be paired; u also feeds sums in the 16-bit decode
+            const float2 ux = NEQ ? xmul2(ax, sp2(sched[s][0])) : mul2(ax, sp2(sched[s][0]));
+            const float2 uy = NEQ ? xmul2(ay, sp2(sched[s][1])) : mul2(ay, sp2(sched[s][1]));
             const float2 phi = walk_collide<NEQ>(f, ux, uy, c);
             const bool keep = mine && y >= ya && y < yb;
             if constexpr (NEQ) {
@@ -494,8 +500,13 @@ __global__ void __launch_bounds__(32 * WALK_WARPS, walk_minb(T)) k_walk_d2q9(con
     };
 #pragma unroll 1
     for (int r = rs; r <= re; r += 2) {   // the row past re, where there is one, computes nothing that is kept
-        row_step(r, std::integral_constant<int, 0>{});
-        row_step(r + 1, std::integral_constant<int, 1>{});
+        auto two = [&](auto rule) {
+            row_step(r, std::integral_constant<int, 0>{}, rule);
+            row_step(r + 1, std::integral_constant<int, 1>{}, rule);
+        };
+        if (WALLS && ywall && (r - T <= 0 || r >= ny - 1)) two(std::integral_constant<int, WALLS ? 2 : 0>{});
+        else if (edge) two(std::integral_constant<int, WALLS ? 1 : 0>{});
+        else two(std::integral_constant<int, 0>{});
     }
 }
 

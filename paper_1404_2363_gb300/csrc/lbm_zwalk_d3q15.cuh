@@ -91,10 +91,10 @@ __device__ __forceinline__ void zw_issue_g(const uint16_t* __restrict__ g, uint1
 // 80 registers: 3 CTAs of 256 threads (TY = 8) or 6 of 128 (TY = 4) per SM; at
 // 64 registers, for a fourth 256-thread CTA, the kernel spills.
 template <int STORE, int UK, bool WALLS, int TY>
-__global__ void __launch_bounds__(32 * TY, TY == 8 ? 3 : 6) k_step_zw_d3q15(const StepArgs a)
+__global__ void __launch_bounds__(32 * TY, TY == 8 ? 3 : 6) k_step_zw_d3q15(const StepArgs args)
 {
-    grid_dep_launch();
-    grid_dep_wait();
+    StepArgs a = args;
+    step_after_dep(a);
     using Gm = ZwGeom<TY>;
     constexpr int PLANE = Gm::PLANE, CHUNKS = Gm::CHUNKS, GPOS = Gm::GPOS;
     using P = Pair<STORE>;
