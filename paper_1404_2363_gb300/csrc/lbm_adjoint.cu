@@ -104,8 +104,7 @@ template <class L, int UK, int WM, bool DA, typename IX, bool QUAD>
 __global__ void __launch_bounds__(256, (L::Q == 9 && !DA && WM < 2) ? 4 : 3) k_adjoint(const AdjArgs args)
 {
     AdjArgs a = args;
-    grid_dep_launch();
-    grid_dep_wait();
+    grid_dep_sync();
     a.mu_in = after_dep(a.mu_in);
     a.fprev = after_dep(a.fprev);
     a.ua = after_dep(a.ua);
@@ -183,12 +182,12 @@ __global__ void __launch_bounds__(256, (L::Q == 9 && !DA && WM < 2) ? 4 : 3) k_a
         }
 #pragma unroll
         for (int i = 0; i < Q; ++i) {
-            mu[i] = __ldg(a.mu_in + (IX)i * N + cell);
+            mu[i] = ld_dep(a.mu_in + (IX)i * N + cell);
             if constexpr (BOX) {
-                f[i] = !bout[i] ? __ldg(a.fprev + (IX)i * N + bsrc[i])
-                                : (bbb[i] ? __ldg(a.fprev + (IX)opposite<L>(i) * N + cell) : 0.f);
+                f[i] = !bout[i] ? ld_dep(a.fprev + (IX)i * N + bsrc[i])
+                                : (bbb[i] ? ld_dep(a.fprev + (IX)opposite<L>(i) * N + cell) : 0.f);
             } else {
-                f[i] = __ldg(a.fprev + (IX)i * N + tgt(i));
+                f[i] = ld_dep(a.fprev + (IX)i * N + tgt(i));
             }
         }
         if constexpr (BOX) {
@@ -212,7 +211,7 @@ __global__ void __launch_bounds__(256, (L::Q == 9 && !DA && WM < 2) ? 4 : 3) k_a
             for (int i = 0; i < Q; ++i)
                 if (L::ey(i) != 0 && ((L::ey(i) == 1) == lo)) {
                     if (kind == BC_NOFLUX) f[i] = f[mirror_y<L>(i)];
-                    else if (kind == BC_BOUNCE) f[i] = __ldg(a.fprev + (IX)opposite<L>(i) * N + cell);
+                    else if (kind == BC_BOUNCE) f[i] = ld_dep(a.fprev + (IX)opposite<L>(i) * N + cell);
                 }
         }
         // Dirichlet fill (y faces, wall mode 1 or 2): the inward populations are

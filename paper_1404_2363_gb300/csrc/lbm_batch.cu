@@ -447,8 +447,7 @@ __global__ void __launch_bounds__(32 * WALK_WARPS, 3) k_batch_walk(const __grid_
 {
     constexpr int T = BWALK_T, HALO = WALK_HALO;
     extern __shared__ __align__(16) unsigned char bwalk_sm[];
-    grid_dep_launch();
-    grid_dep_wait();
+    grid_dep_sync();
     const BatchTask tk = after_dep(p.tasks)[blockIdx.x];
     const InstK& I = p.c.inst[tk.inst];
     const float* const urow = after_dep(I.urow);
@@ -1194,7 +1193,18 @@ static lbm_status setup_walk(lbm_cde_batch_t b)
         b->ss.wcpart[p] = static_cast<double*>(balloc(b, sizeof(double) * 3 * (size_t)b->ncblk * T));
         ok = b->ss.wstrip[p] && b->ss.wcpart[p];
     }
-    if (!ok) return LBM_E_OOM;
+    if (!ok) {   // no memory to spare: one step a launch
+        bfree(b, b->tasks);
+        b->tasks = nullptr;
+        for (int p = 0; p < 2; ++p) {
+            bfree(b, b->ss.wstrip[p]);
+            bfree(b, b->ss.wcpart[p]);
+            b->ss.wstrip[p] = nullptr;
+            b->ss.wcpart[p] = nullptr;
+        }
+        b->ntasks.clear();
+        return LBM_OK;
+    }
     if (cudaFuncSetAttribute(lbm::k_batch_walk, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              lbm::WALK_WARPS * lbm::BWALK_WARP) != cudaSuccess)
         return LBM_E_CUDA;

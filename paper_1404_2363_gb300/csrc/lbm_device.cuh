@@ -388,13 +388,13 @@ template <> struct StT<ST_BF16> { using T = __nv_bfloat16; };
 // instead of its subnormals, while |g| up to 32 remains representable.
 constexpr float F16_SCALE = 2048.0f;
 
-__device__ __forceinline__ float ldg_f(const float* p) { return __ldg(p); }
+__device__ __forceinline__ float ldg_f(const float* p) { return ld_dep(p); }
 __device__ __forceinline__ float ldg_f(const __half* p) {
-    return __half2float(__ushort_as_half(__ldg(reinterpret_cast<const unsigned short*>(p)))) *
+    return __half2float(__ushort_as_half(ld_dep(reinterpret_cast<const unsigned short*>(p)))) *
            (1.0f / F16_SCALE);
 }
 __device__ __forceinline__ float ldg_f(const __nv_bfloat16* p) {
-    return __bfloat162float(__ushort_as_bfloat16(__ldg(reinterpret_cast<const unsigned short*>(p))));
+    return __bfloat162float(__ushort_as_bfloat16(ld_dep(reinterpret_cast<const unsigned short*>(p))));
 }
 __device__ __forceinline__ void st_f(float* p, float v) { *p = v; }
 __device__ __forceinline__ void st_f(__half* p, float v) { *p = __float2half_rn(v * F16_SCALE); }
@@ -512,7 +512,7 @@ __global__ void __launch_bounds__(256) k_step(const StepArgs args)
             if (NEQ) {
                 float ux, uy, uz;
                 vel_ix<UK, L::DIM, IX>(a, N, sc, ys[L::ey(i) + 1], s_prev, ux, uy, uz);
-                v = fmaf(__ldg(a.phi_src + sc), feq_unit<L>(a.c, i, ux, uy, uz), v);
+                v = fmaf(ld_dep(a.phi_src + sc), feq_unit<L>(a.c, i, ux, uy, uz), v);
             }
             f[j][i] = v;
         }
@@ -538,7 +538,7 @@ __global__ void __launch_bounds__(256) k_step(const StepArgs args)
                         if (L::ey(i) != 0 && ((L::ey(i) == 1) == lo)) {
                             const int o = opposite<L>(i);
                             float v = ldg_f(src + (IX)o * N + cell[j]);
-                            if (NEQ) v = fmaf(__ldg(a.phi_src + cell[j]), feq_unit<L>(a.c, o, ux, uy, uz), v);
+                            if (NEQ) v = fmaf(ld_dep(a.phi_src + cell[j]), feq_unit<L>(a.c, o, ux, uy, uz), v);
                             f[j][i] = v;
                         }
                 } else {  // Dirichlet
@@ -646,12 +646,12 @@ __global__ void __launch_bounds__(256) k_step_box(const StepArgs args)
             if (NEQ) {
                 float ux, uy, uz;
                 vel_ix<UK, L::DIM, IX>(a, N, sc, sp[1], s_prev, ux, uy, uz);
-                v = fmaf(__ldg(a.phi_src + sc), feq_unit<L>(a.c, i, ux, uy, uz), v);
+                v = fmaf(ld_dep(a.phi_src + sc), feq_unit<L>(a.c, i, ux, uy, uz), v);
             }
         } else if (bb) {
             const int o = opposite<L>(i);
             v = ldg_f(src + (IX)o * N + cell);
-            if (NEQ) v = fmaf(__ldg(a.phi_src + cell), feq_unit<L>(a.c, o, uxp, uyp, uzp), v);
+            if (NEQ) v = fmaf(ld_dep(a.phi_src + cell), feq_unit<L>(a.c, o, uxp, uyp, uzp), v);
         }
         w[i] = v;
     }

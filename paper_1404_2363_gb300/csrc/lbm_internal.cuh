@@ -107,7 +107,7 @@ struct WalkArgs {
     StepArgs a;          // src: state k - 1; dst: state k - 1 + T
     int srow[5];         // schedule rows of u(k - 1) .. u(k - 1 + T), or -1
     void* mid[3];        // SAVE: the states k .. k + T - 2 (FP32)
-    int strips, ranges;  // strips of walk_cols(T) columns x ranges of rows
+    int strips, ranges;  // strips of WALK_COLS columns x ranges of rows
     int vec;             // pairs are stored as one word (nx even, aligned planes)
     int wide;            // rows are staged by 16-byte copies (nx a multiple of 4, or 8 for 16-bit planes; aligned)
 };
@@ -227,11 +227,42 @@ struct LaunchCfg {
     int vec;     // cells per thread along x (1, 2 or 4)
 };
 
-// Waits for the kernels this launch depends on (programmatic dependent launch),
-// and lets the next one start its prologue.
-__device__ __forceinline__ void grid_dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-// A pointer whose loads stay behind grid_dep_wait(): read-only loads (__ldg) may
-// otherwise be moved ahead of it, where the previous kernel may not have written yet.
+// Programmatic dependent launch. A kernel waits for the one before it before its
+// first read, and only then lets the next one start, so that no more than two are
+// in flight: the next one's launch drops what the L1 caches held from before the
+// kernel that is still writing. What that kernel writes is read with ld_dep (or
+// cp.async): __ldg and the loads the compiler makes of it promise data that nothing
+// writes while the kernel exists, and were seen to return the state of two steps before.
+__device__ __forceinline__ void grid_dep_sync()
+{
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+__device__ __forceinline__ float ld_dep(const float* p)
+{
+    float v;
+    asm volatile("ld.global.f32 %0, [%1];" : "=f"(v) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ float2 ld_dep(const float2* p)
+{
+    float2 v;
+    asm volatile("ld.global.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ unsigned ld_dep(const unsigned* p)
+{
+    unsigned v;
+    asm volatile("ld.global.u32 %0, [%1];" : "=r"(v) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ unsigned short ld_dep(const unsigned short* p)
+{
+    unsigned short v;
+    asm volatile("ld.global.u16 %0, [%1];" : "=h"(v) : "l"(p));
+    return v;
+}
+// A pointer whose read-only loads (__ldg, for what the caller owns) stay behind grid_dep_sync().
 template <class P>
 __device__ __forceinline__ P after_dep(P p)
 {
@@ -239,12 +270,10 @@ __device__ __forceinline__ P after_dep(P p)
     asm volatile("" : "+l"(v)::"memory");
     return reinterpret_cast<P>(v);
 }
-__device__ __forceinline__ void grid_dep_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 __device__ __forceinline__ void step_after_dep(StepArgs& a)
 {
-    grid_dep_launch();
-    grid_dep_wait();
+    grid_dep_sync();
     a.src = after_dep(a.src);
     a.phi_src = after_dep(a.phi_src);
     a.ua = after_dep(a.ua);
@@ -252,7 +281,7 @@ __device__ __forceinline__ void step_after_dep(StepArgs& a)
 }
 
 // A launch that may start while the stream's previous kernel drains: it waits
-// in grid_dep_wait() before it reads anything. From launch to launch of dependent
+// in grid_dep_sync() before it reads anything. From launch to launch of dependent
 // kernels: D3Q15 40^3 4.6 -> 3.4 us a step, 64^3 8.2 -> 5.8, 97 x 80 x 66 12.4 -> 10.2.
 template <class A>
 cudaError_t launch_dependent(void (*kernel)(A), dim3 grid, dim3 block, int smem, cudaStream_t st, const A& args)

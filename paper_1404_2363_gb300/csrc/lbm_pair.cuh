@@ -164,7 +164,7 @@ template <> struct Pair<ST_BF16> {
 template <class T2>
 __device__ __forceinline__ T2 ldg_pair(const T2* p)
 {
-    const unsigned w = __ldg(reinterpret_cast<const unsigned*>(p));
+    const unsigned w = ld_dep(reinterpret_cast<const unsigned*>(p));
     return *reinterpret_cast<const T2*>(&w);
 }
 

@@ -22,8 +22,8 @@ namespace lbm {
 __device__ __forceinline__ float2 pair_window(const float* row, float2 c, int ex, int xlo, int xhi)
 {
     if (ex == 0) return c;
-    if (ex > 0) return make_float2(__ldg(row + xlo), c.x);
-    return make_float2(c.y, __ldg(row + xhi));
+    if (ex > 0) return make_float2(ld_dep(row + xlo), c.x);
+    return make_float2(c.y, ld_dep(row + xhi));
 }
 
 // f^eq_i / phi = w_i + k_i e_i.u for two nodes with u given (wall rules)
@@ -95,7 +95,7 @@ __global__ void __launch_bounds__(256) k_step_pair_d3q15(const StepArgs args)
         else if (ex > 0) h = P::join(ldg_pair(prow + xlp / 2), ldg_pair(prow + x0 / 2));
         else h = P::join(ldg_pair(prow + x0 / 2), ldg_pair(prow + xhi / 2));
         const float* prw = a.phi_src + row;
-        const float2 ps = pair_window(prw, __ldg(reinterpret_cast<const float2*>(prw + x0)), ex, xlo, xhi);
+        const float2 ps = pair_window(prw, ld_dep(reinterpret_cast<const float2*>(prw + x0)), ex, xlo, xhi);
         const int wc = wclass<L>(i);
         float2 e = sp2(wc == 0 ? w0 : (wc == 1 ? wa : wd));
         if (UK == U_FIELD) {
@@ -105,7 +105,7 @@ __global__ void __launch_bounds__(256) k_step_pair_d3q15(const StepArgs args)
             for (int d = 0; d < 3; ++d) {
                 if (ed[d] == 0) continue;
                 const float* ar = a.ua + d * N + row;
-                const float2 ad = pair_window(ar, __ldg(reinterpret_cast<const float2*>(ar + x0)), ex, xlo, xhi);
+                const float2 ad = pair_window(ar, ld_dep(reinterpret_cast<const float2*>(ar + x0)), ex, xlo, xhi);
                 e = fma2(sp2(ed[d] > 0 ? ks[d] : -ks[d]), ad, e);
             }
         } else if (UK == U_ROW && wc != 0) {
@@ -143,7 +143,7 @@ __global__ void __launch_bounds__(256) k_step_pair_d3q15(const StepArgs args)
                 for (int i = 0; i < 15; ++i)
                     if (L::ey(i) == inward) f[i] = f[mirror_y<L>(i)];
             } else if (kind == BC_BOUNCE) {
-                const float2 po = __ldg(reinterpret_cast<const float2*>(a.phi_src + cell));
+                const float2 po = ld_dep(reinterpret_cast<const float2*>(a.phi_src + cell));
 #pragma unroll
                 for (int i = 0; i < 15; ++i)
                     if (L::ey(i) == inward) {

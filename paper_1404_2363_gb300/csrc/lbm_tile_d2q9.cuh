@@ -46,8 +46,7 @@ __global__ void __launch_bounds__(TILE_THREADS, 1) k_tile_d2q9(const __grid_cons
     const int xv = blockIdx.x * (P - 2 * T), yv = blockIdx.y * (H - 2 * T);
     const int xe = min(xv + P - 2 * T, nx), ye = min(yv + H - 2 * T, ny);
     const bool xwall = WALLS && a.bcx_lo != BC_PERIODIC, ywall = WALLS && a.bc_lo != BC_PERIODIC;
-    grid_dep_launch();
-    grid_dep_wait();
+    grid_dep_sync();
     const void* const asrc = after_dep(a.src);
     const float* const aua = after_dep(a.ua);
     const float* const aphi = after_dep(a.phi_src);
@@ -95,8 +94,8 @@ __global__ void __launch_bounds__(TILE_THREADS, 1) k_tile_d2q9(const __grid_cons
             unsigned g[9];
 #pragma unroll
             for (int i = 0; i < 9; ++i)
-                g[i] = (unsigned)__ldg(q + i * N + x[0]) | (unsigned)__ldg(q + i * N + x[1]) << 16;
-            const float2 phi = xmul2(make_float2(__ldg(aphi + x[0]), __ldg(aphi + x[1])), sp2(SC));
+                g[i] = (unsigned)ld_dep(q + i * N + x[0]) | (unsigned)ld_dep(q + i * N + x[1]) << 16;
+            const float2 phi = xmul2(make_float2(ld_dep(aphi + x[0]), ld_dep(aphi + x[1])), sp2(SC));
             float2 e[9];
             walk_feq(c, xmul2(ax, sp2(sched[0][0])), xmul2(ay, sp2(sched[0][1])), e);
 #pragma unroll

@@ -135,10 +135,7 @@ __device__ __forceinline__ void walk_feq(const Coef& c, float2 ux, float2 uy, fl
 }
 
 constexpr int WALK_WARPS = 4;    // independent warps per CTA
-#ifndef WALK_WB
-#define WALK_WB 2
-#endif
-__host__ __device__ constexpr int walk_minb(int T, bool walls) { return T <= 2 ? 4 : (walls ? WALK_WB : 3); }   // 128 / 168 registers
+__host__ __device__ constexpr int walk_minb(int T, bool walls) { return T <= 2 ? 4 : (walls ? 2 : 3); }   // 128 / 168 / up to 255 (walls) registers
 
 // What a level keeps of its last two rows for the rows that still pull from
 // them, unshifted: the e_y = 0 populations {0, 1, 3} of the last row and the
@@ -202,8 +199,7 @@ __global__ void __launch_bounds__(32 * WALK_WARPS, walk_minb(T, WALLS)) k_walk_d
     const int N = (int)a.ncell;
     extern __shared__ __align__(16) unsigned char walk_sm[];
     __shared__ float sched[T + 1][2];
-    grid_dep_launch();
-    grid_dep_wait();
+    grid_dep_sync();
     const void* const asrc = after_dep(a.src);
     const float* const aua = after_dep(a.ua);
     if (threadIdx.x <= T) {
@@ -295,7 +291,7 @@ __global__ void __launch_bounds__(32 * WALK_WARPS, walk_minb(T, WALLS)) k_walk_d
                     unsigned g[9];
 #pragma unroll
                     for (int i = 0; i < 9; ++i)
-                        g[i] = (unsigned)__ldg(q + i * N + row + c0) | (unsigned)__ldg(q + i * N + row + c1) << 16;
+                        g[i] = (unsigned)ld_dep(q + i * N + row + c0) | (unsigned)ld_dep(q + i * N + row + c1) << 16;
 #pragma unroll
                     for (int i = 0; i < 9; ++i)
                         *reinterpret_cast<unsigned*>(st + Slot::plane * i + Slot::first + 4 * lane) = g[i];

@@ -131,3 +131,33 @@ def test_batch_walk_equals_one_step_launches():
         b.close()
     assert np.array_equal(out[0][0], out[1][0])
     assert torch.equal(out[0][1], out[1][1])
+
+
+@pytest.mark.parametrize("lattice,storage,launch", [
+    (15, "f32", (64, 1)), (15, "f16", (64, 1)), (15, "bf16", (64, 1)), (15, "bf16", (64, 5)), (15, "f16", (128, 9)),
+    (9, "f32", (64, 1)), (9, "bf16", (64, 1)), (9, "f32", (128, 11)), (9, "f16", (128, 12)), (9, "f32", None)])
+def test_overlapping_launches_equal_separate_ones(lattice, storage, launch):
+    """Each launch may start while the one before it drains: many launches in a row on a grid small enough for
+    several to be resident at once, against the same launches with the stream drained after each."""
+    kw = dict(nx=64, ny=24, nz=20, bc_z=("periodic", "periodic")) if lattice == 15 else dict(nx=192, ny=60)
+    D = np.array([[0.03, 0.005, -0.004], [0.005, 0.025, 0.003], [-0.004, 0.003, 0.035]])
+    case = Case(lattice=lattice, storage=storage, bc=("noflux", "noflux"), ukind="row", **kw)
+    phi0, a, sched = case.inputs()
+    chunk = 8 if launch is None or launch[1] > 10 else 1
+    out = []
+    for wait in (True, False):
+        s = Solver(lattice=lattice, nx=case.nx, ny=case.ny, nz=case.nz, storage=storage, bc=case.bc)
+        if launch is not None:
+            s.set_launch(*launch)
+        s.set_D(D if lattice == 15 else case.D)
+        s.set_velocity(torch.from_numpy(a).cuda(), torch.from_numpy(sched).cuda(), kind="row")
+        s.set_phi(torch.from_numpy(phi0).cuda())
+        if wait:
+            for _ in range(400 // chunk):
+                s.step(chunk)
+                torch.cuda.synchronize()
+        else:
+            s.step(400)
+        out.append(s.get_state()[0].cpu().numpy())
+        s.close()
+    assert np.array_equal(out[0], out[1])
