@@ -108,6 +108,7 @@ struct WalkArgs {
     int srow[5];         // schedule rows of u(k - 1) .. u(k - 1 + T), or -1
     void* mid[3];        // SAVE: the states k .. k + T - 2 (FP32)
     int strips, ranges;  // strips of WALK_COLS columns x ranges of rows
+    int eranges;         // ranges of the first and the last strip where they have an x wall, or 0
     int vec;             // pairs are stored as one word (nx even, aligned planes)
     int wide;            // rows are staged by 16-byte copies (nx a multiple of 4, or 8 for 16-bit planes; aligned)
 };

@@ -211,9 +211,18 @@ __global__ void __launch_bounds__(32 * WALK_WARPS, walk_minb(T, WALLS)) k_walk_d
     __syncthreads();
     const int lane = threadIdx.x & 31;
     const int w = blockIdx.x * WALK_WARPS + (threadIdx.x >> 5);
-    if (w >= p.strips * p.ranges) return;
-    const int range = w / p.strips, strip = w - range * p.strips;
-    const int ya = (int)((long long)range * ny / p.ranges), yb = (int)((long long)(range + 1) * ny / p.ranges);
+    int strip, range, ranges = p.ranges;
+    if (WALLS && p.eranges > 0) {   // the strips with an x wall have more ranges
+        const int inner = p.strips - 2, e = w - inner * p.ranges;
+        if (e >= 2 * p.eranges) return;
+        range = e < 0 ? w / inner : e >> 1;
+        strip = e < 0 ? 1 + w - range * inner : ((e & 1) ? p.strips - 1 : 0);
+        if (e >= 0) ranges = p.eranges;
+    } else {
+        if (w >= p.strips * p.ranges) return;
+        range = w / p.strips, strip = w - range * p.strips;
+    }
+    const int ya = (int)((long long)range * ny / ranges), yb = (int)((long long)(range + 1) * ny / ranges);
     if (ya >= yb) return;
     const int x0 = strip * COLS - HALO + 2 * lane;   // even
     const bool xwall = WALLS && a.bcx_lo != BC_PERIODIC;
@@ -524,7 +533,17 @@ cudaError_t walk_d2q9(WalkArgs& p, cudaStream_t st)
     }
     p.strips = (p.a.nx + WALK_COLS - 1) / WALK_COLS;
     p.ranges = walk_ranges(p.strips, p.a.ny, T, sms[dev], per_sm[dev] * WALK_WARPS, nullptr);
-    const int ctas = (p.strips * p.ranges + WALK_WARPS - 1) / WALK_WARPS;
+    int warps = p.strips * p.ranges;
+    if (WALLS && p.a.bcx_lo != BC_PERIODIC && p.strips >= 3) {
+        // a row of a strip with an x wall takes about 1.6 times as long (selects in every level)
+        const int most = sms[dev] * per_sm[dev] * WALK_WARPS;
+        auto total = [&] { return (p.strips - 2) * p.ranges + 2 * p.eranges; };
+        p.eranges = (8 * p.ranges + 4) / 5;
+        while (p.ranges > 1 && total() > most) p.eranges = (8 * --p.ranges + 4) / 5;
+        if (p.eranges > p.a.ny) p.eranges = p.a.ny;
+        warps = total();
+    }
+    const int ctas = (warps + WALK_WARPS - 1) / WALK_WARPS;
     return launch_dependent(k_walk_d2q9<STORE, FIELD, WALLS, T, SAVE>, dim3((unsigned)ctas), dim3(32 * WALK_WARPS), smem, st, p);
 }
 
