@@ -101,14 +101,11 @@ AdjBlock adjoint_block(long long nx)
 // a compile-time choice: behind a run-time test the kernel executed 7 % more
 // instructions for the other models, which never take them.
 template <class L, int UK, int WM, bool DA, typename IX, bool QUAD>
-__global__ void __launch_bounds__(256, (L::Q == 9 && !DA && WM < 2) ? 4 : 3) k_adjoint(const AdjArgs args)
+__global__ void __launch_bounds__(256, (L::Q == 9 && !DA && WM < 2) ? 4 : 3) k_adjoint(const AdjArgs a)
 {
-    AdjArgs a = args;
     grid_dep_sync();
-    a.mu_in = after_dep(a.mu_in);
-    a.fprev = after_dep(a.fprev);
-    a.ua = after_dep(a.ua);
-    a.sched = after_dep(a.sched);
+    const float* const ua = after_dep(a.ua);
+    const float* const sched = after_dep(a.sched);
     static_assert(!QUAD || (L::Q == 9 && UK != U_NONE), "u^2 terms only for D2Q9 with a velocity");
     constexpr bool WALLS = WM == 1, BOX = WM == 2;
     constexpr int Q = L::Q, DIM = L::DIM, NG = ngrad<L>();
@@ -123,7 +120,7 @@ __global__ void __launch_bounds__(256, (L::Q == 9 && !DA && WM < 2) ? 4 : 3) k_a
     const int zs[3] = {z + 1 == nz ? 0 : z + 1, z, z == 0 ? nz - 1 : z - 1};
     const Coef& c = a.c;
     float s_now[3];
-    sched_row_at(a.sched, a.srow, DIM, s_now);
+    sched_row_at(sched, a.srow, DIM, s_now);
 
     float g[NG];
 #pragma unroll
@@ -222,13 +219,13 @@ __global__ void __launch_bounds__(256, (L::Q == 9 && !DA && WM < 2) ? 4 : 3) k_a
         if (dlo || dhi) {
             float up[3] = {0.f, 0.f, 0.f};
             float sp[3];
-            sched_row_at(a.sched, a.srow_prev, DIM, sp);
+            sched_row_at(sched, a.srow_prev, DIM, sp);
             if (UK == U_FIELD) {
 #pragma unroll
-                for (int d = 0; d < DIM; ++d) up[d] = __fmul_rn(__ldg(a.ua + (IX)d * N + cell), sp[d]);
+                for (int d = 0; d < DIM; ++d) up[d] = __fmul_rn(__ldg(ua + (IX)d * N + cell), sp[d]);
             } else if (UK == U_ROW) {
 #pragma unroll
-                for (int d = 0; d < DIM; ++d) up[d] = __fmul_rn(__ldg(a.ua + d * ny + y), sp[d]);
+                for (int d = 0; d < DIM; ++d) up[d] = __fmul_rn(__ldg(ua + d * ny + y), sp[d]);
             }
             const int inward = dlo ? 1 : -1;
             float known = 0.f, wk = 0.f;
@@ -246,13 +243,13 @@ __global__ void __launch_bounds__(256, (L::Q == 9 && !DA && WM < 2) ? 4 : 3) k_a
         }
         float ux = 0.f, uy = 0.f, uz = 0.f;
         if (UK == U_FIELD) {
-            ux = __fmul_rn(__ldg(a.ua + cell), s_now[0]);
-            uy = __fmul_rn(__ldg(a.ua + N + cell), s_now[1]);
-            if (DIM == 3) uz = __fmul_rn(__ldg(a.ua + 2 * N + cell), s_now[2]);
+            ux = __fmul_rn(__ldg(ua + cell), s_now[0]);
+            uy = __fmul_rn(__ldg(ua + N + cell), s_now[1]);
+            if (DIM == 3) uz = __fmul_rn(__ldg(ua + 2 * N + cell), s_now[2]);
         } else if (UK == U_ROW) {
-            ux = __fmul_rn(__ldg(a.ua + y), s_now[0]);
-            uy = __fmul_rn(__ldg(a.ua + ny + y), s_now[1]);
-            if (DIM == 3) uz = __fmul_rn(__ldg(a.ua + 2 * ny + y), s_now[2]);
+            ux = __fmul_rn(__ldg(ua + y), s_now[0]);
+            uy = __fmul_rn(__ldg(ua + ny + y), s_now[1]);
+            if (DIM == 3) uz = __fmul_rn(__ldg(ua + 2 * ny + y), s_now[2]);
         }
         const float u[3] = {ux, uy, uz};
 
