@@ -271,6 +271,13 @@ def time_steps(s, steps, warmup, label=None):
     return e0.elapsed_time(e1) / 1e3
 
 
+def passes(vec: int, steps: int) -> int:
+    """Kernel launches, each one pass over HBM, of `steps` steps on the 4096^2 grid:
+    the fused steps (vec 10) take four a launch there, the last ones of a run two
+    and one; every other launch shape one."""
+    return steps // 4 + (0, 1, 1, 2)[steps % 4] if vec == 10 else steps
+
+
 def copy_rate_same_size(nbytes: int, reps: int = 20):
     """Read + write GB/s of a device-to-device copy of nbytes (torch copy_),
     best of reps: the copy peak at the size of one step's state, beside the
@@ -484,6 +491,12 @@ def d3q15_bench(steps: int, storage: str = "f32"):
             "launch": {"block": shape[0], "vec": shape[1]}}
 
 
+def batch_bytes(mode) -> int:
+    """HBM bytes per lattice update of the 64-channel batch: a PER_STEP launch takes four steps, a
+    persistent one reads and writes the state every step."""
+    return 18 if mode == "per_step" else 72
+
+
 def batch_bench(steps: int):
     """The Taylor-Aris batch workload: 64 uneven channels in one launch per graph
     chunk, moments every step; mode and tile width from the autotuner."""
@@ -527,13 +540,13 @@ def batch_bench(steps: int):
         w, d = timed(n)
         key = m if m == "per_step" else ("persistent_cell_tiles" if tr == 0 else f"persistent_warp_tiles{tr}")
         modes[key] = {
-            "MLUPS_device": cells * n / d / 1e6, "frac_of_" + kind + "_hbm": cells * 72 / (d / n) / 1e9 / peak}
+            "MLUPS_device": cells * n / d / 1e6, "frac_of_" + kind + "_hbm": cells * batch_bytes(m) / (d / n) / 1e9 / peak}
     b.close()
-    gbs = cells * 72 / (dt / n) / 1e9
-    gbs_dev = cells * 72 / (dt_dev / n) / 1e9
+    gbs = cells * batch_bytes(mode) / (dt / n) / 1e9
+    gbs_dev = cells * batch_bytes(mode) / (dt_dev / n) / 1e9
     return {"instances": len(chans), "cells": cells, "steps": n, "MLUPS": cells * n / dt / 1e6,
             "MLUPS_device": cells * n / dt_dev / 1e6,
-            "bytes_per_lu": 72, "achieved_gbs": gbs, f"frac_of_{kind}_hbm": gbs / peak,
+            "bytes_per_lu": batch_bytes(mode), "achieved_gbs": gbs, f"frac_of_{kind}_hbm": gbs / peak,
             f"frac_of_{kind}_hbm_device": gbs_dev / peak,
             "mode": mode, "tile_rows": tile, "modes": modes,
             "timing": "MLUPS: host wall clock around lbm_cde_batch_run (graph replays + per-step moment "
@@ -673,7 +686,8 @@ def main():
     mass_ok = s.sum_phi()
     s.close()
     value = units / dt_max / 1e6
-    avg_launch = dt / args.steps
+    launches = passes(f32_shape[1], args.steps)
+    avg_launch = dt / launches
     peak, peak_kind = peaks()
     achieved = ncell * B_LU[store] / avg_launch / 1e9
     clocks = cs.summary((t_wall0, t_wall1))
@@ -699,9 +713,11 @@ def main():
             shape = sv.autotune(20)
             dtv = time_steps(sv, args.steps, args.warmup)
             sv.close()
-            av = ncell * B_LU[vs] / (dtv / args.steps) / 1e9
+            np_ = passes(shape[1], args.steps)
+            av = ncell * B_LU[vs] / (dtv / np_) / 1e9
             key = vs if tau == TAU else f"{vs}_tau{tau}"
-            variants[key] = {"MLUPS": ncell * args.steps / dtv / 1e6, "bytes_per_lu": B_LU[vs], "tau": tau,
+            variants[key] = {"MLUPS": ncell * args.steps / dtv / 1e6, "bytes_per_lu": B_LU[vs] * np_ / args.steps,
+                             "tau": tau,
                              "achieved_gbs": av, "frac_of_" + peak_kind + "_hbm": av / peak,
                              "launch": {"block": shape[0], "vec": shape[1]}}
         torch.cuda.empty_cache()
@@ -730,11 +746,12 @@ def main():
                    "l2": "inputs larger than L2: 1.21 GB of state per step (129 MB L2)"},
         "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
                      "frac": achieved / peak, "traffic": profile_traffic(store),
-                     "peak_source": peak_kind, "bytes_per_lu": B_LU[store],
+                     "peak_source": peak_kind, "bytes_per_lu": B_LU[store] * launches / args.steps,
                      "copy_gbs_same_size": copy_same,
-                     "kernel": "k_step<D2Q9, F32, FIELD> (one launch per step)",
+                     "kernel": ("k_walk_d2q9<F32, FIELD> (four steps per launch)" if f32_shape[1] == 10 else
+                                "k_step<D2Q9, F32, FIELD> (one launch per step)"),
                      "launch": {"block": f32_shape[0], "vec": f32_shape[1]}},
-        "gpu_launches": args.steps,
+        "gpu_launches": launches,
         "clocks": clocks,
         "variants": variants,
         "adjoint": adjoint,
