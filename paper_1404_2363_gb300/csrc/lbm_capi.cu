@@ -41,6 +41,7 @@ struct lbm_cde_s {
     long long t = 0;
     bool ready = false;
     LaunchCfg cfg{256, 1};
+    int pair_block = 0;                    // default shape with a velocity field: node pairs with this block (0: none)
     cudaStream_t st = nullptr;
     std::string err;
     // adjoint: checkpoints of the forward run, segment recompute buffer, adjoint states
@@ -451,9 +452,18 @@ lbm_status lbm_cde_create(const lbm_cde_desc* desc, lbm_cde_t* out)
     h->cfg.vec = 0;   // fused steps where they apply, else one node per thread
     if (h->q == 15 && h->neq && ncell >= (1LL << 20) && 18LL * ncell < (1LL << 31)) {
         // D3Q15 16-bit forms: the z-walk kernel, or the node pairs, where the rows allow them (256^3 BF16 272 us a
-        // step against 401 with one node per thread; 200 x 101 x 77 39 against 47; but 64^3 10.4 against 8.1)
+        // step against 401 with one node per thread; 200 x 101 x 77 39 against 47; but 64^3 10.4 against 8.1).
+        // The pairs' block takes the width that wastes fewest columns, the widest of those (64 x 225 x 163 BF16: 49 us
+        // with 32 threads, 84 with 64, 59 with one node per thread); they pay with a velocity field (FP16
+        // 320 x 101 x 91 without one: 55 against 49)
         if (d.nx % 64 == 0 && d.ny % 4 == 0) h->cfg = LaunchCfg{128, 9};
-        else if (d.nx % 2 == 0) h->cfg = LaunchCfg{64, 5};
+        else if (d.nx % 2 == 0) {
+            auto columns = [&](int per) { return (d.nx + per - 1) / per * per; };
+            int block = 128;
+            for (int w = 96; w >= 32; w -= 32)
+                if (columns(2 * w) < columns(2 * block)) block = w;
+            if (4 * columns(2 * block) <= 5 * columns(h->cfg.block)) h->pair_block = block;
+        }
     }
     *out = h;
     return LBM_OK;
@@ -558,6 +568,7 @@ lbm_status lbm_cde_step(lbm_cde_t h, int64_t nsteps)
     if (!h->ready) return fail(h, LBM_E_STATE, "set_phi must come before step");
     const bool walls = h->d.bc_lo_y != LBM_BC_PERIODIC;
     const int uk = ukind_internal(h->ukind);
+    const LaunchCfg cfg = h->cfg.vec == 0 && h->pair_block && uk == lbm::U_FIELD ? LaunchCfg{h->pair_block, 5} : h->cfg;
     const bool tma = (h->cfg.vec == 7 || h->cfg.vec == 8) && h->neq && h->q == 9;
     if (tma) {
         const lbm_status ts = ensure_tma_maps(h);
@@ -574,7 +585,7 @@ lbm_status lbm_cde_step(lbm_cde_t h, int64_t nsteps)
             continue;
         }
         if (tma) a.tma = &h->tmaps[h->cur];
-        CK(h, lbm::launch_step(h->q, h->d.storage, uk, walls, h->cfg, a, h->st));
+        CK(h, lbm::launch_step(h->q, h->d.storage, uk, walls, cfg, a, h->st));
         h->cur ^= 1;
         h->t += 1;
         ++n;

@@ -31,7 +31,9 @@ int walk_ranges(int strips, int ny, int T, int sms, int warps, double* cost)
 //             1.5 (16-bit) times as long;
 //   tile:     2.3 us + per wave of one tile per SM: 1 us to load, 0.2 us a step and
 //             0.05 us a row and step (128^2: 6.2 us for 6 steps on 16-row tiles; 256^2: 8.7 on
-//             24 rows; 512^2: 15.7 on 48 rows).
+//             24 rows; 512^2: 15.7 on 48 rows); on grids whose two states do not fit in L2 a tile's
+//             loads and stores come from HBM, which nothing overlaps with one CTA per SM (FP16 2913 x 2240:
+//             77 us a step; without this term the plan took it for 47 and the walk, 52, for slower).
 // The tile kernel wins below about 1M nodes (us a step: 512^2 2.5, walk 8.0, one step 6.2; 896^2 6.4, 9.2,
 // 10.3), the walk above (1024^2: 7.7 against 8.5 and 12.3; 2048^2: 21, 43, 52; 4096^2: 72, 166, 192).
 FusePlan plan_fused(int store, int nx, int ny, int sms, long long left, int kinds)
@@ -39,6 +41,8 @@ FusePlan plan_fused(int store, int nx, int ny, int sms, long long left, int kind
     const double n = (double)nx * ny;
     const double single = n * 80 / 6.8e6;
     const double slow = store == ST_F32 ? (nx % 4 ? 1.1 : 1.0) : (nx % 8 ? 1.5 : 1.0);
+    const double bytes = store == ST_F32 ? 80 : 52;   // a node's, read and written
+    const double fetch = n * bytes > 1e8 ? 64 * bytes * sms / 6.8e6 : 0;   // us a row of every SM's tile
     double best = kinds != FUSE_ANY ? 1e300 : (single > 4.1 ? single : 4.1);
     FusePlan p{1, 0};
     for (int T = 2; T <= 4 && T <= left && (kinds & FUSE_WALK); T += 2) {
@@ -53,7 +57,7 @@ FusePlan plan_fused(int store, int nx, int ny, int sms, long long left, int kind
         for (int rows = 2 * T + 2; rows <= TILE_ROWS; rows += 2) {
             const int h = rows - 2 * T;
             const long long tiles = (long long)((nx + 63 - 2 * T) / (64 - 2 * T)) * ((ny + h - 1) / h);
-            const double c = 2.3 + (double)((tiles + sms - 1) / sms) * (1.0 + 0.2 * T + 0.05 * T * (h + T - 1));
+            const double c = 2.3 + (double)((tiles + sms - 1) / sms) * (1.0 + fetch * rows + 0.2 * T + 0.05 * T * (h + T - 1));
             if (c / T < best) {
                 best = c / T;
                 p = {T, rows};

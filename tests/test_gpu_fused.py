@@ -161,3 +161,27 @@ def test_overlapping_launches_equal_separate_ones(lattice, storage, launch):
         out.append(s.get_state()[0].cpu().numpy())
         s.close()
     assert np.array_equal(out[0], out[1])
+
+
+@pytest.mark.parametrize("nx,ny,nz,ukind,shape", [
+    (64, 225, 74, "field", (32, 5)), (96, 133, 90, "field", (96, 1)), (200, 101, 53, "field", (128, 5)),
+    (200, 101, 53, "none", (224, 1)), (64, 128, 130, "none", (128, 9)), (64, 128, 130, "field", (128, 9))])
+def test_default_d3q15_16bit_kernel(nx, ny, nz, ukind, shape):
+    """The default of the D3Q15 16-bit forms from 2^20 nodes on: the bits of the kernel that the rule on the row
+    length and the velocity names (one node per thread gives its bits with any block)."""
+    g = np.random.default_rng(3)
+    phi0 = torch.from_numpy((0.5 + 0.1 * g.random((nz, ny, nx))).astype(np.float32)).cuda()
+    a = torch.from_numpy((0.05 * g.random((3, nz, ny, nx)) - 0.025).astype(np.float32)).cuda()
+    out = []
+    for launch in (None, shape):
+        s = Solver(lattice=15, nx=nx, ny=ny, nz=nz, storage="bf16")
+        if launch is not None:
+            s.set_launch(*launch)
+        s.set_D([[0.03, 0.005, -0.004], [0.005, 0.025, 0.003], [-0.004, 0.003, 0.035]])
+        if ukind == "field":
+            s.set_velocity(a)
+        s.set_phi(phi0)
+        s.step(6)
+        out.append(s.get_state()[0].cpu().numpy())
+        s.close()
+    assert np.array_equal(out[0], out[1])
