@@ -1131,11 +1131,20 @@ lbm_status lbm_cde_backward(lbm_cde_t h, const float* dL_dphiN_dev, float* dL_dp
         if (t == 0) return static_cast<float*>(h->ck[j]);
         return reinterpret_cast<float*>(static_cast<char*>(segbuf[j & 1]) + sb * (t - 1));
     };
+    // The recompute runs beside the reverse steps, which are what the sweep waits for. Several steps a launch take
+    // less time but leave the reverse steps no room (the walk's CTAs hold an SM's registers for tens of us), so on
+    // most grids one step a launch ends the sweep sooner (us of backward a step, fused against single steps: 1024^2
+    // between walls 40.2 / 34.7 with a field and 37.5 / 31.9 without, 1537 x 1023 59.7 / 50.8, 4096^2 with a field
+    // 479 / 457). Fused steps where the sweep waits for the recompute's launches or memory: 128^2 6.6 / 7.0; from 2^22
+    // nodes on without a velocity field (4096^2 397 / 422) and with x walls (705 / 752); and where the caller chose
+    // the walk or the tile kernel.
+    const bool fused = h->cfg.vec == 11 || h->cfg.vec == 12 || h->ncell < (1LL << 15) ||
+                       (h->ncell >= (1LL << 22) && (uk != lbm::U_FIELD || h->d.bc_lo_x != LBM_BC_PERIODIC));
     // recompute B_{jK+1} .. B_{end-1} of segment j from its checkpoint, on stream rs
     auto recompute = [&](int64_t j, cudaStream_t rs) -> lbm_status {
         const int64_t start = j * K, end = std::min(start + K, Nst);
         for (int64_t t = 1; t < end - start;) {
-            const lbm::FusePlan plan = fuse_plan(h, end - start - t);
+            const lbm::FusePlan plan = fused ? fuse_plan(h, end - start - t) : lbm::FusePlan{1, 0};
             StepArgs a = make_args(h, 0);
             a.src = seg_state(j, t - 1);
             a.dst = seg_state(j, t + plan.T - 1);

@@ -56,3 +56,12 @@ def test_reverse_step_of_multi_row_blocks():
     forward = step_us(s)
     assert backward_us(s, want_da=True) < 3.1 * forward
     s.close()
+
+
+def test_recompute_leaves_the_reverse_steps_room():
+    """The sweep with the default launches against one step a launch throughout (it was 1.18 times as long)."""
+    s = solver((1024, 1024), bc="noflux", u="none")
+    default = backward_us(s)
+    s.set_launch(256, 1)
+    assert default < 1.08 * backward_us(s)
+    s.close()
