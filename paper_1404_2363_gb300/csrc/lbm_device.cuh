@@ -388,14 +388,23 @@ template <> struct StT<ST_BF16> { using T = __nv_bfloat16; };
 // instead of its subnormals, while |g| up to 32 remains representable.
 constexpr float F16_SCALE = 2048.0f;
 
-__device__ __forceinline__ float ldg_f(const float* p) { return ld_dep(p); }
-__device__ __forceinline__ float ldg_f(const __half* p) {
-    return __half2float(__ushort_as_half(ld_dep(reinterpret_cast<const unsigned short*>(p)))) *
-           (1.0f / F16_SCALE);
+// a 16-bit value: LD_PLAIN reads it in the type that is stored
+template <int LD, class T>
+__device__ __forceinline__ T ld_16(const T* p)
+{
+    if constexpr (LD == LD_PLAIN) return *p;
+    else {
+        const unsigned short w = ld_src<LD>(reinterpret_cast<const unsigned short*>(p));
+        if constexpr (std::is_same<T, __half>::value) return __ushort_as_half(w);
+        else return __ushort_as_bfloat16(w);
+    }
 }
-__device__ __forceinline__ float ldg_f(const __nv_bfloat16* p) {
-    return __bfloat162float(__ushort_as_bfloat16(ld_dep(reinterpret_cast<const unsigned short*>(p))));
-}
+template <int LD = LD_READONLY>
+__device__ __forceinline__ float ldg_f(const float* p) { return ld_src<LD>(p); }
+template <int LD = LD_READONLY>
+__device__ __forceinline__ float ldg_f(const __half* p) { return __half2float(ld_16<LD>(p)) * (1.0f / F16_SCALE); }
+template <int LD = LD_READONLY>
+__device__ __forceinline__ float ldg_f(const __nv_bfloat16* p) { return __bfloat162float(ld_16<LD>(p)); }
 __device__ __forceinline__ void st_f(float* p, float v) { *p = v; }
 __device__ __forceinline__ void st_f(__half* p, float v) { *p = __float2half_rn(v * F16_SCALE); }
 __device__ __forceinline__ void st_f(__nv_bfloat16* p, float v) { *p = __float2bfloat16_rn(v); }
@@ -417,11 +426,12 @@ __device__ __forceinline__ void sched_at(const StepArgs& a, long long k, int dim
 }
 
 // the same from a row computed on the host (row < 0: no schedule)
+template <int LD = LD_ORDERED>
 __device__ __forceinline__ void sched_row_at(const float* sched, int row, int dim, float* s)
 {
     s[0] = s[1] = s[2] = 1.f;
     if (row >= 0)
-        for (int d = 0; d < dim; ++d) s[d] = __ldg(sched + row * dim + d);
+        for (int d = 0; d < dim; ++d) s[d] = ld_vel<LD>(sched + row * dim + d);
 }
 
 // u(x, k) = a(x) s(k) for a field, a(y) s(k) for a row profile, 0 otherwise.
@@ -455,27 +465,27 @@ __device__ __forceinline__ void vel_at(const StepArgs& a, long long cell, int y,
 // ---------------------------------------------------------------------------
 // IX is the index type: int when every plane offset fits in 31 bits (fewer
 // address instructions), long long otherwise.
-template <int UK, int DIM, typename IX>
+template <int UK, int DIM, typename IX, int LD = LD_ORDERED>
 __device__ __forceinline__ void vel_ix(const StepArgs& a, IX N, IX cell, int y, const float* s,
                                        float& ux, float& uy, float& uz)
 {
     ux = uy = uz = 0.f;
     if (UK == U_FIELD) {
-        ux = __fmul_rn(__ldg(a.ua + cell), s[0]);
-        uy = __fmul_rn(__ldg(a.ua + N + cell), s[1]);
-        if (DIM == 3) uz = __fmul_rn(__ldg(a.ua + 2 * N + cell), s[2]);
+        ux = __fmul_rn(ld_vel<LD>(a.ua + cell), s[0]);
+        uy = __fmul_rn(ld_vel<LD>(a.ua + N + cell), s[1]);
+        if (DIM == 3) uz = __fmul_rn(ld_vel<LD>(a.ua + 2 * N + cell), s[2]);
     } else if (UK == U_ROW) {
-        ux = __fmul_rn(__ldg(a.ua + y), s[0]);
-        uy = __fmul_rn(__ldg(a.ua + a.ny + y), s[1]);
-        if (DIM == 3) uz = __fmul_rn(__ldg(a.ua + 2 * a.ny + y), s[2]);
+        ux = __fmul_rn(ld_vel<LD>(a.ua + y), s[0]);
+        uy = __fmul_rn(ld_vel<LD>(a.ua + a.ny + y), s[1]);
+        if (DIM == 3) uz = __fmul_rn(ld_vel<LD>(a.ua + 2 * a.ny + y), s[2]);
     }
 }
 
-template <class L, int STORE, int UK, bool WALLS, int VEC, typename IX>
+template <class L, int STORE, int UK, bool WALLS, int VEC, typename IX, int LD>
 __global__ void __launch_bounds__(256) k_step(const StepArgs args)
 {
-    StepArgs a = args;
-    step_after_dep(a);
+    StepArgsLD<LD> a = args;
+    step_after_dep<LD>(a);
     using T = typename StT<STORE>::T;
     constexpr int Q = L::Q;
     constexpr bool NEQ = (STORE != ST_F32);
@@ -491,8 +501,8 @@ __global__ void __launch_bounds__(256) k_step(const StepArgs args)
 
     float s_now[3], s_prev[3];
     if (UK != U_NONE) {
-        sched_row_at(a.sched, a.srow_now, L::DIM, s_now);
-        sched_row_at(a.sched, a.srow_prev, L::DIM, s_prev);
+        sched_row_at<LD>(a.sched, a.srow_now, L::DIM, s_now);
+        sched_row_at<LD>(a.sched, a.srow_prev, L::DIM, s_prev);
     }
 
     float f[VEC][Q];
@@ -508,11 +518,11 @@ __global__ void __launch_bounds__(256) k_step(const StepArgs args)
 #pragma unroll
         for (int i = 0; i < Q; ++i) {
             const IX sc = (IX)xs[L::ex(i) + 1] + (IX)nx * ((IX)ys[L::ey(i) + 1] + (IX)ny * (IX)zs[L::ez(i) + 1]);
-            float v = ldg_f(src + (IX)i * N + sc);
+            float v = ldg_f<LD>(src + (IX)i * N + sc);
             if (NEQ) {
                 float ux, uy, uz;
-                vel_ix<UK, L::DIM, IX>(a, N, sc, ys[L::ey(i) + 1], s_prev, ux, uy, uz);
-                v = fmaf(ld_dep(a.phi_src + sc), feq_unit<L>(a.c, i, ux, uy, uz), v);
+                vel_ix<UK, L::DIM, IX, LD>(a, N, sc, ys[L::ey(i) + 1], s_prev, ux, uy, uz);
+                v = fmaf(ld_src<LD>(a.phi_src + sc), feq_unit<L>(a.c, i, ux, uy, uz), v);
             }
             f[j][i] = v;
         }
@@ -532,18 +542,18 @@ __global__ void __launch_bounds__(256) k_step(const StepArgs args)
                         if (L::ey(i) != 0 && ((L::ey(i) == 1) == lo)) f[j][i] = f[j][mirror_y<L>(i)];
                 } else if (kind == BC_BOUNCE) {
                     float ux = 0.f, uy = 0.f, uz = 0.f;
-                    if (NEQ) vel_ix<UK, L::DIM, IX>(a, N, cell[j], y, s_prev, ux, uy, uz);
+                    if (NEQ) vel_ix<UK, L::DIM, IX, LD>(a, N, cell[j], y, s_prev, ux, uy, uz);
 #pragma unroll
                     for (int i = 0; i < Q; ++i)
                         if (L::ey(i) != 0 && ((L::ey(i) == 1) == lo)) {
                             const int o = opposite<L>(i);
-                            float v = ldg_f(src + (IX)o * N + cell[j]);
-                            if (NEQ) v = fmaf(ld_dep(a.phi_src + cell[j]), feq_unit<L>(a.c, o, ux, uy, uz), v);
+                            float v = ldg_f<LD>(src + (IX)o * N + cell[j]);
+                            if (NEQ) v = fmaf(ld_src<LD>(a.phi_src + cell[j]), feq_unit<L>(a.c, o, ux, uy, uz), v);
                             f[j][i] = v;
                         }
                 } else {  // Dirichlet
                     float ux, uy, uz;
-                    vel_ix<UK, L::DIM, IX>(a, N, cell[j], y, s_prev, ux, uy, uz);
+                    vel_ix<UK, L::DIM, IX, LD>(a, N, cell[j], y, s_prev, ux, uy, uz);
                     float known = 0.f, wk = 0.f;
 #pragma unroll
                     for (int i = 0; i < Q; ++i) {
@@ -559,7 +569,7 @@ __global__ void __launch_bounds__(256) k_step(const StepArgs args)
             }
         }
         float ux, uy, uz;
-        vel_ix<UK, L::DIM, IX>(a, N, cell[j], y, s_now, ux, uy, uz);
+        vel_ix<UK, L::DIM, IX, LD>(a, N, cell[j], y, s_now, ux, uy, uz);
         const float phi = collide<L, NEQ>(f[j], ux, uy, uz, a.c);
         if (!live[j]) continue;
 #pragma unroll
@@ -593,11 +603,11 @@ __device__ __forceinline__ int reflect_mask(int i, int mask)
     return r;
 }
 
-template <class L, int STORE, int UK, typename IX>
+template <class L, int STORE, int UK, typename IX, int LD>
 __global__ void __launch_bounds__(256) k_step_box(const StepArgs args)
 {
-    StepArgs a = args;
-    step_after_dep(a);
+    StepArgsLD<LD> a = args;
+    step_after_dep<LD>(a);
     using T = typename StT<STORE>::T;
     constexpr int Q = L::Q;
     constexpr bool NEQ = (STORE != ST_F32);
@@ -606,18 +616,18 @@ __global__ void __launch_bounds__(256) k_step_box(const StepArgs args)
     const int y = blockIdx.y, z = blockIdx.z;
     if (x >= nx) return;
     const IX N = (IX)a.ncell;
-    const T* __restrict__ src = static_cast<const T*>(a.src);
-    T* __restrict__ dst = static_cast<T*>(a.dst);
+    const T* src = static_cast<const T*>(a.src);
+    T* dst = static_cast<T*>(a.dst);
     const int pos[3] = {x, y, z}, n[3] = {nx, ny, nz};
     const int klo[3] = {a.bcx_lo, a.bc_lo, a.bcz_lo}, khi[3] = {a.bcx_hi, a.bc_hi, a.bcz_hi};
     const IX cell = (IX)x + (IX)nx * ((IX)y + (IX)ny * (IX)z);
     float s_now[3], s_prev[3];
     if (UK != U_NONE) {
-        sched_row_at(a.sched, a.srow_now, L::DIM, s_now);
-        sched_row_at(a.sched, a.srow_prev, L::DIM, s_prev);
+        sched_row_at<LD>(a.sched, a.srow_now, L::DIM, s_now);
+        sched_row_at<LD>(a.sched, a.srow_prev, L::DIM, s_prev);
     }
     float uxp = 0.f, uyp = 0.f, uzp = 0.f;   // u(k - 1) at the node (bounce-back decode, Dirichlet)
-    vel_ix<UK, L::DIM, IX>(a, N, cell, y, s_prev, uxp, uyp, uzp);
+    vel_ix<UK, L::DIM, IX, LD>(a, N, cell, y, s_prev, uxp, uyp, uzp);
     float w[Q];
     int nf[Q];
 #pragma unroll
@@ -642,16 +652,16 @@ __global__ void __launch_bounds__(256) k_step_box(const StepArgs args)
         float v = 0.f;
         if (!out) {
             const IX sc = (IX)sp[0] + (IX)nx * ((IX)sp[1] + (IX)ny * (IX)sp[2]);
-            v = ldg_f(src + (IX)i * N + sc);
+            v = ldg_f<LD>(src + (IX)i * N + sc);
             if (NEQ) {
                 float ux, uy, uz;
-                vel_ix<UK, L::DIM, IX>(a, N, sc, sp[1], s_prev, ux, uy, uz);
-                v = fmaf(ld_dep(a.phi_src + sc), feq_unit<L>(a.c, i, ux, uy, uz), v);
+                vel_ix<UK, L::DIM, IX, LD>(a, N, sc, sp[1], s_prev, ux, uy, uz);
+                v = fmaf(ld_src<LD>(a.phi_src + sc), feq_unit<L>(a.c, i, ux, uy, uz), v);
             }
         } else if (bb) {
             const int o = opposite<L>(i);
-            v = ldg_f(src + (IX)o * N + cell);
-            if (NEQ) v = fmaf(ld_dep(a.phi_src + cell), feq_unit<L>(a.c, o, uxp, uyp, uzp), v);
+            v = ldg_f<LD>(src + (IX)o * N + cell);
+            if (NEQ) v = fmaf(ld_src<LD>(a.phi_src + cell), feq_unit<L>(a.c, o, uxp, uyp, uzp), v);
         }
         w[i] = v;
     }
@@ -681,7 +691,7 @@ __global__ void __launch_bounds__(256) k_step_box(const StepArgs args)
             if (L::ey(i) == inward) f[i] = __fmul_rn(ps, feq_unit<L>(a.c, i, uxp, uyp, uzp));
     }
     float ux, uy, uz;
-    vel_ix<UK, L::DIM, IX>(a, N, cell, y, s_now, ux, uy, uz);
+    vel_ix<UK, L::DIM, IX, LD>(a, N, cell, y, s_now, ux, uy, uz);
     const float phi = collide<L, NEQ>(f, ux, uy, uz, a.c);
 #pragma unroll
     for (int i = 0; i < Q; ++i) st_f(dst + (IX)i * N + cell, f[i]);

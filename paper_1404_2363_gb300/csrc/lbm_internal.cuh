@@ -7,6 +7,7 @@
 #include <cuda_fp16.h>
 #include <cuda_bf16.h>
 #include <stdint.h>
+#include <type_traits>
 
 namespace lbm {
 
@@ -272,20 +273,54 @@ __device__ __forceinline__ P after_dep(P p)
     return reinterpret_cast<P>(v);
 }
 
-__device__ __forceinline__ void step_after_dep(StepArgs& a)
+// The forms a one-step kernel reads its source in. The first two are for dependent
+// launches; which one a kernel takes was measured (the compiler places, merges and
+// addresses their loads differently): see the launchers.
+//   LD_ORDERED:  ld_dep, and __ldg of pointers that went through after_dep()
+//   LD_PLAIN:    plain loads (velocity too). They stay behind grid_dep_sync(), which clobbers
+//                memory, and no pointer in the kernel is __restrict__ or read in another type than
+//                it is written in, so that nothing tells the compiler that the data is read-only
+//   LD_READONLY: __ldg throughout, no wait: for ordinary launches, which start when the
+//                previous kernel has ended
+enum { LD_ORDERED = 0, LD_PLAIN = 1, LD_READONLY = 2 };
+
+template <int LD, class T>
+__device__ __forceinline__ T ld_src(const T* p)
 {
-    grid_dep_sync();
-    a.src = after_dep(a.src);
-    a.phi_src = after_dep(a.phi_src);
-    a.ua = after_dep(a.ua);
-    a.sched = after_dep(a.sched);
+    if constexpr (LD == LD_ORDERED) return ld_dep(p);
+    else if constexpr (LD == LD_PLAIN) return *p;
+    else return __ldg(p);
+}
+template <int LD, class T>
+__device__ __forceinline__ T ld_vel(const T* p)   // what the caller owns
+{
+    if constexpr (LD == LD_PLAIN) return *p;
+    else return __ldg(p);
+}
+
+// The arguments a kernel of form LD works with: a copy whose pointers went through
+// after_dep(), or the kernel parameters themselves (as uniform operands).
+template <int LD>
+using StepArgsLD = typename std::conditional<LD == LD_ORDERED, StepArgs, const StepArgs&>::type;
+template <int LD>
+__device__ __forceinline__ void step_after_dep(StepArgsLD<LD>& a)
+{
+    if constexpr (LD != LD_READONLY) grid_dep_sync();
+    if constexpr (LD == LD_ORDERED) {
+        a.src = after_dep(a.src);
+        a.phi_src = after_dep(a.phi_src);
+        a.ua = after_dep(a.ua);
+        a.sched = after_dep(a.sched);
+    }
 }
 
 // A launch that may start while the stream's previous kernel drains: it waits
 // in grid_dep_sync() before it reads anything. From launch to launch of dependent
 // kernels: D3Q15 40^3 4.6 -> 3.4 us a step, 64^3 8.2 -> 5.8, 97 x 80 x 66 12.4 -> 10.2.
+// overlap = false: an ordinary launch (LD_READONLY).
 template <class A>
-cudaError_t launch_dependent(void (*kernel)(A), dim3 grid, dim3 block, int smem, cudaStream_t st, const A& args)
+cudaError_t launch_dependent(void (*kernel)(A), dim3 grid, dim3 block, int smem, cudaStream_t st, const A& args,
+                             bool overlap = true)
 {
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = grid;
@@ -296,7 +331,7 @@ cudaError_t launch_dependent(void (*kernel)(A), dim3 grid, dim3 block, int smem,
     at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     at[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = at;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = overlap ? 1 : 0;
     return cudaLaunchKernelEx(&cfg, kernel, args);
 }
 

@@ -161,11 +161,14 @@ template <> struct Pair<ST_BF16> {
     }
 };
 
-template <class T2>
-__device__ __forceinline__ T2 ldg_pair(const T2* p)
+template <int LD, class T2>
+__device__ __forceinline__ T2 ld_pair(const T2* p)
 {
-    const unsigned w = ld_dep(reinterpret_cast<const unsigned*>(p));
-    return *reinterpret_cast<const T2*>(&w);
+    if constexpr (LD == LD_PLAIN) return *p;
+    else {
+        const unsigned w = ld_src<LD>(reinterpret_cast<const unsigned*>(p));
+        return *reinterpret_cast<const T2*>(&w);
+    }
 }
 
 // f^eq_i / phi = w_i + k_i e_i.u for two nodes (feq_unit<D2Q9>)
@@ -257,9 +260,9 @@ __global__ void __launch_bounds__(256) k_step_pair_d2q9(const StepArgs a)
         const int r = ey + 1, cp = 1 - ex;
         const T2* row = src + i * NP + ys[r] * nxp;
         T2 h;
-        if (ex == 0) h = ldg_pair(row + x0 / 2);
-        else if (ex > 0) h = P::join(ldg_pair(row + xl / 2), ldg_pair(row + x0 / 2));
-        else h = P::join(ldg_pair(row + x0 / 2), ldg_pair(row + xr / 2));
+        if (ex == 0) h = ld_pair<LD_READONLY>(row + x0 / 2);
+        else if (ex > 0) h = P::join(ld_pair<LD_READONLY>(row + xl / 2), ld_pair<LD_READONLY>(row + x0 / 2));
+        else h = P::join(ld_pair<LD_READONLY>(row + x0 / 2), ld_pair<LD_READONLY>(row + xr / 2));
         f[i] = fma2(Ps[r][cp], feq_unit_pair(c, i, Ux[r][cp], Uy[r][cp]), P::to_f(h));
     }
     const int cellp = y * nxp + x0 / 2;
@@ -279,7 +282,7 @@ __global__ void __launch_bounds__(256) k_step_pair_d2q9(const StepArgs a)
                 for (int i = 0; i < 9; ++i)
                     if (L::ey(i) == inward) {
                         const int o = opposite<L>(i);
-                        const float2 g = P::to_f(ldg_pair(src + o * NP + cellp));
+                        const float2 g = P::to_f(ld_pair<LD_READONLY>(src + o * NP + cellp));
                         f[i] = fma2(Ps[1][1], feq_unit_pair(c, o, uxp, uyp), g);
                     }
             } else {   // Dirichlet

@@ -19,11 +19,12 @@ namespace lbm {
 
 // (v(x0 - e_x), v(x0 + 1 - e_x)) of one FP32 plane row; c = (v(x0), v(x0 + 1)),
 // xlo = column x0 - 1, xhi = column x0 + 2 (periodic)
+template <int LD>
 __device__ __forceinline__ float2 pair_window(const float* row, float2 c, int ex, int xlo, int xhi)
 {
     if (ex == 0) return c;
-    if (ex > 0) return make_float2(ld_dep(row + xlo), c.x);
-    return make_float2(c.y, ld_dep(row + xhi));
+    if (ex > 0) return make_float2(ld_src<LD>(row + xlo), c.x);
+    return make_float2(c.y, ld_src<LD>(row + xhi));
 }
 
 // f^eq_i / phi = w_i + k_i e_i.u for two nodes with u given (wall rules)
@@ -47,11 +48,11 @@ __device__ __forceinline__ float2 feq_unit_pair15(float w0, float wa, float wd, 
 }
 
 // Needs nx even and 18 ncell < 2^31 (int offsets; checked by the launcher).
-template <int STORE, int UK, bool WALLS>
+template <int STORE, int UK, bool WALLS, int LD>
 __global__ void __launch_bounds__(256) k_step_pair_d3q15(const StepArgs args)
 {
-    StepArgs a = args;
-    step_after_dep(a);
+    StepArgsLD<LD> a = args;
+    step_after_dep<LD>(a);
     using P = Pair<STORE>;
     using T2 = typename P::T2;
     using L = D3Q15;
@@ -68,12 +69,12 @@ __global__ void __launch_bounds__(256) k_step_pair_d3q15(const StepArgs args)
     const int ys[3] = {y + 1 == ny ? 0 : y + 1, y, y == 0 ? ny - 1 : y - 1};
     const int zs[3] = {z + 1 == nz ? 0 : z + 1, z, z == 0 ? nz - 1 : z - 1};
     const Coef& c = a.c;
-    const T2* __restrict__ src = static_cast<const T2*>(a.src);   // pair index = cell / 2
-    T2* __restrict__ dst = static_cast<T2*>(a.dst);
+    const T2* src = static_cast<const T2*>(a.src);   // pair index = cell / 2
+    T2* dst = static_cast<T2*>(a.dst);
     const int NP = N / 2;
     float s_now[3], s_prev[3];
-    sched_row_at(a.sched, a.srow_now, 3, s_now);
-    sched_row_at(a.sched, a.srow_prev, 3, s_prev);
+    sched_row_at<LD>(a.sched, a.srow_now, 3, s_now);
+    sched_row_at<LD>(a.sched, a.srow_prev, 3, s_prev);
     const float w0 = c.w0 * SC, wa = c.wa * SC, wd = c.wd * SC;   // exact (power of two)
     const float ka = c.ka * SC, kd = c.kd * SC;
     float kas[3], kds[3];   // slopes with the schedule factor of u(k - 1)
@@ -91,11 +92,11 @@ __global__ void __launch_bounds__(256) k_step_pair_d3q15(const StepArgs args)
         const int row = (ys[ey + 1] + ny * zs[ez + 1]) * nx;   // first cell of the source row
         const T2* prow = src + (i * N + row) / 2;
         T2 h;
-        if (ex == 0) h = ldg_pair(prow + x0 / 2);
-        else if (ex > 0) h = P::join(ldg_pair(prow + xlp / 2), ldg_pair(prow + x0 / 2));
-        else h = P::join(ldg_pair(prow + x0 / 2), ldg_pair(prow + xhi / 2));
+        if (ex == 0) h = ld_pair<LD>(prow + x0 / 2);
+        else if (ex > 0) h = P::join(ld_pair<LD>(prow + xlp / 2), ld_pair<LD>(prow + x0 / 2));
+        else h = P::join(ld_pair<LD>(prow + x0 / 2), ld_pair<LD>(prow + xhi / 2));
         const float* prw = a.phi_src + row;
-        const float2 ps = pair_window(prw, ld_dep(reinterpret_cast<const float2*>(prw + x0)), ex, xlo, xhi);
+        const float2 ps = pair_window<LD>(prw, ld_src<LD>(reinterpret_cast<const float2*>(prw + x0)), ex, xlo, xhi);
         const int wc = wclass<L>(i);
         float2 e = sp2(wc == 0 ? w0 : (wc == 1 ? wa : wd));
         if (UK == U_FIELD) {
@@ -105,14 +106,14 @@ __global__ void __launch_bounds__(256) k_step_pair_d3q15(const StepArgs args)
             for (int d = 0; d < 3; ++d) {
                 if (ed[d] == 0) continue;
                 const float* ar = a.ua + d * N + row;
-                const float2 ad = pair_window(ar, ld_dep(reinterpret_cast<const float2*>(ar + x0)), ex, xlo, xhi);
+                const float2 ad = pair_window<LD>(ar, ld_src<LD>(reinterpret_cast<const float2*>(ar + x0)), ex, xlo, xhi);
                 e = fma2(sp2(ed[d] > 0 ? ks[d] : -ks[d]), ad, e);
             }
         } else if (UK == U_ROW && wc != 0) {
             const int yr = ys[ey + 1];
-            const float ux = __fmul_rn(__ldg(a.ua + yr), s_prev[0]);
-            const float uy = __fmul_rn(__ldg(a.ua + ny + yr), s_prev[1]);
-            const float uz = __fmul_rn(__ldg(a.ua + 2 * ny + yr), s_prev[2]);
+            const float ux = __fmul_rn(ld_vel<LD>(a.ua + yr), s_prev[0]);
+            const float uy = __fmul_rn(ld_vel<LD>(a.ua + ny + yr), s_prev[1]);
+            const float uz = __fmul_rn(ld_vel<LD>(a.ua + 2 * ny + yr), s_prev[2]);
             e = sp2(fmaf(wc == 1 ? ka : kd, e_dot<L>(i, ux, uy, uz), wc == 1 ? wa : wd));
         }
         f[i] = fma2(ps, e, P::to_f_raw(h));
@@ -124,10 +125,10 @@ __global__ void __launch_bounds__(256) k_step_pair_d3q15(const StepArgs args)
     float2 ao[3] = {sp2(0.f), sp2(0.f), sp2(0.f)};
     if (UK == U_FIELD) {
 #pragma unroll
-        for (int d = 0; d < 3; ++d) ao[d] = __ldg(reinterpret_cast<const float2*>(a.ua + d * N + cell));
+        for (int d = 0; d < 3; ++d) ao[d] = ld_vel<LD>(reinterpret_cast<const float2*>(a.ua + d * N + cell));
     } else if (UK == U_ROW) {
 #pragma unroll
-        for (int d = 0; d < 3; ++d) ao[d] = sp2(__ldg(a.ua + d * ny + y));
+        for (int d = 0; d < 3; ++d) ao[d] = sp2(ld_vel<LD>(a.ua + d * ny + y));
     }
     if (WALLS) {
         const bool lo = (y == 0) && a.bc_lo != BC_PERIODIC;
@@ -143,12 +144,12 @@ __global__ void __launch_bounds__(256) k_step_pair_d3q15(const StepArgs args)
                 for (int i = 0; i < 15; ++i)
                     if (L::ey(i) == inward) f[i] = f[mirror_y<L>(i)];
             } else if (kind == BC_BOUNCE) {
-                const float2 po = ld_dep(reinterpret_cast<const float2*>(a.phi_src + cell));
+                const float2 po = ld_src<LD>(reinterpret_cast<const float2*>(a.phi_src + cell));
 #pragma unroll
                 for (int i = 0; i < 15; ++i)
                     if (L::ey(i) == inward) {
                         const int o = opposite<L>(i);
-                        const float2 g = P::to_f_raw(ldg_pair(src + o * NP + cellp));
+                        const float2 g = P::to_f_raw(ld_pair<LD>(src + o * NP + cellp));
                         f[i] = fma2(po, feq_unit_pair15(w0, wa, wd, ka, kd, o, up[0], up[1], up[2]), g);
                     }
             } else {   // Dirichlet

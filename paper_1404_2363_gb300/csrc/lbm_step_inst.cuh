@@ -16,8 +16,8 @@ static cudaError_t step_vec(LaunchCfg cfg, const StepArgs& a, cudaStream_t st)
         // walls on the x or z faces: the general one-node kernel, whatever the launch shape
         dim3 grid((unsigned)((a.nx + 255) / 256), (unsigned)a.ny, (unsigned)a.nz);
         if ((long long)(L::Q + 3) * a.ncell < (1LL << 31))
-            return launch_dependent(k_step_box<L, STORE, UK, int>, grid, dim3(256), 0, st, a);
-        return launch_dependent(k_step_box<L, STORE, UK, long long>, grid, dim3(256), 0, st, a);
+            return launch_dependent(k_step_box<L, STORE, UK, int, LD_PLAIN>, grid, dim3(256), 0, st, a);
+        return launch_dependent(k_step_box<L, STORE, UK, long long, LD_PLAIN>, grid, dim3(256), 0, st, a);
     }
     if constexpr (L::Q == 9) {
         if (cfg.vec == 6 && quad_ok(a, UK)) {
@@ -36,7 +36,7 @@ static cudaError_t step_vec(LaunchCfg cfg, const StepArgs& a, cudaStream_t st)
             // node-pair variant (paired FP32 arithmetic, two adjacent nodes per thread)
             const int per = 2 * cfg.block;
             dim3 grid((unsigned)((a.nx + per - 1) / per), (unsigned)a.ny, (unsigned)a.nz);
-            return launch_dependent(k_step_pair_d3q15<STORE, UK, WALLS>, grid, dim3((unsigned)cfg.block), 0, st, a);
+            return launch_dependent(k_step_pair_d3q15<STORE, UK, WALLS, LD_ORDERED>, grid, dim3((unsigned)cfg.block), 0, st, a);
         }
     }
     if constexpr (L::Q == 9 && STORE != ST_F32) {
@@ -58,10 +58,10 @@ static cudaError_t step_vec(LaunchCfg cfg, const StepArgs& a, cudaStream_t st)
     // 32-bit offsets when every plane and velocity offset fits
     const bool idx32 = (long long)(L::Q + 3) * a.ncell < (1LL << 31);
     if (idx32)
-        return vec == 2 ? launch_dependent(k_step<L, STORE, UK, WALLS, 2, int>, grid, block, 0, st, a)
-                        : launch_dependent(k_step<L, STORE, UK, WALLS, 1, int>, grid, block, 0, st, a);
-    return vec == 2 ? launch_dependent(k_step<L, STORE, UK, WALLS, 2, long long>, grid, block, 0, st, a)
-                    : launch_dependent(k_step<L, STORE, UK, WALLS, 1, long long>, grid, block, 0, st, a);
+        return vec == 2 ? launch_dependent(k_step<L, STORE, UK, WALLS, 2, int, LD_ORDERED>, grid, block, 0, st, a)
+                        : launch_dependent(k_step<L, STORE, UK, WALLS, 1, int, LD_ORDERED>, grid, block, 0, st, a);
+    return vec == 2 ? launch_dependent(k_step<L, STORE, UK, WALLS, 2, long long, LD_ORDERED>, grid, block, 0, st, a)
+                    : launch_dependent(k_step<L, STORE, UK, WALLS, 1, long long, LD_ORDERED>, grid, block, 0, st, a);
 }
 
 template <class L, int STORE, int UK>

@@ -93,8 +93,9 @@ __device__ __forceinline__ void zw_issue_g(const uint16_t* __restrict__ g, uint1
 template <int STORE, int UK, bool WALLS, int TY>
 __global__ void __launch_bounds__(32 * TY, TY == 8 ? 3 : 6) k_step_zw_d3q15(const StepArgs args)
 {
-    StepArgs a = args;
-    step_after_dep(a);
+    constexpr int LD = UK == U_ROW && WALLS ? LD_PLAIN : LD_ORDERED;
+    StepArgsLD<LD> a = args;
+    step_after_dep<LD>(a);
     using Gm = ZwGeom<TY>;
     constexpr int PLANE = Gm::PLANE, CHUNKS = Gm::CHUNKS, GPOS = Gm::GPOS;
     using P = Pair<STORE>;
@@ -169,8 +170,8 @@ __global__ void __launch_bounds__(32 * TY, TY == 8 ? 3 : 6) k_step_zw_d3q15(cons
 
     const Coef& c = a.c;
     float s_now[3], s_prev[3];
-    sched_row_at(a.sched, a.srow_now, 3, s_now);
-    sched_row_at(a.sched, a.srow_prev, 3, s_prev);
+    sched_row_at<LD>(a.sched, a.srow_now, 3, s_now);
+    sched_row_at<LD>(a.sched, a.srow_prev, 3, s_prev);
     const float w0 = c.w0 * SC, wa = c.wa * SC, wd = c.wd * SC;   // exact (power of two)
     const float ka = c.ka * SC, kd = c.kd * SC;
     float kas[3], kds[3];   // decode slopes with the schedule factor of u(k - 1)
@@ -179,8 +180,8 @@ __global__ void __launch_bounds__(32 * TY, TY == 8 ? 3 : 6) k_step_zw_d3q15(cons
         kas[d] = __fmul_rn(ka, s_prev[d]);
         kds[d] = __fmul_rn(kd, s_prev[d]);
     }
-    const T2* __restrict__ src = static_cast<const T2*>(a.src);
-    T2* __restrict__ dst = static_cast<T2*>(a.dst);
+    const T2* src = static_cast<const T2*>(a.src);
+    T2* dst = static_cast<T2*>(a.dst);
     const int yr3[3] = {y + 1 == ny ? 0 : y + 1, y, y == 0 ? ny - 1 : y - 1};   // row y - e_y by e_y + 1
     const int own = (1 + ly) * ZW_W + 4 + 2 * lane;   // the pair's staged position in a plane slot
     // the pair's offsets in the staged block of a population: 32-bit words at
@@ -230,9 +231,9 @@ __global__ void __launch_bounds__(32 * TY, TY == 8 ? 3 : 6) k_step_zw_d3q15(cons
                 }
             } else if (UK == U_ROW && wc != 0) {
                 const int yr = yr3[ey + 1];
-                const float ux = __fmul_rn(__ldg(a.ua + yr), s_prev[0]);
-                const float uy = __fmul_rn(__ldg(a.ua + ny + yr), s_prev[1]);
-                const float uz = __fmul_rn(__ldg(a.ua + 2 * ny + yr), s_prev[2]);
+                const float ux = __fmul_rn(ld_vel<LD>(a.ua + yr), s_prev[0]);
+                const float uy = __fmul_rn(ld_vel<LD>(a.ua + ny + yr), s_prev[1]);
+                const float uz = __fmul_rn(ld_vel<LD>(a.ua + 2 * ny + yr), s_prev[2]);
                 e = sp2(fmaf(wc == 1 ? ka : kd, e_dot<L>(i, ux, uy, uz), wc == 1 ? wa : wd));
             }
             f[i] = fma2(ps, e, P::to_f_raw(QuadH<STORE>::as_t2(hw)));
@@ -244,7 +245,7 @@ __global__ void __launch_bounds__(32 * TY, TY == 8 ? 3 : 6) k_step_zw_d3q15(cons
             for (int d = 0; d < 3; ++d) ao[d] = *reinterpret_cast<const float2*>(S[1] + (1 + d) * PLANE);
         } else if (UK == U_ROW) {
 #pragma unroll
-            for (int d = 0; d < 3; ++d) ao[d] = sp2(__ldg(a.ua + d * ny + y));
+            for (int d = 0; d < 3; ++d) ao[d] = sp2(ld_vel<LD>(a.ua + d * ny + y));
         }
         const float2 po = *reinterpret_cast<const float2*>(S[1]);
 
@@ -272,7 +273,7 @@ __global__ void __launch_bounds__(32 * TY, TY == 8 ? 3 : 6) k_step_zw_d3q15(cons
                     for (int i = 0; i < 15; ++i)
                         if (L::ey(i) == inward) {
                             const int o = opposite<L>(i);
-                            const float2 g = P::to_f_raw(ldg_pair(src + o * NP + cellp));
+                            const float2 g = P::to_f_raw(ld_pair<LD>(src + o * NP + cellp));
                             f[i] = fma2(po, feq_unit_pair15(w0, wa, wd, ka, kd, o, up[0], up[1], up[2]), g);
                         }
                 } else {   // Dirichlet

@@ -1,0 +1,49 @@
+"""The forms in which the one-step kernels read their source (ordered, plain and read-only loads; overlapping and
+ordinary launches): the same bits whichever a size, a storage form or a launch shape leads to."""
+import numpy as np
+import pytest
+import torch
+
+from paper_1404_2363_gb300.solver import Solver
+
+pytestmark = pytest.mark.gpu
+
+D2 = [[0.03, 0.005], [0.005, 0.04]]
+D3 = [[0.03, 0.005, -0.004], [0.005, 0.025, 0.003], [-0.004, 0.003, 0.035]]
+
+
+def run(n, storage, u, bc, bc_x, launch, chunks, wait=False):
+    lattice = 15 if len(n) == 3 else 9
+    g = torch.Generator(device="cuda").manual_seed(11)
+    s = Solver(lattice=lattice, nx=n[0], ny=n[1], nz=n[2] if lattice == 15 else 1, storage=storage, bc=bc, bc_x=bc_x,
+               phi_w=(0.4, 0.2))
+    s.set_D(np.array(D3 if lattice == 15 else D2))
+    if launch is not None:
+        s.set_launch(*launch)
+    sched = torch.rand((5, s.dim), device="cuda", generator=g)
+    shape = (s.dim,) + s.shape if u == "field" else (s.dim, n[1])
+    if u != "none":
+        s.set_velocity(0.04 * torch.rand(shape, device="cuda", generator=g) - 0.02, sched, kind=u)
+    s.set_phi(torch.rand(s.shape, device="cuda", generator=g))
+    for k in chunks:
+        s.step(k)
+        if wait:
+            torch.cuda.synchronize()
+    state = s.get_state()[0].cpu().numpy()
+    s.close()
+    return state
+
+
+@pytest.mark.parametrize("n,u,bc_x,launch", [
+    ((64, 24, 20), "field", ("bounceback", "noflux"), (256, 1)), ((97, 60), "field", ("noflux", "bounceback"), (256, 1)),
+    ((64, 24, 20), "none", ("bounceback", "noflux"), (256, 1)), ((64, 24, 20), "row", ("periodic", "periodic"), (128, 9)),
+    ((64, 24, 20), "row", ("periodic", "periodic"), (256, 9)), ((64, 24, 20), "field", ("periodic", "periodic"), (32, 5))])
+@pytest.mark.parametrize("storage", ["f32", "f16", "bf16"])
+def test_overlapping_launches_equal_separate_ones(storage, n, u, bc_x, launch):
+    """Many launches in a row on a grid small enough for several to be resident at once, against the same with the
+    stream drained after each."""
+    if storage == "f32":
+        launch = (launch[0], 1)
+    a, b = (run(n, storage, u, ("noflux", "bounceback"), bc_x, launch, [1] * 300, wait) for wait in (True, False))
+    assert np.array_equal(a, b)
+    assert np.array_equal(a, run(n, storage, u, ("noflux", "bounceback"), bc_x, launch, [300]))

@@ -65,3 +65,12 @@ def test_recompute_leaves_the_reverse_steps_room():
     s.set_launch(256, 1)
     assert default < 1.08 * backward_us(s)
     s.close()
+
+
+def test_kernel_of_x_walls():
+    """D2Q9 BF16 between x and y walls, one step a launch, against the kernel for y walls alone: the source of every
+    population is checked against every face (1.65 times as long; it was 2.0)."""
+    walled, plain = solver((2048, 2048), "bf16", "noflux", "bounceback"), solver((2048, 2048), "bf16", "noflux")
+    assert step_us(walled, (256, 1)) < 1.82 * step_us(plain, (256, 1))
+    walled.close()
+    plain.close()
