@@ -590,6 +590,8 @@ __global__ void __launch_bounds__(256) k_step(const StepArgs args)
 //     applied per axis; at an edge of two Neumann faces, reflected in both);
 //   - Dirichlet (y faces only) replaces every population entering from beyond
 //     the y wall, as in k_step.
+// Plain loads: in order (LD_ORDERED) they took 64 registers instead of 48 (D2Q9 2048^2
+// BF16 114 -> 90.5 us a step, D3Q15 160^3 BF16 318 -> 242).
 // ---------------------------------------------------------------------------
 template <class L>
 __device__ __forceinline__ int reflect_mask(int i, int mask)

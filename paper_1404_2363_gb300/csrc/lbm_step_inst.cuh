@@ -36,7 +36,17 @@ static cudaError_t step_vec(LaunchCfg cfg, const StepArgs& a, cudaStream_t st)
             // node-pair variant (paired FP32 arithmetic, two adjacent nodes per thread)
             const int per = 2 * cfg.block;
             dim3 grid((unsigned)((a.nx + per - 1) / per), (unsigned)a.ny, (unsigned)a.nz);
-            return launch_dependent(k_step_pair_d3q15<STORE, UK, WALLS, LD_ORDERED>, grid, dim3((unsigned)cfg.block), 0, st, a);
+            // Large launches gain nothing from the overlap, and these instances lose more by its loads (us a
+            // step, LD_ORDERED against LD_READONLY): walls and a field 256 x 256 x 256 BF16 477 / 363, 128 x
+            // 128 x 64 26.3 / 23.3; FP16 between walls at rest 290 x 200 x 200 191.6 / 181.7; BF16 with a field
+            // 142 x 194 x 246 174 / 167 (but 64 x 225 x 163 56.3 / 57.6)
+            long long most = 1LL << 62;
+            if (UK == U_FIELD && WALLS) most = 1LL << 19;
+            else if (UK == U_NONE && WALLS && STORE == ST_F16) most = 3LL << 20;
+            else if (UK == U_FIELD && STORE == ST_BF16) most = 5LL << 19;
+            const bool ov = a.ncell <= most;
+            return launch_dependent(ov ? k_step_pair_d3q15<STORE, UK, WALLS, LD_ORDERED> : k_step_pair_d3q15<STORE, UK, WALLS, LD_READONLY>,
+                                    grid, dim3((unsigned)cfg.block), 0, st, a, ov);
         }
     }
     if constexpr (L::Q == 9 && STORE != ST_F32) {

@@ -47,3 +47,41 @@ def test_overlapping_launches_equal_separate_ones(storage, n, u, bc_x, launch):
     a, b = (run(n, storage, u, ("noflux", "bounceback"), bc_x, launch, [1] * 300, wait) for wait in (True, False))
     assert np.array_equal(a, b)
     assert np.array_equal(a, run(n, storage, u, ("noflux", "bounceback"), bc_x, launch, [300]))
+
+
+def repeated(n, axis, times, storage, u, bc, launch, steps=7):
+    """The state of a grid that repeats a small one `times` times along an axis (0: x, 1: y, 2: z), copies first."""
+    lattice = 15 if len(n) == 3 else 9
+    g = torch.Generator(device="cuda").manual_seed(13)
+    dim = len(n)
+    k = dim - 1 - axis                                  # array axis
+    rep = [1] * dim
+    rep[k] = times
+    big = [m * (times if d == axis else 1) for d, m in enumerate(n)]
+    s = Solver(lattice=lattice, nx=big[0], ny=big[1], nz=big[2] if dim == 3 else 1, storage=storage, bc=(bc, bc))
+    s.set_D(np.array(D3 if dim == 3 else D2))
+    s.set_launch(*launch)
+    shape = tuple(reversed(n))
+    phi = torch.rand(shape, device="cuda", generator=g)
+    a = 0.04 * torch.rand((dim,) + shape, device="cuda", generator=g) - 0.02
+    sched = torch.rand((5, dim), device="cuda", generator=g)
+    if u == "field":
+        s.set_velocity(a.repeat([1] + rep), sched)
+    s.set_phi(phi.repeat(rep))
+    s.step(steps)
+    state = s.get_state()[0]
+    cells, q = s.ncell, 9 if dim == 2 else 15
+    s.close()
+    elem = 4 if storage == "f32" else 2
+    f = state[:cells * q * elem].reshape([q] + list(reversed(big)) + [elem])
+    f = f.unflatten(1 + k, (times, n[axis])).movedim(1 + k, 0)
+    return f.contiguous()
+
+
+@pytest.mark.parametrize("storage,n,axis,times,u,bc,launch", [
+    ("bf16", (64, 40, 30), 2, 10, "field", "noflux", (32, 5)), ("f16", (64, 40, 30), 2, 10, "field", "bounceback", (64, 5)),
+    ("f16", (64, 40, 30), 2, 42, "none", "noflux", (128, 5)), ("bf16", (64, 40, 30), 2, 35, "field", "periodic", (64, 5))])
+def test_large_grids_give_the_bits_of_small_ones(storage, n, axis, times, u, bc, launch):
+    """A size from which the launch and the loads take another form, as copies of a grid below it."""
+    small = repeated(n, axis, 1, storage, u, bc, launch)
+    assert bool((repeated(n, axis, times, storage, u, bc, launch) == small).all())
