@@ -64,14 +64,20 @@ static cudaError_t step_vec(LaunchCfg cfg, const StepArgs& a, cudaStream_t st)
     const int vec = cfg.vec == 2 ? 2 : 1;
     const int per = cfg.block * vec;
     dim3 grid((unsigned)((a.nx + per - 1) / per), (unsigned)a.ny, (unsigned)a.nz);
-    dim3 block((unsigned)cfg.block);
     // 32-bit offsets when every plane and velocity offset fits
     const bool idx32 = (long long)(L::Q + 3) * a.ncell < (1LL << 31);
+    // between walls with a field, the D2Q9 16-bit forms lose more by the ordered loads than large launches gain
+    // (4096^2 FP16, LD_ORDERED against LD_READONLY: two nodes per thread 245 / 213 us a step, one 220 / 214)
+    constexpr bool slow = L::Q == 9 && STORE != ST_F32 && UK == U_FIELD && WALLS;
+    const bool ov = !(slow && idx32 && a.ncell >= (vec == 2 ? 1LL << 21 : 1LL << 23));
+    auto launch = [&](auto kernel) { return launch_dependent(kernel, grid, dim3((unsigned)cfg.block), 0, st, a, ov); };
+    if constexpr (slow) {
+        if (!ov)
+            return vec == 2 ? launch(k_step<L, STORE, UK, WALLS, 2, int, LD_READONLY>) : launch(k_step<L, STORE, UK, WALLS, 1, int, LD_READONLY>);
+    }
     if (idx32)
-        return vec == 2 ? launch_dependent(k_step<L, STORE, UK, WALLS, 2, int, LD_ORDERED>, grid, block, 0, st, a)
-                        : launch_dependent(k_step<L, STORE, UK, WALLS, 1, int, LD_ORDERED>, grid, block, 0, st, a);
-    return vec == 2 ? launch_dependent(k_step<L, STORE, UK, WALLS, 2, long long, LD_ORDERED>, grid, block, 0, st, a)
-                    : launch_dependent(k_step<L, STORE, UK, WALLS, 1, long long, LD_ORDERED>, grid, block, 0, st, a);
+        return vec == 2 ? launch(k_step<L, STORE, UK, WALLS, 2, int, LD_ORDERED>) : launch(k_step<L, STORE, UK, WALLS, 1, int, LD_ORDERED>);
+    return vec == 2 ? launch(k_step<L, STORE, UK, WALLS, 2, long long, LD_ORDERED>) : launch(k_step<L, STORE, UK, WALLS, 1, long long, LD_ORDERED>);
 }
 
 template <class L, int STORE, int UK>

@@ -84,3 +84,10 @@ def test_d3q15_pairs_between_walls():
         default = step_us(s)
         assert default < 1.12 * step_us(s, (128, 1))
         s.close()
+
+
+def test_two_nodes_per_thread_between_walls():
+    """D2Q9 FP16, field, walls: two nodes per thread against one (it was 1.12 times as long)."""
+    s = solver((4096, 4096), "f16", "noflux")
+    assert step_us(s, (128, 2), 8) < 1.06 * step_us(s, (256, 1), 8)
+    s.close()
