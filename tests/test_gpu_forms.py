@@ -81,7 +81,11 @@ def repeated(n, axis, times, storage, u, bc, launch, steps=7):
 @pytest.mark.parametrize("storage,n,axis,times,u,bc,launch", [
     ("bf16", (64, 40, 30), 2, 10, "field", "noflux", (32, 5)), ("f16", (64, 40, 30), 2, 10, "field", "bounceback", (64, 5)),
     ("f16", (64, 40, 30), 2, 42, "none", "noflux", (128, 5)), ("bf16", (64, 40, 30), 2, 35, "field", "periodic", (64, 5)),
-    ("f16", (64, 40), 0, 850, "field", "noflux", (128, 2)), ("bf16", (64, 40), 0, 3300, "field", "bounceback", (256, 1))])
+    ("f16", (64, 40), 0, 850, "field", "noflux", (128, 2)), ("bf16", (64, 40), 0, 3300, "field", "bounceback", (256, 1)),
+    # blocks so many that starting them overlapped would take longer than the nodes
+    ("f32", (40, 40), 1, 400, "field", "periodic", (64, 1)), ("f32", (40, 40, 20), 2, 30, "none", "periodic", (96, 1)),
+    ("f16", (40, 40, 20), 2, 30, "field", "noflux", (64, 1)), ("bf16", (40, 40), 1, 400, "none", "periodic", (64, 2)),
+    ("bf16", (40, 40, 20), 2, 30, "none", "noflux", (32, 5))])
 def test_large_grids_give_the_bits_of_small_ones(storage, n, axis, times, u, bc, launch):
     """A size from which the launch and the loads take another form, as copies of a grid below it."""
     small = repeated(n, axis, 1, storage, u, bc, launch)

@@ -50,11 +50,11 @@ def backward_us(s, steps=48, want_da=False):
 
 
 def test_reverse_step_of_multi_row_blocks():
-    """A reverse step reads twice what a forward step reads and writes as much or, with dL/da, 1.1 times; blocks of
-    several rows took 3.7 times a forward step, 2.6 with the row offsets out of the vector registers."""
+    """dL/da adds a read and a write of three planes to the fifty of a D3Q15 reverse step (1.0 times as long with the
+    row offsets out of the vector registers; the spills made it 1.28)."""
     s = solver((97, 80, 66), bc="periodic")
-    forward = step_us(s)
-    assert backward_us(s, want_da=True) < 3.1 * forward
+    plain = backward_us(s)
+    assert backward_us(s, want_da=True) < 1.15 * plain
     s.close()
 
 
@@ -90,4 +90,12 @@ def test_two_nodes_per_thread_between_walls():
     """D2Q9 FP16, field, walls: two nodes per thread against one (it was 1.12 times as long)."""
     s = solver((4096, 4096), "f16", "noflux")
     assert step_us(s, (128, 2), 8) < 1.06 * step_us(s, (256, 1), 8)
+    s.close()
+
+
+def test_small_blocks():
+    """64 threads a block against 256, one step a launch: the rate at which overlapping blocks start bounded the
+    first (1.5 times as long)."""
+    s = solver((4096, 4096), u="none")
+    assert step_us(s, (64, 1), 8) < 1.2 * step_us(s, (256, 1), 8)
     s.close()
