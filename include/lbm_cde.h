@@ -415,6 +415,11 @@ lbm_status lbm_cde_batch_autotune(lbm_cde_batch_t b, int64_t steps, int32_t* mod
 /* Selects an execution mode and tile height explicitly. */
 lbm_status lbm_cde_batch_config(lbm_cde_batch_t b, int32_t mode, int32_t tile_rows);
 
+/* Steps that one launch of the current configuration takes: 4 where PER_STEP groups eight
+ * steps into two launches, else 1 (a PERSISTENT launch takes a chunk, one step at a time),
+ * and the most ranges of rows that such a launch splits a channel into. */
+lbm_status lbm_cde_batch_launch_info(lbm_cde_batch_t b, int32_t* steps_out, int32_t* ranges_out);
+
 const char* lbm_cde_batch_last_error(lbm_cde_batch_t b);
 
 /* Allocation-free FP64 sum of phi over a raw state (no counterpart in the

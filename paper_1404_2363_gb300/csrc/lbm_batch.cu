@@ -23,7 +23,9 @@
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
+#include <functional>
 #include <new>
+#include <queue>
 #include <string>
 #include <vector>
 
@@ -957,9 +959,10 @@ struct lbm_cde_batch_s {
     lbm::StepStreams ss{};              // PER_STEP: moment stream, events, odd-step column sums
     lbm::BatchTask* tasks = nullptr;    // walk launches: the CTAs' tasks, group by group
     std::vector<int> ntasks;
+    int ranges = 1;                     // most row ranges of a channel in the walk launches
     int* cblk_inst = nullptr;           // instance of each 256-column block of the moment pass
     int ncblk = 0;
-    double* cpart = nullptr;            // [2][ncblk][3] moment partials (PER_STEP uses the first)
+    double* cpart = nullptr;            // [2][ncblk][3] moment partials, by step parity (PER_STEP: by launch parity)
     cudaStream_t st = nullptr;
     std::string err;
 };
@@ -1137,40 +1140,47 @@ static lbm_status rebuild_tiles(lbm_cde_batch_t b)
     return LBM_OK;
 }
 
-// Tasks and buffers of the walk launches, where they pay: the time of four steps
-// by the walk's rule (walk_ranges: a row takes 0.45 + 0.47 k us at k warps per
-// scheduler, at most three) against that of four one-step launches (4.1 us each,
-// or 72 bytes a node at 6 TB/s).
-static lbm_status setup_walk(lbm_cde_batch_t b)
+// Whether the walk launches pay, and their tasks. Times in us, measured on GB300 over 1 to 64 channels of 300 to 8192
+// columns and 17 to 128 rows (0.25M to 26M cells):
+//   four one-step launches: each 6 us and 6.3 us a million nodes of its 32 x 16 tiles while both states stay in L2,
+//     beyond that 72 bytes a node at 5.2 TB/s if that is more;
+//   the walk: 6 us and 1.1 + 0.4 k us a row at k warps per scheduler on average, the rows of the longest SM slot when the
+//     CTAs, three per SM, are taken in order (the step kernel's walk takes 0.45 + 0.47 k, without column sums).
+// The walk has to be 5 % faster: near the break-even the rule is off by up to a tenth (us a step by the walk and by single
+// steps: 1 x 8192 x 64 10.5 / 7.8, 2 x 8192 x 64 13.2 / 12.0, 8 x 8192 x 17 13.5 / 18.7, 64 x 8192 x 40 141 / 297).
+static bool walk_tasks(lbm_cde_batch_t b, std::vector<lbm::BatchTask>& all)
 {
-    if (9LL * b->ncat >= (1LL << 31)) return LBM_OK;
+    b->ntasks.clear();
+    b->ranges = 1;
+    if (9LL * b->ncat >= (1LL << 31)) return false;
     int dev = 0, sms = 0;
     if (cudaGetDevice(&dev) != cudaSuccess ||
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1) {
         cudaGetLastError();
-        return LBM_OK;
+        return false;
     }
     const int T = lbm::BWALK_T;
     auto strips = [&](const lbm::InstDev& I) { return (I.nx + lbm::WALK_COLS - 1) / lbm::WALK_COLS; };
     long long warps = 0;
-    for (const lbm::InstDev& I : b->inst) warps += strips(I);
+    double padded = 0;
+    for (const lbm::InstDev& I : b->inst) {
+        warps += strips(I);
+        padded += 512.0 * I.tx * I.tyc;
+    }
     // ranges of a channel: enough for two warps per scheduler, at least 16 rows each
     const long long want = 8LL * sms;
     const int split = (int)std::max<long long>(1, (want + warps - 1) / warps);
-    std::vector<lbm::BatchTask> all;
-    double rows = 0, longest = 0, used = 0;
-    b->ntasks.clear();
+    double walked = 0;   // rows of all warps
     for (int g0 = 0; g0 < b->n; g0 += lbm::CELL_INST) {
         std::vector<lbm::BatchTask> t;
         for (int j = 0; j < std::min(lbm::CELL_INST, b->n - g0); ++j) {
             const lbm::InstDev& I = b->inst[g0 + j];
             const int blocks = (I.ny + 15) / 16, nr = std::min(split, blocks);
+            b->ranges = std::max(b->ranges, nr);
             for (int q = 0; q < nr; ++q) {
                 const int ya = 16 * (blocks * q / nr), yb = std::min(16 * (blocks * (q + 1) / nr), I.ny);
                 for (int s0 = 0; s0 < strips(I); s0 += lbm::WALK_WARPS) t.push_back({j, s0, ya, yb});
-                rows += (double)strips(I) * (yb - ya + 2 * T);
-                longest = std::max(longest, (double)(yb - ya + 2 * T));
-                used += strips(I);
+                walked += (double)strips(I) * (yb - ya + 2 * T);
             }
         }
         std::stable_sort(t.begin(), t.end(), [](const lbm::BatchTask& x, const lbm::BatchTask& y) {
@@ -1179,13 +1189,50 @@ static lbm_status setup_walk(lbm_cde_batch_t b)
         b->ntasks.push_back((int)t.size());
         all.insert(all.end(), t.begin(), t.end());
     }
-    const double slots = 4.0 * sms, k = std::min(3.0, std::max(1.0, used / slots));
-    const double walk = std::max(rows / (slots * k), longest) * (0.45 + 0.47 * k) + 1.5;
-    const double single = T * std::max(4.1, b->ncat * 72 / 6.0e6);
-    if (walk >= single) {
+    std::priority_queue<int, std::vector<int>, std::greater<int>> slots;   // rows walked by each
+    for (int q = 0; q < 3 * sms; ++q) slots.push(0);
+    int rows = 0;
+    for (const lbm::BatchTask& t : all) {
+        const int r = slots.top() + t.yb - t.ya + 2 * T;
+        slots.pop();
+        slots.push(r);
+        rows = std::max(rows, r);
+    }
+    const double k = std::max(1.0, walked / (4.0 * sms * rows));
+    const double walk = 6.0 + rows * (1.1 + 0.4 * k);
+    const double hbm = 72.0 * b->ncat > 1.1e8 ? b->ncat * 72 / 5.2e6 : 0;   // both states past L2
+    const double single = T * std::max(6.0 + 6.3e-6 * padded, hbm);
+    return walk < 0.95 * single;
+}
+
+static void release_walk(lbm_cde_batch_t b)
+{
+    bfree(b, b->tasks);
+    b->tasks = nullptr;
+    for (int p = 0; p < 2; ++p) {
+        bfree(b, b->ss.wstrip[p]);
+        bfree(b, b->ss.wcpart[p]);
+        b->ss.wstrip[p] = nullptr;
+        b->ss.wcpart[p] = nullptr;
+    }
+    b->ss.tasks = nullptr;
+    b->ntasks.clear();
+}
+
+// Buffers of the walk launches, where they pay; without memory to spare, one step a launch.
+static lbm_status setup_walk(lbm_cde_batch_t b)
+{
+    std::vector<lbm::BatchTask> all;
+    try {
+        if (!walk_tasks(b, all)) {
+            b->ntasks.clear();
+            return LBM_OK;
+        }
+    } catch (const std::bad_alloc&) {
         b->ntasks.clear();
         return LBM_OK;
     }
+    const int T = lbm::BWALK_T;
     b->tasks = static_cast<lbm::BatchTask*>(balloc(b, sizeof(lbm::BatchTask) * all.size()));
     bool ok = b->tasks != nullptr;
     for (int p = 0; p < 2 && ok; ++p) {
@@ -1193,16 +1240,8 @@ static lbm_status setup_walk(lbm_cde_batch_t b)
         b->ss.wcpart[p] = static_cast<double*>(balloc(b, sizeof(double) * 3 * (size_t)b->ncblk * T));
         ok = b->ss.wstrip[p] && b->ss.wcpart[p];
     }
-    if (!ok) {   // no memory to spare: one step a launch
-        bfree(b, b->tasks);
-        b->tasks = nullptr;
-        for (int p = 0; p < 2; ++p) {
-            bfree(b, b->ss.wstrip[p]);
-            bfree(b, b->ss.wcpart[p]);
-            b->ss.wstrip[p] = nullptr;
-            b->ss.wcpart[p] = nullptr;
-        }
-        b->ntasks.clear();
+    if (!ok) {
+        release_walk(b);
         return LBM_OK;
     }
     if (cudaFuncSetAttribute(lbm::k_batch_walk, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -1588,6 +1627,15 @@ lbm_status lbm_cde_batch_config(lbm_cde_batch_t b, int32_t mode, int32_t tile_ro
         b->rows = tile_rows;
         return rebuild_tiles(b);
     }
+    return LBM_OK;
+}
+
+lbm_status lbm_cde_batch_launch_info(lbm_cde_batch_t b, int32_t* steps_out, int32_t* ranges_out)
+{
+    if (!b || !steps_out || !ranges_out) return bfail(b, LBM_E_ARG, "NULL argument");
+    const bool walk = b->mode == LBM_BATCH_PER_STEP && b->ss.tasks != nullptr;
+    *steps_out = walk ? lbm::BWALK_T : 1;
+    *ranges_out = walk ? b->ranges : 1;
     return LBM_OK;
 }
 

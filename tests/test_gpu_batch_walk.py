@@ -1,0 +1,49 @@
+"""PER_STEP batches that take several steps per launch: when they do, and their bits over ranges of rows."""
+import numpy as np
+import pytest
+import torch
+
+from paper_1404_2363_gb300.batch import Batch, poiseuille_row
+
+pytestmark = pytest.mark.gpu
+
+WALLS = [("noflux", "noflux"), ("periodic", "periodic"), ("bounceback", "noflux"), ("noflux", "bounceback"),
+         ("bounceback", "bounceback")]
+
+
+def channels(n, nx, ny, walls=WALLS[:1], spread=0):
+    return [{"nx": nx + spread * i, "ny": ny + (3 * i) % (spread + 1), "bc": walls[i % len(walls)],
+             "D": [[0.03, 0.004], [0.004, 0.05]],
+             "u_row": poiseuille_row(ny + (3 * i) % (spread + 1), 0.08) if i % 4 else None, "x_ref0": float(nx // 5),
+             "x_ref_velocity": 0.05, "model": ("A", "B1", "B3")[i % 3]} for i in range(n)]
+
+
+# us a step by single steps / by the walk: 7.8 / 10.5, 9.5 / 10.5, 10.4 / 13.0, 12.0 / 13.2, 16.7 / 20.6; then 18.7 / 13.5,
+# 33.4 / 19.7, 31.2 / 22.8, 66 / 41
+@pytest.mark.parametrize("n,nx,ny,steps", [
+    (1, 8192, 64, 1), (4, 1100, 128, 1), (32, 300, 64, 1), (2, 8192, 64, 1), (64, 300, 64, 1), (2, 300, 17, 1),
+    (8, 8192, 17, 4), (8, 4097, 64, 4), (2, 8192, 128, 4), (64, 1100, 64, 4)])
+def test_walk_only_where_it_pays(n, nx, ny, steps):
+    b = Batch(channels(n, nx, ny), mode="per_step")
+    assert b.launch_info()[0] == steps
+    b.close()
+
+
+@pytest.mark.parametrize("n,nx,ny,ranges", [(6, 3999, 70, 3), (8, 4000, 101, 3), (4, 4001, 128, 5), (4, 8190, 97, 3)])
+def test_walk_over_row_ranges(n, nx, ny, ranges):
+    """Channels split into ranges of rows, on every wall pair, odd and even row lengths and heights off the 16-row
+    tiles, against the persistent cell tiles (one step at a time): fields and moments bit for bit."""
+    chs = channels(n, nx, ny, WALLS, spread=5)
+    g = np.random.default_rng(17)
+    phis = [(0.05 + g.random((c["ny"], c["nx"]))).astype(np.float32) for c in chs]
+    out = []
+    for mode in ("persistent", "per_step"):
+        b = Batch(chs, mode=mode, graph_steps=16)
+        if mode == "per_step":
+            assert b.launch_info()[0] == 4 and b.launch_info()[1] >= ranges
+        b.set_phi(phis)
+        m = b.run(21)
+        out.append((m, torch.cat([p.reshape(-1) for p in b.get_phi()])))
+        b.close()
+    assert np.array_equal(out[0][0], out[1][0])
+    assert torch.equal(out[0][1], out[1][1])
