@@ -374,7 +374,10 @@ typedef struct {
                                 PER_STEP taken by whole blocks, one grid barrier per step, the
                                 moment passes of steps k - 1 and k - 2 run ahead of the cells of
                                 step k inside the launch; 1 .. 1024: tiles of 32 columns x
-                                tile_rows rows, one warp each, one node per thread */
+                                tile_rows rows, one warp each, one node per thread. PER_STEP: 1
+                                one step per launch, 4 four steps per launch where they can run
+                                (9 cells < 2^31 and memory for their sums), others the one that
+                                is expected to be faster */
     int32_t graph_steps;     /* steps per captured CUDA graph (ring of moments), 1 .. 4096 */
     int64_t barrier_timeout_cycles; /* clock64 cycles a CTA waits at a grid barrier (and, on
                                 cell tiles, at its shared-memory barriers) before the launch
@@ -408,8 +411,9 @@ lbm_status lbm_cde_batch_get_phi(lbm_cde_batch_t b, float* phi_dev);
  * then invalid until the next set_phi). */
 lbm_status lbm_cde_batch_run(lbm_cde_batch_t b, int64_t nsteps, double* moments_host);
 
-/* Times PERSISTENT on cell tiles (0) and at tile heights 8, 16, 32 rows, and PER_STEP on `steps` steps,
- * keeps the fastest (restoring the state and step count) and reports it. */
+/* Times PERSISTENT on cell tiles (0) and at tile heights 8, 16, 32 rows, and PER_STEP with one and with four steps
+ * per launch on `steps` steps (rounded up to a multiple of 8), keeps the fastest (restoring the state and step count)
+ * and reports it (PER_STEP: tile 0 where tile_rows = 0 chooses the same, else 1 or 4). */
 lbm_status lbm_cde_batch_autotune(lbm_cde_batch_t b, int64_t steps, int32_t* mode_out, int32_t* tile_out);
 
 /* Selects an execution mode and tile height explicitly. */

@@ -944,6 +944,7 @@ struct lbm_cde_batch_s {
     long long t = 0;
     bool ready = false;
     int mode = LBM_BATCH_PERSISTENT;
+    bool mode_set = false;         // set_mode has run
     int rows = 0;                  // rows per warp tile (PERSISTENT); 0: the cell tiles
     int chunk = 64;                // steps per graph replay
     cudaGraphExec_t graph = nullptr;   // one chunk of steps, built lazily for (mode, rows)
@@ -959,6 +960,7 @@ struct lbm_cde_batch_s {
     lbm::StepStreams ss{};              // PER_STEP: moment stream, events, odd-step column sums
     lbm::BatchTask* tasks = nullptr;    // walk launches: the CTAs' tasks, group by group
     std::vector<int> ntasks;
+    int launch_steps = 0;               // PER_STEP: 0 by the rule of walk_tasks, 1 single steps, BWALK_T the walk
     int ranges = 1;                     // most row ranges of a channel in the walk launches
     int* cblk_inst = nullptr;           // instance of each 256-column block of the moment pass
     int ncblk = 0;
@@ -1148,6 +1150,7 @@ static lbm_status rebuild_tiles(lbm_cde_batch_t b)
 //     CTAs, three per SM, are taken in order (the step kernel's walk takes 0.45 + 0.47 k, without column sums).
 // The walk has to be 5 % faster: near the break-even the rule is off by up to a tenth (us a step by the walk and by single
 // steps: 1 x 8192 x 64 10.5 / 7.8, 2 x 8192 x 64 13.2 / 12.0, 8 x 8192 x 17 13.5 / 18.7, 64 x 8192 x 40 141 / 297).
+// b->launch_steps = BWALK_T: the walk wherever it can run.
 static bool walk_tasks(lbm_cde_batch_t b, std::vector<lbm::BatchTask>& all)
 {
     b->ntasks.clear();
@@ -1202,7 +1205,7 @@ static bool walk_tasks(lbm_cde_batch_t b, std::vector<lbm::BatchTask>& all)
     const double walk = 6.0 + rows * (1.1 + 0.4 * k);
     const double hbm = 72.0 * b->ncat > 1.1e8 ? b->ncat * 72 / 5.2e6 : 0;   // both states past L2
     const double single = T * std::max(6.0 + 6.3e-6 * padded, hbm);
-    return walk < 0.95 * single;
+    return b->launch_steps == lbm::BWALK_T || walk < 0.95 * single;
 }
 
 static void release_walk(lbm_cde_batch_t b)
@@ -1256,6 +1259,26 @@ static lbm_status setup_walk(lbm_cde_batch_t b)
     return LBM_OK;
 }
 
+// Execution mode and, for PER_STEP, the steps of a launch (its tile_rows 1 and BWALK_T; others: by the rule). The walk's
+// buffers are held only while PER_STEP uses them.
+static lbm_status set_mode(lbm_cde_batch_t b, int mode, int tile_rows)
+{
+    const int steps = mode == LBM_BATCH_PER_STEP && (tile_rows == 1 || tile_rows == lbm::BWALK_T) ? tile_rows : 0;
+    if (b->mode == mode && b->launch_steps == steps && b->mode_set) return LBM_OK;
+    drop_graph(b);
+    release_walk(b);
+    b->mode = mode;
+    b->launch_steps = steps;
+    b->mode_set = true;
+    if (mode != LBM_BATCH_PER_STEP || steps == 1) return LBM_OK;
+    const lbm_status s = setup_walk(b);
+    if (s != LBM_OK) {
+        release_walk(b);
+        return bfail(b, s, "walk setup failed");
+    }
+    return LBM_OK;
+}
+
 extern "C" {
 
 lbm_status lbm_cde_batch_opts_init(lbm_cde_batch_opts* o)
@@ -1288,7 +1311,6 @@ lbm_status lbm_cde_batch_create(const lbm_cde_channel_desc* descs, int32_t n, co
     b->st = static_cast<cudaStream_t>(o.stream);
     b->rows = o.tile_rows == 0 && n > lbm::CELL_INST ? 16 : o.tile_rows;   // cell tiles: <= CELL_INST instances
     b->chunk = o.graph_steps;
-    b->mode = o.mode == LBM_BATCH_PER_STEP ? LBM_BATCH_PER_STEP : LBM_BATCH_PERSISTENT;
     b->inst.resize(n);
     long long off = 0;
     for (int i = 0; i < n; ++i) {
@@ -1433,10 +1455,12 @@ lbm_status lbm_cde_batch_create(const lbm_cde_channel_desc* descs, int32_t n, co
         cudaMemcpyAsync(b->tile_inst, ti.data(), sizeof(int) * ti.size(), cudaMemcpyHostToDevice, b->st);
         cudaStreamSynchronize(b->st);
     }
-    if (lbm_status ws = setup_walk(b); ws != LBM_OK) {
+    if (lbm_status ws = set_mode(b, o.mode == LBM_BATCH_PER_STEP ? LBM_BATCH_PER_STEP : LBM_BATCH_PERSISTENT, o.tile_rows);
+        ws != LBM_OK) {
         lbm_cde_batch_destroy(b);
         return bfail(nullptr, ws, "walk setup failed");
     }
+    if (b->launch_steps != 0) b->rows = n > lbm::CELL_INST ? 16 : 0;   // tile_rows is no tile height
     cudaMemsetAsync(b->sync, 0, 64, b->st);
     lbm_status s = rebuild_tiles(b);
     if (s != LBM_OK) {
@@ -1462,11 +1486,7 @@ lbm_status lbm_cde_batch_destroy(lbm_cde_batch_t b)
     bfree(b, b->moments);
     bfree(b, b->strip);
     bfree(b, b->ss.strip2);
-    bfree(b, b->tasks);
-    for (int p = 0; p < 2; ++p) {
-        bfree(b, b->ss.wstrip[p]);
-        bfree(b, b->ss.wcpart[p]);
-    }
+    release_walk(b);
     if (b->ss.st2) {
         cudaStreamSynchronize(b->ss.st2);
         cudaStreamDestroy(b->ss.st2);
@@ -1553,9 +1573,9 @@ lbm_status lbm_cde_batch_run(lbm_cde_batch_t b, int64_t nsteps, double* moments_
     return LBM_OK;
 }
 
-// Times candidate execution modes and tile widths on `steps` steps each, then
-// keeps the fastest (the state is restored afterwards). Writes the choice to
-// *mode_out / *tile_out (may be NULL).
+// Times candidate execution modes, tile heights and launches on `steps` steps each (rounded
+// up to a multiple of 8), then keeps the fastest (the state is restored afterwards).
+// Writes the choice to *mode_out / *tile_out (may be NULL).
 lbm_status lbm_cde_batch_autotune(lbm_cde_batch_t b, int64_t steps, int32_t* mode_out, int32_t* tile_out)
 {
     if (!b || steps < 1) return bfail(b, LBM_E_ARG, "bad argument");
@@ -1566,45 +1586,50 @@ lbm_status lbm_cde_batch_autotune(lbm_cde_batch_t b, int64_t steps, int32_t* mod
     if (!save) return bfail(b, LBM_E_OOM, "autotune buffer allocation failed");
     BCK(b, cudaMemcpyAsync(save, b->buf[b->t & 1], sb, cudaMemcpyDeviceToDevice, b->st));
     const long long t_save = b->t;
-    const int modes[2] = {LBM_BATCH_PERSISTENT, LBM_BATCH_PER_STEP};
-    const int tws[4] = {0, 8, 16, 32};
+    // PERSISTENT on cell tiles (not above CELL_INST instances) and at heights of 8, 16 and 32 rows, PER_STEP by single
+    // steps and by the walk, where it can run (groups of eight steps)
+    struct Cand { int mode, tile; };
+    std::vector<Cand> cand;
+    if (b->n <= lbm::CELL_INST) cand.push_back({LBM_BATCH_PERSISTENT, 0});
+    for (int tile : {8, 16, 32}) cand.push_back({LBM_BATCH_PERSISTENT, tile});
+    cand.push_back({LBM_BATCH_PER_STEP, 1});
+    cand.push_back({LBM_BATCH_PER_STEP, lbm::BWALK_T});
+    const int64_t timed = steps + (8 - steps % 8) % 8;
     float best = 1e30f;
-    int best_mode = b->mode, best_tw = b->rows;
+    Cand pick = cand.back();
     cudaEvent_t e0, e1;
     cudaEventCreate(&e0);
     cudaEventCreate(&e1);
-    for (int m : modes)
-        for (int tw : tws) {
-            if (m == LBM_BATCH_PER_STEP && tw != tws[0]) continue;   // fixed 32 x 16 cell tiles
-            if (m == LBM_BATCH_PERSISTENT && tw == 0 && b->n > lbm::CELL_INST) continue;
-            b->mode = m;
-            if (b->rows != tw) {
-                b->rows = tw;
-                lbm_status s = rebuild_tiles(b);
-                if (s != LBM_OK) return s;
-            }
-            lbm_status s = lbm_cde_batch_run(b, std::min<int64_t>(steps, b->chunk), nullptr);  // warm
-            if (s != LBM_OK) return s;
-            cudaEventRecord(e0, b->st);
-            s = lbm_cde_batch_run(b, steps, nullptr);
-            cudaEventRecord(e1, b->st);
-            cudaEventSynchronize(e1);
-            if (s != LBM_OK) return s;
-            float ms = 0.f;
-            cudaEventElapsedTime(&ms, e0, e1);
-            if (ms < best) {
-                best = ms;
-                best_mode = m;
-                best_tw = tw;
-            }
+    lbm_status s = LBM_OK;
+    for (const Cand& c : cand) {
+        s = lbm_cde_batch_config(b, c.mode, c.tile);
+        if (s == LBM_OK && c.mode == LBM_BATCH_PER_STEP && c.tile != 1 && b->ss.tasks == nullptr) continue;   // no walk
+        if (s == LBM_OK) s = lbm_cde_batch_run(b, std::min<int64_t>(timed, b->chunk), nullptr);   // warm
+        cudaEventRecord(e0, b->st);
+        if (s == LBM_OK) s = lbm_cde_batch_run(b, timed, nullptr);
+        cudaEventRecord(e1, b->st);
+        cudaEventSynchronize(e1);
+        if (s != LBM_OK) break;
+        float ms = 0.f;
+        cudaEventElapsedTime(&ms, e0, e1);
+        if (ms < best) {
+            best = ms;
+            pick = c;
         }
+    }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
-    b->mode = best_mode;
-    if (b->rows != best_tw) {
-        b->rows = best_tw;
-        lbm_status s = rebuild_tiles(b);
-        if (s != LBM_OK) return s;
+    if (s == LBM_OK) s = lbm_cde_batch_config(b, pick.mode, pick.tile);
+    if (s == LBM_OK && pick.mode == LBM_BATCH_PER_STEP) {
+        // 0 where the rule agrees
+        const bool walk = b->ss.tasks != nullptr;
+        s = lbm_cde_batch_config(b, pick.mode, 0);
+        if (s == LBM_OK && (b->ss.tasks != nullptr) != walk) s = lbm_cde_batch_config(b, pick.mode, pick.tile);
+        else pick.tile = 0;
+    }
+    if (s != LBM_OK) {
+        bfree(b, save);
+        return s;
     }
     // restore: state into buf[t_save & 1], step index on the device
     BCK(b, cudaMemcpyAsync(b->buf[t_save & 1], save, sb, cudaMemcpyDeviceToDevice, b->st));
@@ -1612,8 +1637,8 @@ lbm_status lbm_cde_batch_autotune(lbm_cde_batch_t b, int64_t steps, int32_t* mod
     BCK(b, cudaStreamSynchronize(b->st));
     bfree(b, save);
     b->t = t_save;
-    if (mode_out) *mode_out = best_mode;
-    if (tile_out) *tile_out = best_tw;
+    if (mode_out) *mode_out = pick.mode;
+    if (tile_out) *tile_out = pick.tile;
     return LBM_OK;
 }
 
@@ -1621,7 +1646,9 @@ lbm_status lbm_cde_batch_config(lbm_cde_batch_t b, int32_t mode, int32_t tile_ro
 {
     if (!b || (mode != LBM_BATCH_PERSISTENT && mode != LBM_BATCH_PER_STEP) || tile_rows < 0 || tile_rows > 1024)
         return bfail(b, LBM_E_ARG, "bad mode or tile height");
-    b->mode = mode;
+    const lbm_status ms = set_mode(b, mode, tile_rows);
+    if (ms != LBM_OK) return ms;
+    if (b->launch_steps != 0) tile_rows = 0;                       // steps of a launch, no tiles
     if (tile_rows == 0 && b->n > lbm::CELL_INST) tile_rows = 16;   // cell tiles: <= CELL_INST instances
     if (b->rows != tile_rows) {
         b->rows = tile_rows;

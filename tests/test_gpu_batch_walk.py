@@ -47,3 +47,52 @@ def test_walk_over_row_ranges(n, nx, ny, ranges):
         b.close()
     assert np.array_equal(out[0][0], out[1][0])
     assert torch.equal(out[0][1], out[1][1])
+
+
+def test_launch_steps_can_be_chosen_and_keep_the_bits():
+    """PER_STEP with tile_rows 1 and 4 on both sides of the rule, in one handle; the autotuner's choice is one of them."""
+    for n, nx, ny, rule in ((4, 1100, 100, 1), (8, 4097, 64, 4)):
+        chs = channels(n, nx, ny, WALLS, spread=3)
+        g = np.random.default_rng(23)
+        phis = [(0.05 + g.random((c["ny"], c["nx"]))).astype(np.float32) for c in chs]
+        b = Batch(chs, mode="per_step", graph_steps=16)
+        out = {}
+        for tile, steps in ((0, rule), (1, 1), (4, 4), (0, rule)):
+            b.config("per_step", tile)
+            assert b.launch_info()[0] == steps
+            b.set_phi(phis)
+            m = b.run(21)
+            out[tile] = (m, torch.cat([p.reshape(-1) for p in b.get_phi()]))
+            assert np.array_equal(m, out[0][0]) and torch.equal(out[tile][1], out[0][1])
+        b.set_phi(phis)
+        mode, tile = b.autotune(16)
+        assert b.launch_info()[0] == ((rule if tile == 0 else tile) if mode == "per_step" else 1)
+        m = b.run(21)
+        assert mode != "per_step" or np.array_equal(m, out[0][0])
+        b.close()
+
+
+def test_autotune_measures_single_steps_against_the_walk():
+    """With the walk as the chosen shape of a batch where it is the slower one, tuning ends with single steps again."""
+    b = Batch(channels(1, 8192, 64), mode="per_step", tile_rows=4)
+    assert b.launch_info()[0] == 4
+    b.set_phi([torch.rand((64, 8192))])
+    mode, tile = b.autotune(64)
+    assert mode != "per_step" or (tile == 0 and b.launch_info()[0] == 1)
+    b.close()
+
+
+def test_persistent_batches_hold_no_sums_of_the_walk():
+    """The walk's column sums (2 x 4 strips of 128 bytes a cell tile) are allocated while PER_STEP uses them."""
+    chs = channels(16, 4096, 64)
+    torch.cuda.synchronize()
+    base = torch.cuda.memory_allocated()
+    b = Batch(chs, mode="persistent")
+    held = torch.cuda.memory_allocated() - base
+    b.config("per_step", 0)
+    assert b.launch_info()[0] == 4
+    sums = 2 * 4 * 128 * 16 * 128 * 4        # 16 channels of 128 x 4 cell tiles
+    assert torch.cuda.memory_allocated() - base >= held + sums
+    b.config("persistent", 0)
+    assert torch.cuda.memory_allocated() - base == held
+    b.close()
