@@ -224,10 +224,11 @@ lbm_status lbm_cde_set_wait_limit(lbm_cde_t h, int64_t cycles);
  * (planes < 0). */
 lbm_status lbm_cde_set_zwalk(lbm_cde_t h, int32_t planes);
 
-/* Autotuner: times every launch shape (block 64/128/256 x vec 1/2, the node-quad
+/* Autotuner: times every launch shape (the one in use, the one a handle starts with,
+ * block 64/128/256 x vec 1/2, the fused steps and the node-quad
  * kernel for D2Q9, the node-pair and TMA-staged kernels for D2Q9 16-bit
- * storage, the node-pair kernel at 64 .. 256 threads and the z-walk kernel
- * for D3Q15 16-bit storage) over `steps` steps from the
+ * storage, the node-pair kernel at 32 .. 256 threads and the z-walk kernel
+ * for D3Q15 16-bit storage) over `steps` steps (with the fused steps at least 8) from the
  * current state, keeps the fastest, and restores the state and step count.
  * With LBMCDE_TUNE_CACHE set, the choice is read from / appended to that text
  * file (lines "key block vec"; the key holds lattice, storage, grid, velocity

@@ -41,6 +41,7 @@ struct lbm_cde_s {
     long long t = 0;
     bool ready = false;
     LaunchCfg cfg{256, 1};
+    LaunchCfg cfg0{256, 1};                // the shape the handle started with
     int pair_block = 0;                    // default shape with a velocity field: node pairs with this block (0: none)
     cudaStream_t st = nullptr;
     std::string err;
@@ -465,6 +466,7 @@ lbm_status lbm_cde_create(const lbm_cde_desc* desc, lbm_cde_t* out)
             if (4 * columns(2 * block) <= 5 * columns(h->cfg.block)) h->pair_block = block;
         }
     }
+    h->cfg0 = h->cfg;
     *out = h;
     return LBM_OK;
 }
@@ -664,7 +666,8 @@ static std::string tune_key(lbm_cde_t h)
     for (char& ch : gpu)
         if (ch == ' ') ch = '_';
     char buf[256];
-    snprintf(buf, sizeof(buf), "q%d_s%d_%lldx%lldx%lld_u%d_bc%d%d%d%d%d%d_%s", h->q, h->d.storage,
+    // the leading number counts the sets of candidates: a choice among fewer is made again
+    snprintf(buf, sizeof(buf), "2_q%d_s%d_%lldx%lldx%lld_u%d_bc%d%d%d%d%d%d_%s", h->q, h->d.storage,
              (long long)h->d.nx, (long long)h->d.ny, (long long)h->d.nz, h->ukind, h->d.bc_lo_y, h->d.bc_hi_y,
              h->d.bc_lo_x, h->d.bc_hi_x, h->d.bc_lo_z, h->d.bc_hi_z, gpu.c_str());
     return buf;
@@ -726,18 +729,27 @@ lbm_status lbm_cde_autotune(lbm_cde_t h, int64_t steps, int32_t* block_out, int3
     cudaEvent_t e0, e1;
     cudaEventCreate(&e0);
     cudaEventCreate(&e1);
-    // candidates: generic kernel (1 or 2 nodes per thread) at 64/128/256 threads;
-    // for D2Q9 16-bit storage also the node-pair kernel at 64/128/256 threads; for
-    // D3Q15 16-bit storage the node-pair kernel at 64 .. 256 threads; the node-quad
-    // kernel (D2Q9), the TMA-staged D2Q9 kernel (16-bit storage) and the D3Q15
-    // z-walk kernel where they apply
+    // candidates: the shape in use and the one a handle starts with; generic kernel
+    // (1 or 2 nodes per thread) at 64/128/256 threads; for D2Q9 16-bit storage also
+    // the node-pair kernel at 64/128/256 threads; for D3Q15 16-bit storage the
+    // node-pair kernel at 32 .. 256 threads; the node-quad kernel (D2Q9), the
+    // TMA-staged D2Q9 kernel (16-bit storage), the D3Q15 z-walk kernel and the fused
+    // D2Q9 steps where they apply
     std::vector<LaunchCfg> cand;
+    auto shown = [&](LaunchCfg c) {   // a starting shape as the block and vec that choose the same
+        if (c.vec != 0) return c;
+        if (fused_ok(h)) return LaunchCfg{128, 10};
+        if (h->pair_block && ukind_internal(h->ukind) == lbm::U_FIELD) return LaunchCfg{h->pair_block, 5};
+        return LaunchCfg{c.block, 1};
+    };
+    cand.push_back(shown(keep));
+    cand.push_back(shown(h->cfg0));
     for (int vec = 1; vec <= 2; ++vec)
         for (int b : {64, 128, 256}) cand.push_back(LaunchCfg{b, vec});
     if (h->q == 9 && h->neq && h->d.nx % 2 == 0 && 12LL * h->ncell < (1LL << 31))
         for (int b : {64, 128, 256}) cand.push_back(LaunchCfg{b, 5});
     if (h->q == 15 && h->neq && h->d.nx % 2 == 0 && 18LL * h->ncell < (1LL << 31))
-        for (int b : {64, 96, 128, 192, 256}) cand.push_back(LaunchCfg{b, 5});
+        for (int b : {32, 64, 96, 128, 192, 256}) cand.push_back(LaunchCfg{b, 5});
     if (h->q == 9 && h->d.nx % 4 == 0 && 12LL * h->ncell < (1LL << 31))
         for (int b : {64, 128, 256}) cand.push_back(LaunchCfg{b, 6});
     if (h->q == 15 && h->neq && h->d.nx % 64 == 0 && 18LL * h->ncell < (1LL << 31))
@@ -749,12 +761,14 @@ lbm_status lbm_cde_autotune(lbm_cde_t h, int64_t steps, int32_t* block_out, int3
         cand.push_back(LaunchCfg{128, 8});
     }
     if (fused_ok(h)) cand.push_back(LaunchCfg{128, 10});   // fused steps
+    // at least the steps of one launch of the fused kernels
+    const int64_t timed = fused_ok(h) ? std::max<int64_t>(steps, lbm::TILE_T) : steps;
     for (size_t ci = 0; ci < cand.size() && s == LBM_OK; ++ci) {
         h->cfg = cand[ci];
         s = lbm_cde_set_state(h, save, t0);
-        if (s == LBM_OK) s = lbm_cde_step(h, 2);     // warm
+        if (s == LBM_OK) s = lbm_cde_step(h, h->cfg.vec >= 10 ? timed : 2);   // warm: the kernels that are timed
         cudaEventRecord(e0, h->st);
-        if (s == LBM_OK) s = lbm_cde_step(h, steps);
+        if (s == LBM_OK) s = lbm_cde_step(h, timed);
         cudaEventRecord(e1, h->st);
         cudaEventSynchronize(e1);
         float ms = 0.f;

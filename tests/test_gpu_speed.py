@@ -99,3 +99,29 @@ def test_small_blocks():
     s = solver((4096, 4096), u="none")
     assert step_us(s, (64, 1), 8) < 1.2 * step_us(s, (256, 1), 8)
     s.close()
+
+
+@pytest.mark.parametrize("n,storage", [((80, 160, 160), "f32"), ((64, 225, 163), "bf16"), ((200, 150, 150), "f32")])
+def test_tuned_shape_keeps_up_with_the_default(n, storage):
+    """The starting shape is a candidate: blocks of 96 and 224 threads, pairs of 32 (tuning ended 9 to 20 % above)."""
+    s = solver(n, storage)
+    default = step_us(s)
+    shape = s.autotune(12)
+    assert step_us(s) < 1.05 * default, shape
+    s.close()
+
+
+def test_tuning_on_one_step_times_the_fused_kernels(tmp_path, monkeypatch):
+    """One step would run every shape one step a launch; and a choice that an older set of candidates left in the
+    cache is made again."""
+    path = tmp_path / "tune.txt"
+    monkeypatch.setenv("LBMCDE_TUNE_CACHE", str(path))
+    s = solver((1024, 1024))
+    assert s.autotune(1) == (128, 10)
+    key = path.read_text().split()[0]
+    assert key.startswith("2_")
+    path.write_text(f"{key[2:]} 64 1\n")
+    assert s.autotune(12) == (128, 10)
+    path.write_text(f"{key} 64 1\n")
+    assert s.autotune(12) == (64, 1)
+    s.close()
