@@ -297,10 +297,11 @@ static lbm::FusePlan fuse_plan(lbm_cde_t h, int64_t left)
 {
     const int v = h->cfg.vec;
     if (!fused_ok(h) || left < 2 || !(v == 0 || (v >= 10 && v <= 12))) return {1, 0};
+    const bool walls = h->d.bc_lo_y != LBM_BC_PERIODIC || h->d.bc_lo_x != LBM_BC_PERIODIC;
     const int kinds = v == 11 ? lbm::FUSE_WALK : (v == 12 ? lbm::FUSE_TILE : lbm::FUSE_ANY);
-    if (left < lbm::TILE_T) return lbm::plan_fused(h->d.storage, (int)h->d.nx, (int)h->d.ny, h->sms, left, kinds);
+    if (left < lbm::TILE_T) return lbm::plan_fused(h->d.storage, (int)h->d.nx, (int)h->d.ny, walls, h->sms, left, kinds);
     if (h->plan_kinds != kinds) {   // the plan of a long run is kept
-        h->plan = lbm::plan_fused(h->d.storage, (int)h->d.nx, (int)h->d.ny, h->sms, lbm::TILE_T, kinds);
+        h->plan = lbm::plan_fused(h->d.storage, (int)h->d.nx, (int)h->d.ny, walls, h->sms, lbm::TILE_T, kinds);
         h->plan_kinds = kinds;
     }
     return h->plan;

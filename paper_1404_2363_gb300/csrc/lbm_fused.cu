@@ -1,4 +1,6 @@
 // Several D2Q9 steps per launch: the choice between the kernels and their launch.
+#include <algorithm>
+
 #include "lbm_tile_d2q9.cuh"
 
 namespace lbm {
@@ -29,14 +31,20 @@ int walk_ranges(int strips, int ny, int T, int sms, int warps, double* cost)
 //   one step: 4.1 us from launch to launch, 80 bytes a node at 6.8 TB/s when that is more;
 //   walk:     walk_ranges; rows whose length allows no 16-byte copies take 1.1 (FP32) or
 //             1.5 (16-bit) times as long;
-//   tile:     2.3 us + per wave of one tile per SM: 1 us to load, 0.2 us a step and
+//   tile:     2.3 us + per wave of one tile per SM: 1 us to load and 0.03 us a row beyond 32
+//             (300 x 4000: 13.8 us a step in three waves of two steps, walk 11.9), 0.2 us a step and
 //             0.05 us a row and step (128^2: 6.2 us for 6 steps on 16-row tiles; 256^2: 8.7 on
 //             24 rows; 512^2: 15.7 on 48 rows); on grids whose two states do not fit in L2 a tile's
 //             loads and stores come from HBM, which nothing overlaps with one CTA per SM (FP16 2913 x 2240:
 //             77 us a step; without this term the plan took it for 47 and the walk, 52, for slower).
+// Walls: the walk's T = 4 instances hold 8 warps per SM instead of 12. The strips with an x wall (1.6 times a row's
+// time, with ranges of their own) and the tiles with one (1.5 times) change neither kernel's place: their figures are
+// left out. Over 18 grids (333 x 33 to 4096 x 4096), FP32 and BF16, with a field, a row profile and five wall pairs, the
+// choice takes 1.011 times the fastest of the three in the mean, at most 1.25 times (1280 x 900 BF16 periodic: walk 13.0,
+// tile 10.4).
 // The tile kernel wins below about 1M nodes (us a step: 512^2 2.5, walk 8.0, one step 6.2; 896^2 6.4, 9.2,
 // 10.3), the walk above (1024^2: 7.7 against 8.5 and 12.3; 2048^2: 21, 43, 52; 4096^2: 72, 166, 192).
-FusePlan plan_fused(int store, int nx, int ny, int sms, long long left, int kinds)
+FusePlan plan_fused(int store, int nx, int ny, bool walls, int sms, long long left, int kinds)
 {
     const double n = (double)nx * ny;
     const double single = n * 80 / 6.8e6;
@@ -47,7 +55,7 @@ FusePlan plan_fused(int store, int nx, int ny, int sms, long long left, int kind
     FusePlan p{1, 0};
     for (int T = 2; T <= 4 && T <= left && (kinds & FUSE_WALK); T += 2) {
         double c;
-        walk_ranges((nx + WALK_COLS - 1) / WALK_COLS, ny, T, sms, 12, &c);
+        walk_ranges((nx + WALK_COLS - 1) / WALK_COLS, ny, T, sms, T == 4 ? 4 * walk_minb(4, walls) : 12, &c);
         if (c * slow / T < best) {
             best = c * slow / T;
             p = {T, 0};
@@ -57,7 +65,8 @@ FusePlan plan_fused(int store, int nx, int ny, int sms, long long left, int kind
         for (int rows = 2 * T + 2; rows <= TILE_ROWS; rows += 2) {
             const int h = rows - 2 * T;
             const long long tiles = (long long)((nx + 63 - 2 * T) / (64 - 2 * T)) * ((ny + h - 1) / h);
-            const double c = 2.3 + (double)((tiles + sms - 1) / sms) * (1.0 + fetch * rows + 0.2 * T + 0.05 * T * (h + T - 1));
+            const double load = 1.0 + (fetch > 0 ? fetch * rows : 0.03 * std::max(0, rows - 32));
+            const double c = 2.3 + (double)((tiles + sms - 1) / sms) * (load + 0.2 * T + 0.05 * T * (h + T - 1));
             if (c / T < best) {
                 best = c / T;
                 p = {T, rows};

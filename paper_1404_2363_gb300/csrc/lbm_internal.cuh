@@ -143,7 +143,7 @@ int walk_ranges(int strips, int ny, int T, int sms, int warps, double* cost);
 // kernel (T = 1), of the walk kernel (rows = 0) or of the tile kernel (rows of a tile).
 struct FusePlan { int T, rows; };
 enum { FUSE_WALK = 1, FUSE_TILE = 2, FUSE_ANY = 3 };   // kernels the plan may take (one: at least two steps by it)
-FusePlan plan_fused(int store, int nx, int ny, int sms, long long left, int kinds = FUSE_ANY);
+FusePlan plan_fused(int store, int nx, int ny, bool walls, int sms, long long left, int kinds = FUSE_ANY);
 
 // One reverse-time step (lbm_adjoint.cu).
 struct AdjArgs {

@@ -125,3 +125,11 @@ def test_tuning_on_one_step_times_the_fused_kernels(tmp_path, monkeypatch):
     path.write_text(f"{key} 64 1\n")
     assert s.autotune(12) == (64, 1)
     s.close()
+
+
+def test_plan_of_a_tall_grid_between_walls():
+    """300 x 4000 between walls took the tile kernel in three waves of two steps (1.42 times the walk's time)."""
+    s = solver((300, 4000), bc="noflux")
+    default = step_us(s)
+    assert default < 1.12 * min(step_us(s, (128, 11)), step_us(s, (128, 12)))
+    s.close()
