@@ -7,6 +7,7 @@
 #include <cuda_fp16.h>
 #include <cuda_bf16.h>
 #include <stdint.h>
+#include <atomic>
 #include <type_traits>
 
 namespace lbm {
@@ -333,6 +334,33 @@ cudaError_t launch_dependent(void (*kernel)(A), dim3 grid, dim3 block, int smem,
     cfg.attrs = at;
     cfg.numAttrs = overlap ? 1 : 0;
     return cudaLaunchKernelEx(&cfg, kernel, args);
+}
+
+// How a kernel with dynamic shared memory fits the current device: its multiprocessors and the CTAs each holds. Asked
+// once per kernel and device (`known`, one per instantiation) and published as one word, so that threads with handles
+// of their own see all of it or ask themselves; an error is returned and nothing remembered.
+struct KernelFit { int sms, per_sm; };
+template <class K>
+cudaError_t kernel_fit(std::atomic<unsigned> (&known)[64], K* kernel, int threads, int smem, KernelFit& fit)
+{
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    unsigned w = dev < 64 ? known[dev].load(std::memory_order_acquire) : 0;
+    if (w == 0) {
+        int sms = 0, per_sm = 0;
+        e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+        if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, threads, smem);
+        if (e != cudaSuccess) {
+            cudaGetLastError();   // returned, not left for the next call
+            return e;
+        }
+        w = (unsigned)(sms > 0 ? sms : 1) << 16 | (unsigned)(per_sm > 0 ? per_sm : 1);
+        if (dev < 64) known[dev].store(w, std::memory_order_release);
+    }
+    fit = {(int)(w >> 16), (int)(w & 0xffffu)};
+    return cudaSuccess;
 }
 
 // Kernel launchers (lbm_kernels.cu). Each returns the cudaError_t of the launch.

@@ -281,15 +281,10 @@ __global__ void __launch_bounds__(TILE_THREADS, 1) k_tile_d2q9(const __grid_cons
 template <int STORE, bool WALLS>
 cudaError_t tile_d2q9(const TileArgs& p, cudaStream_t st)
 {
-    static int done[64] = {0};   // per instantiation and device
-    int dev = 0;
-    cudaGetDevice(&dev);
-    if (!done[dev & 63]) {
-        cudaError_t e = cudaFuncSetAttribute(k_tile_d2q9<STORE, WALLS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             tile_smem(TILE_ROWS));
-        if (e != cudaSuccess) return e;
-        done[dev & 63] = 1;
-    }
+    static std::atomic<unsigned> known[64];
+    KernelFit fit;
+    const cudaError_t fe = kernel_fit(known, k_tile_d2q9<STORE, WALLS>, TILE_THREADS, tile_smem(TILE_ROWS), fit);
+    if (fe != cudaSuccess) return fe;
     const dim3 grid((unsigned)((p.a.nx + 64 - 2 * p.T - 1) / (64 - 2 * p.T)),
                     (unsigned)((p.a.ny + p.rows - 2 * p.T - 1) / (p.rows - 2 * p.T)));
     return launch_dependent(k_tile_d2q9<STORE, WALLS>, grid, dim3(TILE_THREADS), tile_smem(p.rows), st, p);

@@ -519,24 +519,16 @@ template <int STORE, bool FIELD, bool WALLS, int T, bool SAVE>
 cudaError_t walk_d2q9(WalkArgs& p, cudaStream_t st)
 {
     constexpr int smem = WALK_WARPS * WalkSlot<STORE>::warp(FIELD);
-    static int per_sm[64] = {0}, sms[64] = {0};   // per instantiation and device
-    int dev = 0;
-    cudaGetDevice(&dev);
-    dev &= 63;
-    if (per_sm[dev] == 0) {
-        int n = 0, k = 0;
-        cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
-        cudaFuncSetAttribute(k_walk_d2q9<STORE, FIELD, WALLS, T, SAVE>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&k, k_walk_d2q9<STORE, FIELD, WALLS, T, SAVE>, 32 * WALK_WARPS, smem);
-        sms[dev] = n > 0 ? n : 1;
-        per_sm[dev] = k > 0 ? k : 1;
-    }
+    static std::atomic<unsigned> known[64];
+    KernelFit fit;
+    const cudaError_t fe = kernel_fit(known, k_walk_d2q9<STORE, FIELD, WALLS, T, SAVE>, 32 * WALK_WARPS, smem, fit);
+    if (fe != cudaSuccess) return fe;
     p.strips = (p.a.nx + WALK_COLS - 1) / WALK_COLS;
-    p.ranges = walk_ranges(p.strips, p.a.ny, T, sms[dev], per_sm[dev] * WALK_WARPS, nullptr);
+    p.ranges = walk_ranges(p.strips, p.a.ny, T, fit.sms, fit.per_sm * WALK_WARPS, nullptr);
     int warps = p.strips * p.ranges;
     if (WALLS && p.a.bcx_lo != BC_PERIODIC && p.strips >= 3) {
         // a row of a strip with an x wall takes about 1.6 times as long (selects in every level)
-        const int most = sms[dev] * per_sm[dev] * WALK_WARPS;
+        const int most = fit.sms * fit.per_sm * WALK_WARPS;
         auto total = [&] { return (p.strips - 2) * p.ranges + 2 * p.eranges; };
         p.eranges = (8 * p.ranges + 4) / 5;
         while (p.ranges > 1 && total() > most) p.eranges = (8 * --p.ranges + 4) / 5;
