@@ -14,7 +14,8 @@ namespace lbm {
 // but blocks that execute the wait and the trigger start at no more than one a ns: with
 // 64 threads a block, D2Q9 4096^2 FP32 takes 263 us a step instead of 175 (262144
 // blocks). So not where starting the blocks takes longer than the nodes, at the rates the
-// kernels reach, and the 2 us. Rates measured with 64 (pairs: 32) threads a block, in TB/s:
+// kernels reach, and the 2 us (3 with D3Q15's longer chain: 41 x 62 x 192 FP32 15.4 us a
+// step overlapping, 16.6 not). Rates measured with 64 (pairs: 32) threads a block, in TB/s:
 // FP32 6; 16 bit: D2Q9 5, D3Q15 with one node per thread 3.7 (at rest, periodic; else 2.6),
 // pairs 5, less by what lanes past the row's end take (FP16 and periodic: 3.2, where the
 // ordered loads are also the faster ones, 290 x 200 x 200 at rest 219 us against 237).
@@ -29,7 +30,7 @@ inline bool overlap_pays(dim3 grid, int block, const StepArgs& a, int q, int sto
         else if (pairs) rate = store == ST_F16 && !walls ? 3.2e6 : 5.0e6 * a.nx / (2.0 * block * grid.x);
         else rate = uk == U_NONE && !walls ? 3.7e6 : 2.6e6;
     }
-    return blocks * 1e-3 + 1.0 <= (double)a.ncell * bytes / rate + 2.0;
+    return blocks * 1e-3 + 1.0 <= (double)a.ncell * bytes / rate + (q == 9 ? 2.0 : 3.0);
 }
 
 template <class L, int STORE, int UK, bool WALLS>
