@@ -376,9 +376,11 @@ typedef struct {
                                 moment passes of steps k - 1 and k - 2 run ahead of the cells of
                                 step k inside the launch; 1 .. 1024: tiles of 32 columns x
                                 tile_rows rows, one warp each, one node per thread. PER_STEP: 1
-                                one step per launch, 4 four steps per launch where they can run
-                                (9 cells < 2^31 and memory for their sums), others the one that
-                                is expected to be faster */
+                                one step per launch in whole chunks of graph_steps, 4 four steps
+                                per launch where they can run (9 cells < 2^31 and memory for
+                                their sums), others the one that is expected to be faster;
+                                shorter chunks, which no graph replays, choose by what their
+                                launches cost the host as well (unless 4) */
     int32_t graph_steps;     /* steps per captured CUDA graph (ring of moments), 1 .. 4096 */
     int64_t barrier_timeout_cycles; /* clock64 cycles a CTA waits at a grid barrier (and, on
                                 cell tiles, at its shared-memory barriers) before the launch
@@ -420,7 +422,7 @@ lbm_status lbm_cde_batch_autotune(lbm_cde_batch_t b, int64_t steps, int32_t* mod
 /* Selects an execution mode and tile height explicitly. */
 lbm_status lbm_cde_batch_config(lbm_cde_batch_t b, int32_t mode, int32_t tile_rows);
 
-/* Steps that one launch of the current configuration takes: 4 where PER_STEP groups eight
+/* Steps that one launch of a whole chunk takes in the current configuration: 4 where PER_STEP groups eight
  * steps into two launches, else 1 (a PERSISTENT launch takes a chunk, one step at a time),
  * and the most ranges of rows that such a launch splits a channel into. */
 lbm_status lbm_cde_batch_launch_info(lbm_cde_batch_t b, int32_t* steps_out, int32_t* ranges_out);

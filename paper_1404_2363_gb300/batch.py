@@ -117,7 +117,7 @@ class Batch:
         return {1: "persistent", 2: "per_step"}[mode.value], tile.value
 
     def launch_info(self):
-        """(steps a launch takes in the current configuration, most row ranges of a channel in it)."""
+        """(steps a launch of a whole chunk takes in the current configuration, most row ranges of a channel in it)."""
         steps, ranges = ctypes.c_int32(), ctypes.c_int32()
         self._ck(self.L.lbm_cde_batch_launch_info(self.h, ctypes.byref(steps), ctypes.byref(ranges)),
                  "lbm_cde_batch_launch_info")

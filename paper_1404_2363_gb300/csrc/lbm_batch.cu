@@ -960,7 +960,9 @@ struct lbm_cde_batch_s {
     lbm::StepStreams ss{};              // PER_STEP: moment stream, events, odd-step column sums
     lbm::BatchTask* tasks = nullptr;    // walk launches: the CTAs' tasks, group by group
     std::vector<int> ntasks;
-    int launch_steps = 0;               // PER_STEP: 0 by the rule of walk_tasks, 1 single steps, BWALK_T the walk
+    int launch_steps = 0;               // PER_STEP: 0 by the rule of walk_tasks, 1 single steps in whole chunks, BWALK_T
+                                        // the walk
+    bool walk_whole = false, walk_direct = false;   // the walk in whole chunks (graph replays), in others
     int ranges = 1;                     // most row ranges of a channel in the walk launches
     int* cblk_inst = nullptr;           // instance of each 256-column block of the moment pass
     int ncblk = 0;
@@ -1063,9 +1065,11 @@ static lbm::BatchArgs batch_args(lbm_cde_batch_t b, int nsteps)
 
 static cudaError_t launch_batch(lbm_cde_batch_t b, const lbm::BatchArgs& a)
 {
+    lbm::StepStreams ss = b->ss;
+    if (!(a.nsteps == b->chunk && b->use_graph ? b->walk_whole : b->walk_direct)) ss.tasks = nullptr;
     return lbm::launch_mode(b->mode, b->rows, a, b->cinst.data(), b->tile_inst, b->n, b->kdev, b->cells, b->cell_tiles,
                             b->nctiles,
-                            b->strip, b->cblk_inst, b->ncblk, b->cpart, b->st, b->ss);
+                            b->strip, b->cblk_inst, b->ncblk, b->cpart, b->st, ss);
 }
 
 static void drop_graph(lbm_cde_batch_t b)
@@ -1148,19 +1152,23 @@ static lbm_status rebuild_tiles(lbm_cde_batch_t b)
 //     beyond that 72 bytes a node at 5.2 TB/s if that is more;
 //   the walk: 6 us and 1.1 + 0.4 k us a row at k warps per scheduler on average, the rows of the longest SM slot when the
 //     CTAs, three per SM, are taken in order (the step kernel's walk takes 0.45 + 0.47 k, without column sums).
+// A chunk that is not a whole one is launched directly, and there a single step costs the host at least 19 us (three
+// launches and the events between), a walk launch of four steps hardly more: 7 channels of 1436 .. 2872 x 60 .. 65, 50
+// steps in chunks of 64, 26.3 us a step by single steps, 18.2 by the walk. That counts from 2^18 nodes on.
 // The walk has to be 5 % faster: near the break-even the rule is off by up to a tenth (us a step by the walk and by single
 // steps: 1 x 8192 x 64 10.5 / 7.8, 2 x 8192 x 64 13.2 / 12.0, 8 x 8192 x 17 13.5 / 18.7, 64 x 8192 x 40 141 / 297).
-// b->launch_steps = BWALK_T: the walk wherever it can run.
-static bool walk_tasks(lbm_cde_batch_t b, std::vector<lbm::BatchTask>& all)
+// *whole, *direct: the choice for whole chunks and for others.
+static void walk_tasks(lbm_cde_batch_t b, std::vector<lbm::BatchTask>& all, bool* whole, bool* direct)
 {
+    *whole = *direct = false;
     b->ntasks.clear();
     b->ranges = 1;
-    if (9LL * b->ncat >= (1LL << 31)) return false;
+    if (9LL * b->ncat >= (1LL << 31)) return;
     int dev = 0, sms = 0;
     if (cudaGetDevice(&dev) != cudaSuccess ||
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1) {
         cudaGetLastError();
-        return false;
+        return;
     }
     const int T = lbm::BWALK_T;
     auto strips = [&](const lbm::InstDev& I) { return (I.nx + lbm::WALK_COLS - 1) / lbm::WALK_COLS; };
@@ -1204,8 +1212,10 @@ static bool walk_tasks(lbm_cde_batch_t b, std::vector<lbm::BatchTask>& all)
     const double k = std::max(1.0, walked / (4.0 * sms * rows));
     const double walk = 6.0 + rows * (1.1 + 0.4 * k);
     const double hbm = 72.0 * b->ncat > 1.1e8 ? b->ncat * 72 / 5.2e6 : 0;   // both states past L2
-    const double single = T * std::max(6.0 + 6.3e-6 * padded, hbm);
-    return b->launch_steps == lbm::BWALK_T || walk < 0.95 * single;
+    const double single = std::max(6.0 + 6.3e-6 * padded, hbm);
+    const bool all_walk = b->launch_steps == lbm::BWALK_T;
+    *whole = all_walk || (b->launch_steps != 1 && walk < 0.95 * T * single);
+    *direct = all_walk || (b->ncat >= (1LL << 18) && walk < 0.95 * T * std::max(single, 19.0));
 }
 
 static void release_walk(lbm_cde_batch_t b)
@@ -1219,6 +1229,7 @@ static void release_walk(lbm_cde_batch_t b)
         b->ss.wcpart[p] = nullptr;
     }
     b->ss.tasks = nullptr;
+    b->walk_whole = b->walk_direct = false;
     b->ntasks.clear();
 }
 
@@ -1227,11 +1238,11 @@ static lbm_status setup_walk(lbm_cde_batch_t b)
 {
     std::vector<lbm::BatchTask> all;
     try {
-        if (!walk_tasks(b, all)) {
-            b->ntasks.clear();
-            return LBM_OK;
-        }
+        walk_tasks(b, all, &b->walk_whole, &b->walk_direct);
     } catch (const std::bad_alloc&) {
+        b->walk_whole = b->walk_direct = false;
+    }
+    if (!b->walk_whole && !b->walk_direct) {
         b->ntasks.clear();
         return LBM_OK;
     }
@@ -1254,7 +1265,7 @@ static lbm_status setup_walk(lbm_cde_batch_t b)
             cudaSuccess ||
         cudaStreamSynchronize(b->st) != cudaSuccess)
         return LBM_E_CUDA;
-    b->ss.tasks = b->tasks;
+    b->ss.tasks = b->tasks;   // one by one where the launch's choice is single steps (launch_batch)
     b->ss.ntasks = b->ntasks.data();
     return LBM_OK;
 }
@@ -1270,7 +1281,7 @@ static lbm_status set_mode(lbm_cde_batch_t b, int mode, int tile_rows)
     b->mode = mode;
     b->launch_steps = steps;
     b->mode_set = true;
-    if (mode != LBM_BATCH_PER_STEP || steps == 1) return LBM_OK;
+    if (mode != LBM_BATCH_PER_STEP) return LBM_OK;
     const lbm_status s = setup_walk(b);
     if (s != LBM_OK) {
         release_walk(b);
@@ -1603,7 +1614,7 @@ lbm_status lbm_cde_batch_autotune(lbm_cde_batch_t b, int64_t steps, int32_t* mod
     lbm_status s = LBM_OK;
     for (const Cand& c : cand) {
         s = lbm_cde_batch_config(b, c.mode, c.tile);
-        if (s == LBM_OK && c.mode == LBM_BATCH_PER_STEP && c.tile != 1 && b->ss.tasks == nullptr) continue;   // no walk
+        if (s == LBM_OK && c.mode == LBM_BATCH_PER_STEP && c.tile != 1 && !b->walk_whole) continue;   // cannot run
         if (s == LBM_OK) s = lbm_cde_batch_run(b, std::min<int64_t>(timed, b->chunk), nullptr);   // warm
         cudaEventRecord(e0, b->st);
         if (s == LBM_OK) s = lbm_cde_batch_run(b, timed, nullptr);
@@ -1622,9 +1633,9 @@ lbm_status lbm_cde_batch_autotune(lbm_cde_batch_t b, int64_t steps, int32_t* mod
     if (s == LBM_OK) s = lbm_cde_batch_config(b, pick.mode, pick.tile);
     if (s == LBM_OK && pick.mode == LBM_BATCH_PER_STEP) {
         // 0 where the rule agrees
-        const bool walk = b->ss.tasks != nullptr;
+        const bool walk = b->walk_whole;
         s = lbm_cde_batch_config(b, pick.mode, 0);
-        if (s == LBM_OK && (b->ss.tasks != nullptr) != walk) s = lbm_cde_batch_config(b, pick.mode, pick.tile);
+        if (s == LBM_OK && b->walk_whole != walk) s = lbm_cde_batch_config(b, pick.mode, pick.tile);
         else pick.tile = 0;
     }
     if (s != LBM_OK) {
@@ -1660,7 +1671,7 @@ lbm_status lbm_cde_batch_config(lbm_cde_batch_t b, int32_t mode, int32_t tile_ro
 lbm_status lbm_cde_batch_launch_info(lbm_cde_batch_t b, int32_t* steps_out, int32_t* ranges_out)
 {
     if (!b || !steps_out || !ranges_out) return bfail(b, LBM_E_ARG, "NULL argument");
-    const bool walk = b->mode == LBM_BATCH_PER_STEP && b->ss.tasks != nullptr;
+    const bool walk = b->mode == LBM_BATCH_PER_STEP && b->walk_whole;
     *steps_out = walk ? lbm::BWALK_T : 1;
     *ranges_out = walk ? b->ranges : 1;
     return LBM_OK;

@@ -96,3 +96,33 @@ def test_persistent_batches_hold_no_sums_of_the_walk():
     b.config("persistent", 0)
     assert torch.cuda.memory_allocated() - base == held
     b.close()
+
+
+def compare(chs, steps, graph_steps, tile, seed=31):
+    g = np.random.default_rng(seed)
+    phis = [(0.05 + g.random((c["ny"], c["nx"]))).astype(np.float32) for c in chs]
+    out = []
+    for mode, t in (("persistent", 0), ("per_step", tile)):
+        b = Batch(chs, mode=mode, tile_rows=t, graph_steps=graph_steps)
+        b.set_phi(phis)
+        m = b.run(steps)
+        out.append((m, torch.cat([p.reshape(-1) for p in b.get_phi()])))
+        b.close()
+    assert np.array_equal(out[0][0], out[1][0])
+    assert torch.equal(out[0][1], out[1][1])
+
+
+def test_walk_of_narrow_and_low_channels():
+    """The walk on channels narrower than a strip and lower than its halo (chosen: no rule takes it there)."""
+    g = np.random.default_rng(37)
+    chs = []
+    for i in range(40):
+        nx, ny = int(g.integers(2, 70)), int(g.integers(3, 40))
+        chs += channels(1, nx, ny, [WALLS[i % 5]])
+        chs[-1]["x_ref0"] = float(nx // 3)
+    compare(chs, 29, 16, 4)
+
+
+def test_chunks_that_no_graph_replays():
+    """50 steps in chunks of 64: single steps in whole chunks, the walk in this one."""
+    compare(channels(7, 1436, 62, WALLS, spread=3), 50, 64, 0)

@@ -133,3 +133,19 @@ def test_plan_of_a_tall_grid_between_walls():
     default = step_us(s)
     assert default < 1.12 * min(step_us(s, (128, 11)), step_us(s, (128, 12)))
     s.close()
+
+
+def test_direct_chunks_of_a_batch():
+    """56 steps in chunks of 64 are launched directly, where four steps a launch save the host's time (single steps took
+    1.45 times as long), though whole chunks are as fast by single steps."""
+    from paper_1404_2363_gb300.batch import Batch, poiseuille_row
+
+    chs = [{"nx": 2000, "ny": 62, "D": np.eye(2) * 0.03, "u_row": poiseuille_row(62, 0.05), "x_ref0": 400.0} for _ in range(7)]
+    b = Batch(chs, mode="per_step", graph_steps=64)
+    b.set_phi([torch.rand((62, 2000)) for _ in chs])
+    us = []
+    for tile in (0, 4):
+        b.config("per_step", tile)
+        us.append(best_us(lambda: b.run(56)))
+    b.close()
+    assert us[0] < 1.15 * us[1]
