@@ -37,7 +37,7 @@ int walk_ranges(int strips, int ny, int T, int sms, int warps, double* cost)
 //             24 rows; 512^2: 15.7 on 48 rows); on grids whose two states do not fit in L2 a tile's
 //             loads and stores come from HBM, which nothing overlaps with one CTA per SM (FP16 2913 x 2240:
 //             77 us a step; without this term the plan took it for 47 and the walk, 52, for slower).
-// Walls: the walk's T = 4 instances hold 8 warps per SM instead of 12. The strips with an x wall (1.6 times a row's
+// Walls: the walk's T = 4 instances hold 8 warps per SM instead of 12 (and T = 2 is charged alike). The strips with an x wall (1.6 times a row's
 // time, with ranges of their own) and the tiles with one (1.5 times) change neither kernel's place: their figures are
 // left out. Over 18 grids (333 x 33 to 4096 x 4096), FP32 and BF16, with a field, a row profile and five wall pairs, the
 // choice takes 1.011 times the fastest of the three in the mean, at most 1.25 times (1280 x 900 BF16 periodic: walk 13.0,
@@ -55,7 +55,7 @@ FusePlan plan_fused(int store, int nx, int ny, bool walls, int sms, long long le
     FusePlan p{1, 0};
     for (int T = 2; T <= 4 && T <= left && (kinds & FUSE_WALK); T += 2) {
         double c;
-        walk_ranges((nx + WALK_COLS - 1) / WALK_COLS, ny, T, sms, T == 4 ? 4 * walk_minb(4, walls) : 12, &c);
+        walk_ranges((nx + WALK_COLS - 1) / WALK_COLS, ny, T, sms, walls ? 8 : 12, &c);
         if (c * slow / T < best) {
             best = c * slow / T;
             p = {T, 0};
