@@ -765,6 +765,9 @@ lbm_status lbm_cde_autotune(lbm_cde_t h, int64_t steps, int32_t* block_out, int3
     // at least the steps of one launch of the fused kernels
     const int64_t timed = fused_ok(h) ? std::max<int64_t>(steps, lbm::TILE_T) : steps;
     for (size_t ci = 0; ci < cand.size() && s == LBM_OK; ++ci) {
+        bool seen = false;
+        for (size_t cj = 0; cj < ci; ++cj) seen = seen || (cand[cj].block == cand[ci].block && cand[cj].vec == cand[ci].vec);
+        if (seen) continue;
         h->cfg = cand[ci];
         s = lbm_cde_set_state(h, save, t0);
         if (s == LBM_OK) s = lbm_cde_step(h, h->cfg.vec >= 10 ? timed : 2);   // warm: the kernels that are timed
