@@ -963,6 +963,8 @@ struct lbm_cde_batch_s {
     int launch_steps = 0;               // PER_STEP: 0 by the rule of walk_tasks, 1 single steps in whole chunks, BWALK_T
                                         // the walk
     bool walk_whole = false, walk_direct = false;   // the walk in whole chunks (graph replays), in others
+    // the walk's expected time over that of single steps, in whole chunks (graph replays) and in others
+    double walk_ratio = 1e30, walk_ratio_direct = 1e30;
     int ranges = 1;                     // most row ranges of a channel in the walk launches
     int* cblk_inst = nullptr;           // instance of each 256-column block of the moment pass
     int ncblk = 0;
@@ -1157,10 +1159,10 @@ static lbm_status rebuild_tiles(lbm_cde_batch_t b)
 // steps in chunks of 64, 26.3 us a step by single steps, 18.2 by the walk. That counts from 2^18 nodes on.
 // The walk has to be 5 % faster: near the break-even the rule is off by up to a tenth (us a step by the walk and by single
 // steps: 1 x 8192 x 64 10.5 / 7.8, 2 x 8192 x 64 13.2 / 12.0, 8 x 8192 x 17 13.5 / 18.7, 64 x 8192 x 40 141 / 297).
-// *whole, *direct: the choice for whole chunks and for others.
-static void walk_tasks(lbm_cde_batch_t b, std::vector<lbm::BatchTask>& all, bool* whole, bool* direct)
+// walk_ratio: of the times in whole chunks; walk_ratio_direct: in others.
+static void walk_tasks(lbm_cde_batch_t b, std::vector<lbm::BatchTask>& all)
 {
-    *whole = *direct = false;
+    b->walk_ratio = b->walk_ratio_direct = 1e30;   // cannot run
     b->ntasks.clear();
     b->ranges = 1;
     if (9LL * b->ncat >= (1LL << 31)) return;
@@ -1213,9 +1215,17 @@ static void walk_tasks(lbm_cde_batch_t b, std::vector<lbm::BatchTask>& all, bool
     const double walk = 6.0 + rows * (1.1 + 0.4 * k);
     const double hbm = 72.0 * b->ncat > 1.1e8 ? b->ncat * 72 / 5.2e6 : 0;   // both states past L2
     const double single = std::max(6.0 + 6.3e-6 * padded, hbm);
-    const bool all_walk = b->launch_steps == lbm::BWALK_T;
-    *whole = all_walk || (b->launch_steps != 1 && walk < 0.95 * T * single);
-    *direct = all_walk || (b->ncat >= (1LL << 18) && walk < 0.95 * T * std::max(single, 19.0));
+    b->walk_ratio = walk / (T * single);
+    b->walk_ratio_direct = b->ncat >= (1LL << 18) ? walk / (T * std::max(single, 19.0)) : 1e29;
+}
+
+// The walk in whole chunks and in others, where it can run at all: as chosen (BWALK_T), else 5 % faster (chosen single
+// steps, 1, are those of whole chunks).
+static void walk_choice(lbm_cde_batch_t b)
+{
+    const bool can = b->ss.tasks != nullptr, all_walk = b->launch_steps == lbm::BWALK_T;
+    b->walk_whole = can && (all_walk || (b->launch_steps != 1 && b->walk_ratio < 0.95));
+    b->walk_direct = can && (all_walk || b->walk_ratio_direct < 0.95);
 }
 
 static void release_walk(lbm_cde_batch_t b)
@@ -1233,16 +1243,17 @@ static void release_walk(lbm_cde_batch_t b)
     b->ntasks.clear();
 }
 
-// Buffers of the walk launches, where they pay; without memory to spare, one step a launch.
+// Buffers of the walk launches, where they may be used; without memory to spare, one step a launch.
 static lbm_status setup_walk(lbm_cde_batch_t b)
 {
     std::vector<lbm::BatchTask> all;
     try {
-        walk_tasks(b, all, &b->walk_whole, &b->walk_direct);
+        walk_tasks(b, all);
     } catch (const std::bad_alloc&) {
-        b->walk_whole = b->walk_direct = false;
+        b->walk_ratio = b->walk_ratio_direct = 1e30;
     }
-    if (!b->walk_whole && !b->walk_direct) {
+    const bool all_walk = b->launch_steps == lbm::BWALK_T && b->walk_ratio < 1e30;
+    if (!all_walk && (b->launch_steps == 1 || b->walk_ratio >= 0.95) && b->walk_ratio_direct >= 0.95) {
         b->ntasks.clear();
         return LBM_OK;
     }
@@ -1265,7 +1276,7 @@ static lbm_status setup_walk(lbm_cde_batch_t b)
             cudaSuccess ||
         cudaStreamSynchronize(b->st) != cudaSuccess)
         return LBM_E_CUDA;
-    b->ss.tasks = b->tasks;   // one by one where the launch's choice is single steps (launch_batch)
+    b->ss.tasks = b->tasks;
     b->ss.ntasks = b->ntasks.data();
     return LBM_OK;
 }
@@ -1276,17 +1287,25 @@ static lbm_status set_mode(lbm_cde_batch_t b, int mode, int tile_rows)
 {
     const int steps = mode == LBM_BATCH_PER_STEP && (tile_rows == 1 || tile_rows == lbm::BWALK_T) ? tile_rows : 0;
     if (b->mode == mode && b->launch_steps == steps && b->mode_set) return LBM_OK;
-    drop_graph(b);
-    release_walk(b);
+    const bool was = b->walk_whole;
+    if (b->mode != mode) drop_graph(b);
     b->mode = mode;
     b->launch_steps = steps;
     b->mode_set = true;
-    if (mode != LBM_BATCH_PER_STEP) return LBM_OK;
-    const lbm_status s = setup_walk(b);
-    if (s != LBM_OK) {
+    if (mode != LBM_BATCH_PER_STEP) {
         release_walk(b);
-        return bfail(b, s, "walk setup failed");
+        return LBM_OK;
     }
+    if (b->ss.tasks == nullptr) {
+        const lbm_status s = setup_walk(b);
+        if (s != LBM_OK) {
+            release_walk(b);
+            return bfail(b, s, "walk setup failed");
+        }
+    }
+    walk_choice(b);
+    if (b->walk_whole != was) drop_graph(b);
+    if (!b->walk_whole && !b->walk_direct) release_walk(b);
     return LBM_OK;
 }
 
@@ -1613,8 +1632,12 @@ lbm_status lbm_cde_batch_autotune(lbm_cde_batch_t b, int64_t steps, int32_t* mod
     cudaEventCreate(&e1);
     lbm_status s = LBM_OK;
     for (const Cand& c : cand) {
+        // no doubt left by the rule, which is good to a tenth
+        if (c.mode == LBM_BATCH_PER_STEP && c.tile != 1 && b->walk_ratio > 1.4) continue;
         s = lbm_cde_batch_config(b, c.mode, c.tile);
-        if (s == LBM_OK && c.mode == LBM_BATCH_PER_STEP && c.tile != 1 && !b->walk_whole) continue;   // cannot run
+        if (s == LBM_OK && c.mode == LBM_BATCH_PER_STEP &&
+            (c.tile == 1 ? b->walk_direct && b->walk_ratio < 0.7 : !b->walk_whole))
+            continue;
         if (s == LBM_OK) s = lbm_cde_batch_run(b, std::min<int64_t>(timed, b->chunk), nullptr);   // warm
         cudaEventRecord(e0, b->st);
         if (s == LBM_OK) s = lbm_cde_batch_run(b, timed, nullptr);
@@ -1630,14 +1653,11 @@ lbm_status lbm_cde_batch_autotune(lbm_cde_batch_t b, int64_t steps, int32_t* mod
     }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
-    if (s == LBM_OK) s = lbm_cde_batch_config(b, pick.mode, pick.tile);
     if (s == LBM_OK && pick.mode == LBM_BATCH_PER_STEP) {
-        // 0 where the rule agrees
-        const bool walk = b->walk_whole;
-        s = lbm_cde_batch_config(b, pick.mode, 0);
-        if (s == LBM_OK && b->walk_whole != walk) s = lbm_cde_batch_config(b, pick.mode, pick.tile);
-        else pick.tile = 0;
+        if ((b->walk_ratio < 0.95) == (pick.tile != 1)) pick.tile = 0;   // the rule agrees
     }
+    if (s == LBM_OK) s = lbm_cde_batch_config(b, pick.mode, pick.tile);
+    if (s == LBM_OK && b->use_graph) s = ensure_graph(b);   // not left for the first run
     if (s != LBM_OK) {
         bfree(b, save);
         return s;
