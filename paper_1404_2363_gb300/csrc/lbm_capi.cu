@@ -43,6 +43,7 @@ struct lbm_cde_s {
     LaunchCfg cfg{256, 1};
     LaunchCfg cfg0{256, 1};                // the shape the handle started with
     int pair_block = 0;                    // default shape with a velocity field: node pairs with this block (0: none)
+    bool zw_default = false;               // default shape: the z-walk kernel
     cudaStream_t st = nullptr;
     std::string err;
     // adjoint: checkpoints of the forward run, segment recompute buffer, adjoint states
@@ -285,6 +286,15 @@ static int ukind_internal(int k)
     return k == LBM_U_FIELD ? lbm::U_FIELD : (k == LBM_U_ROW_PROFILE ? lbm::U_ROW : lbm::U_NONE);
 }
 
+// The shape of a one-step launch: as set, or the default where its fields are aligned for it.
+static LaunchCfg one_step_cfg(lbm_cde_t h, const StepArgs& a, int uk)
+{
+    if (h->cfg.vec != 0) return h->cfg;
+    if (h->zw_default && lbm::zw_ok(a, uk, 4)) return LaunchCfg{128, 9};
+    if (h->pair_block && uk == lbm::U_FIELD && lbm::pair_ok(a, uk, h->q)) return LaunchCfg{h->pair_block, 5};
+    return h->cfg;
+}
+
 static bool fused_ok(lbm_cde_t h)
 {
     return lbm::fused_ok(h->q, h->ncell);
@@ -453,12 +463,13 @@ lbm_status lbm_cde_create(const lbm_cde_desc* desc, lbm_cde_t* out)
         if ((d.nx + w - 1) / w * w < (d.nx + h->cfg.block - 1) / h->cfg.block * h->cfg.block) h->cfg.block = w;
     h->cfg.vec = 0;   // fused steps where they apply, else one node per thread
     if (h->q == 15 && h->neq && ncell >= (1LL << 20) && 18LL * ncell < (1LL << 31)) {
-        // D3Q15 16-bit forms: the z-walk kernel, or the node pairs, where the rows allow them (256^3 BF16 272 us a
-        // step against 401 with one node per thread; 200 x 101 x 77 39 against 47; but 64^3 10.4 against 8.1).
-        // The pairs' block takes the width that wastes fewest columns, the widest of those (64 x 225 x 163 BF16: 49 us
-        // with 32 threads, 84 with 64, 59 with one node per thread); they pay with a velocity field (FP16
-        // 320 x 101 x 91 without one: 55 against 49)
-        if (d.nx % 64 == 0 && d.ny % 4 == 0) h->cfg = LaunchCfg{128, 9};
+        // D3Q15 16-bit forms: the z-walk kernel (BF16, us a step, and one node per thread: 256^3 with a field 268 / 401,
+        // row profile 220 / 296, at rest 201 / 255, between walls at rest 203 / 358; 64^3 is too small for it, 10.4 / 8.1),
+        // or with a velocity field node pairs (FP16 320 x 101 x 91 at rest 55 / 49). The pairs' block takes the width that
+        // covers fewest columns, the widest of those (64 x 225 x 163 BF16: 49 with 32 threads, 84 with 64). Per column
+        // covered they take 0.77 to 0.87 of the time of one node per thread, so they may cover up to 5/4 of its columns
+        // (142 x 194 x 246, 1.2: 166 / 184; 70 x 150 x 160, 1.33: 56 / 55)
+        if (d.nx % 64 == 0 && d.ny % 4 == 0) h->zw_default = true;
         else if (d.nx % 2 == 0) {
             auto columns = [&](int per) { return (d.nx + per - 1) / per * per; };
             int block = 128;
@@ -571,7 +582,6 @@ lbm_status lbm_cde_step(lbm_cde_t h, int64_t nsteps)
     if (!h->ready) return fail(h, LBM_E_STATE, "set_phi must come before step");
     const bool walls = h->d.bc_lo_y != LBM_BC_PERIODIC;
     const int uk = ukind_internal(h->ukind);
-    const LaunchCfg cfg = h->cfg.vec == 0 && h->pair_block && uk == lbm::U_FIELD ? LaunchCfg{h->pair_block, 5} : h->cfg;
     const bool tma = (h->cfg.vec == 7 || h->cfg.vec == 8) && h->neq && h->q == 9;
     if (tma) {
         const lbm_status ts = ensure_tma_maps(h);
@@ -588,7 +598,7 @@ lbm_status lbm_cde_step(lbm_cde_t h, int64_t nsteps)
             continue;
         }
         if (tma) a.tma = &h->tmaps[h->cur];
-        CK(h, lbm::launch_step(h->q, h->d.storage, uk, walls, cfg, a, h->st));
+        CK(h, lbm::launch_step(h->q, h->d.storage, uk, walls, one_step_cfg(h, a, uk), a, h->st));
         h->cur ^= 1;
         h->t += 1;
         ++n;
@@ -740,8 +750,11 @@ lbm_status lbm_cde_autotune(lbm_cde_t h, int64_t steps, int32_t* block_out, int3
     auto shown = [&](LaunchCfg c) {   // a starting shape as the block and vec that choose the same
         if (c.vec != 0) return c;
         if (fused_ok(h)) return LaunchCfg{128, 10};
-        if (h->pair_block && ukind_internal(h->ukind) == lbm::U_FIELD) return LaunchCfg{h->pair_block, 5};
-        return LaunchCfg{c.block, 1};
+        const LaunchCfg set = h->cfg;
+        h->cfg = c;
+        const LaunchCfg r = one_step_cfg(h, make_args(h, h->cur), ukind_internal(h->ukind));
+        h->cfg = set;
+        return r.vec == 0 ? LaunchCfg{r.block, 1} : r;
     };
     cand.push_back(shown(keep));
     cand.push_back(shown(h->cfg0));

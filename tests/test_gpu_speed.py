@@ -149,3 +149,14 @@ def test_direct_chunks_of_a_batch():
         us.append(best_us(lambda: b.run(56)))
     b.close()
     assert us[0] < 1.15 * us[1]
+
+
+@pytest.mark.parametrize("n,shape", [((64, 128, 130), (64, 1)), ((66, 120, 140), (96, 1))])
+def test_default_of_an_unaligned_velocity(n, shape):
+    """D3Q15 BF16 with a velocity that starts 4 bytes past a boundary: neither the z-walk nor pairs, one node per thread
+    on the block of the row length (half a block's lanes were past the row's end)."""
+    s = solver(n, "bf16", u="none")
+    buf = 0.02 * torch.rand(3 * s.ncell + 1, device="cuda")
+    s.set_velocity(buf[1:].reshape((3,) + s.shape))
+    assert step_us(s) < 1.1 * step_us(s, shape)
+    s.close()
