@@ -467,15 +467,17 @@ lbm_status lbm_cde_create(const lbm_cde_desc* desc, lbm_cde_t* out)
         // row profile 220 / 296, at rest 201 / 255, between walls at rest 203 / 358; 64^3 is too small for it, 10.4 / 8.1),
         // or with a velocity field node pairs (FP16 320 x 101 x 91 at rest 55 / 49). The pairs' block takes the width that
         // covers fewest columns, the widest of those (64 x 225 x 163 BF16: 49 with 32 threads, 84 with 64). Per column
-        // covered they take 0.77 to 0.87 of the time of one node per thread, so they may cover up to 5/4 of its columns
-        // (142 x 194 x 246, 1.2: 166 / 184; 70 x 150 x 160, 1.33: 56 / 55)
+        // covered they take 0.77 to 0.87 of the time of one node per thread, between walls 0.90 to 1.0, so they may cover
+        // up to 5/4 of its columns (142 x 194 x 246, 1.2: 166 / 184; 70 x 150 x 160, 1.33: 56 / 55), between walls no
+        // more than its (290 x 200 x 200, 1.0: 267 / 291; 160^3, 1.2: 105 / 96)
         if (d.nx % 64 == 0 && d.ny % 4 == 0) h->zw_default = true;
         else if (d.nx % 2 == 0) {
             auto columns = [&](int per) { return (d.nx + per - 1) / per * per; };
             int block = 128;
             for (int w = 96; w >= 32; w -= 32)
                 if (columns(2 * w) < columns(2 * block)) block = w;
-            if (4 * columns(2 * block) <= 5 * columns(h->cfg.block)) h->pair_block = block;
+            const bool y_walls = d.bc_lo_y != LBM_BC_PERIODIC;
+            if (4 * columns(2 * block) <= (y_walls ? 4 : 5) * columns(h->cfg.block)) h->pair_block = block;
         }
     }
     h->cfg0 = h->cfg;

@@ -160,3 +160,11 @@ def test_default_of_an_unaligned_velocity(n, shape):
     s.set_velocity(buf[1:].reshape((3,) + s.shape))
     assert step_us(s) < 1.1 * step_us(s, shape)
     s.close()
+
+
+@pytest.mark.parametrize("n", [(150, 100, 100), (160, 120, 120)])
+def test_d3q15_default_between_walls_covers_no_more_columns(n):
+    """Pairs that cover 1.2 times the columns take 1.1 times as long between walls."""
+    s = solver(n, "bf16", "noflux")
+    assert step_us(s) < 1.06 * step_us(s, (160, 1))
+    s.close()
