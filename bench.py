@@ -32,7 +32,7 @@ N_GRID = 4096
 TAU = 1.0
 B_LU = {"f32": 80, "f16": 52, "bf16": 52}      # algorithmic DRAM bytes per lattice update
 WORKLOAD = "D2Q9 modified-MRT Gaussian hill, 4096x4096 periodic, time-varying vortex u, D of Eq. 44 (tau=1)"
-PROFILE = os.path.join(ROOT, "profiles", "step_d2q9_f32_vortex4096.md")
+PROFILE = os.path.join(ROOT, "profiles", "fused_steps_d2q9.md")
 
 
 def peaks():
@@ -45,12 +45,12 @@ def peaks():
         return 6800.0, "fallback"
 
 
-STEP_SOURCES = ["lbm_internal.cuh", "lbm_device.cuh", "lbm_d3q15.cuh", "lbm_pair.cuh", "lbm_pair_d3q15.cuh",
-                "lbm_tma_d2q9.cuh", "lbm_step_inst.cuh", "step_d2q9_f32.cu"]
+STEP_SOURCES = ["lbm_internal.cuh", "lbm_device.cuh", "lbm_d3q15.cuh", "lbm_pair.cuh", "lbm_walk_d2q9.cuh",
+                "walk_d2q9_f32.cu"]
 
 
 def kernel_source_hash():
-    """Hash of the sources that define the D2Q9 FP32 step kernel (the profiled one)."""
+    """Hash of the sources that define the D2Q9 FP32 walk kernel (the profiled one)."""
     h = hashlib.sha256()
     csrc = os.path.join(ROOT, "paper_1404_2363_gb300", "csrc")
     for f in STEP_SOURCES:
@@ -250,8 +250,8 @@ def make_solver(store: str, tau: float = TAU):
 
 
 def time_steps(s, steps, warmup, label=None):
-    """Seconds for `steps` steps after `warmup` untimed ones (CUDA events on the
-    solver's stream). `label` names an NVTX range around the timed launches, so
+    """(Seconds, kernel launches) of `steps` steps after `warmup` untimed ones (CUDA events on
+    the solver's stream; the launches as the solver counts them, each one pass over HBM). `label` names an NVTX range around the timed launches, so
     that a profiler can select exactly the timed region."""
     import torch
 
@@ -262,20 +262,14 @@ def time_steps(s, steps, warmup, label=None):
     e1 = torch.cuda.Event(enable_timing=True)
     if label:
         torch.cuda.nvtx.range_push(label)
+    before = s.launches
     e0.record(st)
     s.step(steps)
     e1.record(st)
     if label:
         torch.cuda.nvtx.range_pop()
     torch.cuda.synchronize()
-    return e0.elapsed_time(e1) / 1e3
-
-
-def passes(vec: int, steps: int) -> int:
-    """Kernel launches, each one pass over HBM, of `steps` steps on the 4096^2 grid:
-    the fused steps (vec 10) take four a launch there, the last ones of a run two
-    and one; every other launch shape one."""
-    return steps // 4 + (0, 1, 1, 2)[steps % 4] if vec == 10 else steps
+    return e0.elapsed_time(e1) / 1e3, s.launches - before
 
 
 def copy_rate_same_size(nbytes: int, reps: int = 20):
@@ -480,7 +474,7 @@ def d3q15_bench(steps: int, storage: str = "f32"):
     del wl
     shape = s.autotune(10)
     k = max(50, min(steps, 600))
-    dt = time_steps(s, k, 5)
+    dt, _ = time_steps(s, k, 5)
     s.close()
     peak, kind = peaks()
     cells = n ** 3
@@ -491,10 +485,10 @@ def d3q15_bench(steps: int, storage: str = "f32"):
             "launch": {"block": shape[0], "vec": shape[1]}}
 
 
-def batch_bytes(mode) -> int:
-    """HBM bytes per lattice update of the 64-channel batch: a PER_STEP launch takes four steps, a
-    persistent one reads and writes the state every step."""
-    return 18 if mode == "per_step" else 72
+def batch_bytes(b) -> float:
+    """HBM bytes per lattice update of a batch in its current configuration: each launch reads and writes
+    the state once for the steps it takes (a persistent one every step)."""
+    return 72 / b.launch_info()[0]
 
 
 def batch_bench(steps: int):
@@ -534,19 +528,20 @@ def batch_bench(steps: int):
         return time.perf_counter() - t0, e0.elapsed_time(e1) / 1e3
 
     dt, dt_dev = timed(n)
+    per_lu = batch_bytes(b)
     modes = {}
     for m, tr in (("persistent", 0), ("persistent", 16), ("per_step", 0)):
         b.config(m, tr)
         w, d = timed(n)
         key = m if m == "per_step" else ("persistent_cell_tiles" if tr == 0 else f"persistent_warp_tiles{tr}")
         modes[key] = {
-            "MLUPS_device": cells * n / d / 1e6, "frac_of_" + kind + "_hbm": cells * batch_bytes(m) / (d / n) / 1e9 / peak}
+            "MLUPS_device": cells * n / d / 1e6, "frac_of_" + kind + "_hbm": cells * batch_bytes(b) / (d / n) / 1e9 / peak}
     b.close()
-    gbs = cells * batch_bytes(mode) / (dt / n) / 1e9
-    gbs_dev = cells * batch_bytes(mode) / (dt_dev / n) / 1e9
+    gbs = cells * per_lu / (dt / n) / 1e9
+    gbs_dev = cells * per_lu / (dt_dev / n) / 1e9
     return {"instances": len(chans), "cells": cells, "steps": n, "MLUPS": cells * n / dt / 1e6,
             "MLUPS_device": cells * n / dt_dev / 1e6,
-            "bytes_per_lu": batch_bytes(mode), "achieved_gbs": gbs, f"frac_of_{kind}_hbm": gbs / peak,
+            "bytes_per_lu": per_lu, "achieved_gbs": gbs, f"frac_of_{kind}_hbm": gbs / peak,
             f"frac_of_{kind}_hbm_device": gbs_dev / peak,
             "mode": mode, "tile_rows": tile, "modes": modes,
             "timing": "MLUPS: host wall clock around lbm_cde_batch_run (graph replays + per-step moment "
@@ -676,7 +671,7 @@ def main():
         t_wall0 = time.time()
         roll(s, 0.6)
         t_timed0 = time.time()
-        dt = time_steps(s, args.steps, args.warmup, label="timed_f32")
+        dt, launches = time_steps(s, args.steps, args.warmup, label="timed_f32")
         t_timed1 = time.time()
         roll(s, 0.6)
         t_wall1 = time.time()
@@ -686,7 +681,6 @@ def main():
     mass_ok = s.sum_phi()
     s.close()
     value = units / dt_max / 1e6
-    launches = passes(f32_shape[1], args.steps)
     avg_launch = dt / launches
     peak, peak_kind = peaks()
     achieved = ncell * B_LU[store] / avg_launch / 1e9
@@ -711,9 +705,8 @@ def main():
         for vs in (("f16", "bf16") if tau == TAU else ("f32", "f16", "bf16")):
             sv, *_ = make_solver(vs, tau)
             shape = sv.autotune(20)
-            dtv = time_steps(sv, args.steps, args.warmup)
+            dtv, np_ = time_steps(sv, args.steps, args.warmup)
             sv.close()
-            np_ = passes(shape[1], args.steps)
             av = ncell * B_LU[vs] / (dtv / np_) / 1e9
             key = vs if tau == TAU else f"{vs}_tau{tau}"
             variants[key] = {"MLUPS": ncell * args.steps / dtv / 1e6, "bytes_per_lu": B_LU[vs] * np_ / args.steps,

@@ -238,6 +238,9 @@ lbm_status lbm_cde_autotune(lbm_cde_t h, int64_t steps, int32_t* block_out, int3
 /* Number of steps taken since the last set_phi / set_state. */
 lbm_status lbm_cde_get_time(lbm_cde_t h, int64_t* t_out);
 
+/* Kernel launches of lbm_cde_step since the handle was made. */
+lbm_status lbm_cde_get_launches(lbm_cde_t h, int64_t* launches_out);
+
 /* Writes phi = sum_i f_i (Eq. 8) of the current state into phi_dev [ncell]
  * (device FP32, caller-owned). Asynchronous. */
 lbm_status lbm_cde_get_phi(lbm_cde_t h, float* phi_dev);

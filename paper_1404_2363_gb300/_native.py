@@ -138,6 +138,7 @@ SIGNATURES = {
     "lbm_cde_batch_run": [_P, _I64, _DP],
     "lbm_cde_batch_autotune": [_P, _I64, ctypes.POINTER(ctypes.c_int32), ctypes.POINTER(ctypes.c_int32)],
     "lbm_cde_batch_config": [_P, ctypes.c_int32, ctypes.c_int32],
+    "lbm_cde_get_launches": [_P, ctypes.POINTER(_I64)],
     "lbm_cde_batch_launch_info": [_P, ctypes.POINTER(ctypes.c_int32), ctypes.POINTER(ctypes.c_int32)],
     "lbm_cde_batch_last_error": [_P],
     "lbm_cde_sum_state_noalloc": [_P, ctypes.c_int32, ctypes.c_int32, _I64, _P, _P],

@@ -39,6 +39,7 @@ struct lbm_cde_s {
     const float* sched = nullptr;
     long long sched_len = 0;
     long long t = 0;
+    long long launches = 0;                // kernel launches of lbm_cde_step
     bool ready = false;
     LaunchCfg cfg{256, 1};
     LaunchCfg cfg0{256, 1};                // the shape the handle started with
@@ -596,6 +597,7 @@ lbm_status lbm_cde_step(lbm_cde_t h, int64_t nsteps)
             CK(h, launch_fused(h, plan, uk, a, nullptr, h->st));
             h->cur ^= 1;
             h->t += plan.T;
+            ++h->launches;
             n += plan.T;
             continue;
         }
@@ -603,6 +605,7 @@ lbm_status lbm_cde_step(lbm_cde_t h, int64_t nsteps)
         CK(h, lbm::launch_step(h->q, h->d.storage, uk, walls, one_step_cfg(h, a, uk), a, h->st));
         h->cur ^= 1;
         h->t += 1;
+        ++h->launches;
         ++n;
     }
     return LBM_OK;
@@ -814,6 +817,13 @@ lbm_status lbm_cde_get_time(lbm_cde_t h, int64_t* t_out)
 {
     if (!h || !t_out) return fail(h, LBM_E_ARG, "NULL argument");
     *t_out = h->t;
+    return LBM_OK;
+}
+
+lbm_status lbm_cde_get_launches(lbm_cde_t h, int64_t* launches_out)
+{
+    if (!h || !launches_out) return fail(h, LBM_E_ARG, "NULL argument");
+    *launches_out = h->launches;
     return LBM_OK;
 }
 

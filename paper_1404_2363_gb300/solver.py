@@ -166,6 +166,13 @@ class Solver:
         self._ck(self.L.lbm_cde_get_time(self.h, ctypes.byref(v)), "lbm_cde_get_time")
         return v.value
 
+    @property
+    def launches(self):
+        """Kernel launches of step() since the handle was made (one of them may take several steps)."""
+        v = ctypes.c_int64()
+        self._ck(self.L.lbm_cde_get_launches(self.h, ctypes.byref(v)), "lbm_cde_get_launches")
+        return v.value
+
     def get_phi(self, out=None):
         if out is None:
             out = torch.empty(self.shape, device=self.device, dtype=torch.float32)

@@ -90,3 +90,15 @@ def test_large_grids_give_the_bits_of_small_ones(storage, n, axis, times, u, bc,
     """A size from which the launch and the loads take another form, as copies of a grid below it."""
     small = repeated(n, axis, 1, storage, u, bc, launch)
     assert bool((repeated(n, axis, times, storage, u, bc, launch) == small).all())
+
+
+@pytest.mark.parametrize("launch,steps,launches", [((256, 1), 11, 11), ((128, 11), 11, 4), ((128, 12), 11, None)])
+def test_launches_are_counted(launch, steps, launches):
+    """One per step, or per group of steps: the walk takes 4 + 4 + 2 + 1; the tiles groups of at most eight."""
+    s = Solver(nx=320, ny=200)
+    s.set_D(np.array(D2))
+    s.set_launch(*launch)
+    s.set_phi(torch.rand((200, 320), device="cuda"))
+    s.step(steps)
+    assert s.launches == launches if launches else 2 <= s.launches < steps
+    s.close()
