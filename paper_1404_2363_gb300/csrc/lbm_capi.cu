@@ -1174,20 +1174,21 @@ lbm_status lbm_cde_backward(lbm_cde_t h, const float* dL_dphiN_dev, float* dL_dp
         if (t == 0) return static_cast<float*>(h->ck[j]);
         return reinterpret_cast<float*>(static_cast<char*>(segbuf[j & 1]) + sb * (t - 1));
     };
-    // The recompute runs beside the reverse steps, which are what the sweep waits for. Several steps a launch take
-    // less time but leave the reverse steps no room (the walk's CTAs hold an SM's registers for tens of us), so on
-    // most grids one step a launch ends the sweep sooner (us of backward a step, fused against single steps: 1024^2
-    // between walls 40.2 / 34.7 with a field and 37.5 / 31.9 without, 1537 x 1023 59.7 / 50.8, 4096^2 with a field
-    // 479 / 457). Fused steps where the sweep waits for the recompute's launches or memory: 128^2 6.6 / 7.0; from 2^22
-    // nodes on without a velocity field (4096^2 397 / 422) and with x walls (705 / 752); and where the caller chose
-    // the walk or the tile kernel.
-    const bool fused = h->cfg.vec == 11 || h->cfg.vec == 12 || h->ncell < (1LL << 15) ||
-                       (h->ncell >= (1LL << 22) && (uk != lbm::U_FIELD || h->d.bc_lo_x != LBM_BC_PERIODIC));
+    // The recompute runs beside the reverse steps, which are what the sweep waits for. Below 2.6M nodes single steps end
+    // it sooner: the walk's CTAs hold an SM's registers for tens of us and leave the reverse steps no room (us of backward
+    // a step, fused / single, 100 steps: 768 x 700 20.0 / 17.5, 1024^2 between walls 35.4 / 33.4, 1537 x 1023 53.0 /
+    // 49.7; 1500^2 68.8 / 68.7). Above, both wait for HBM, which four steps a pass spare (2048^2 113 / 119, 4096^2 424 /
+    // 462); walks of two steps, which store every second state, spare too little (4096^2, segments of seven 511 with one
+    // of them, 436 with single steps in its place), so the steps past the last four run one by one. Below 2^15 nodes the
+    // tiles' fewer launches are as fast; and the caller may have chosen the walk or the tile kernel.
+    const bool chosen = h->cfg.vec == 11 || h->cfg.vec == 12;
+    const bool fused = chosen || h->ncell < (1LL << 15) || h->ncell >= (5LL << 19);
     // recompute B_{jK+1} .. B_{end-1} of segment j from its checkpoint, on stream rs
     auto recompute = [&](int64_t j, cudaStream_t rs) -> lbm_status {
         const int64_t start = j * K, end = std::min(start + K, Nst);
         for (int64_t t = 1; t < end - start;) {
-            const lbm::FusePlan plan = fused ? fuse_plan(h, end - start - t) : lbm::FusePlan{1, 0};
+            lbm::FusePlan plan = fused ? fuse_plan(h, end - start - t) : lbm::FusePlan{1, 0};
+            if (!chosen && plan.T == 2 && plan.rows == 0) plan = {1, 0};
             StepArgs a = make_args(h, 0);
             a.src = seg_state(j, t - 1);
             a.dst = seg_state(j, t + plan.T - 1);

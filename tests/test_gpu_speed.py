@@ -168,3 +168,13 @@ def test_d3q15_default_between_walls_covers_no_more_columns(n):
     s = solver(n, "bf16", "noflux")
     assert step_us(s) < 1.06 * step_us(s, (160, 1))
     s.close()
+
+
+def test_recompute_of_large_grids():
+    """Segments of seven steps on 3000 x 2500: a walk of four, then single steps (with a walk of two 1.18 times as long as
+    with single steps throughout)."""
+    s = solver((3000, 2500))
+    default = backward_us(s, 64)
+    s.set_launch(256, 1)
+    assert default < 1.02 * backward_us(s, 64)
+    s.close()
