@@ -577,8 +577,12 @@ def adjoint_cost(store: str, ms_forward: float, nsteps: int = 400):
         out[f"ratio_backward_vs_forward[{tag}]"] = bwd / ms_forward
         out["forward_ckpt_ms_per_step"] = e[0].elapsed_time(e[1]) / nsteps
     s.close()
-    out["bytes_per_lu_backward"] = {"recompute": 80, "adjoint": 116, "adjoint_with_dL_da": 132}
-    out["note"] = "backward = recompute of each checkpoint segment + one adjoint kernel per step"
+    # per node and step: a walk of four steps reads f and u once (44 B) and stores four
+    # states (36 B each); single steps (small grids, a segment's last one to three) move 80
+    out["bytes_per_lu_backward"] = {"recompute": 47, "recompute_single_step": 80,
+                                    "adjoint": 116, "adjoint_with_dL_da": 132}
+    out["note"] = ("backward = recompute of each checkpoint segment (walks of four steps and the "
+                   "remainder by single steps) + one adjoint kernel per step")
     return out
 
 
