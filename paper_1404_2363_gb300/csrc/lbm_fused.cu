@@ -42,8 +42,8 @@ int walk_ranges(int strips, int ny, int T, int sms, int warps, double* cost)
 // left out. Over 18 grids (333 x 33 to 4096 x 4096), FP32 and BF16, with a field, a row profile and five wall pairs, the
 // choice takes 1.011 times the fastest of the three in the mean, at most 1.25 times (1280 x 900 BF16 periodic: walk 13.0,
 // tile 10.4).
-// The tile kernel wins below about 1M nodes (us a step: 512^2 2.5, walk 8.0, one step 6.2; 896^2 6.4, 9.2,
-// 10.3), the walk above (1024^2: 7.7 against 8.5 and 12.3; 2048^2: 21, 43, 52; 4096^2: 72, 166, 192).
+// The tile kernel wins below about 1M nodes (us a step: 512^2 2.7, walk 5.3, one step 4.1; 896^2 6.6, 9.1,
+// 8.8), the walk above (1024^2: 7.7 against 9.0 and 10.5; 2049^2: 23, 37, 52; 4096^2: 71, 141, 190).
 FusePlan plan_fused(int store, int nx, int ny, bool walls, int sms, long long left, int kinds)
 {
     const double n = (double)nx * ny;

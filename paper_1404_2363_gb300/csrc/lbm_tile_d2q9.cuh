@@ -11,7 +11,7 @@
 // conflict-free wavefront at any shift, and the two nodes form the operands of the
 // paired arithmetic without a move.
 //
-// us a step: 128^2 0.99, 256^2 1.3, 512^2 2.5 (one step a launch: 4.1, 4.1, 6.2).
+// us a step: 128^2 0.92, 256^2 1.3, 512^2 2.7 (one step a launch: 2.1, 2.2, 4.1; not overlapping 4.1, 4.1, 6.2).
 // Bound by the launch and the load (about 3.5 us a launch) on small grids, by
 // issue on larger ones (278 instructions a row of 64 nodes and step at 64
 // registers, 53 % issue active; at 128 registers, one CTA of 16 warps per SM, the

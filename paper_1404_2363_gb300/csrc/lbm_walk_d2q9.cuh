@@ -13,9 +13,9 @@
 // Rows enter through a ring in shared memory, three in flight, by 16-byte cp.async
 // (register prefetch of one row: 105 us a step; 8-byte copies through L1: 74).
 //
-// FP32, 4096^2, T = 4: 72 us a step (HBM traffic per step about 1.5 GB / 4 at
-// 5.2 TB/s, FMA pipe 60 % busy, issue 59 %); 16-bit forms 91 us against 207 (one
-// node per thread) and 120 (TMA-staged), 1024^2 FP32 7.7 against 12.3. Measured and
+// FP32, 4096^2, T = 4: 71 us a step (1.34 GB a launch of four steps, what one step
+// moves, at 4.7 TB/s; issue 60 %, 12 warps per SM); 16-bit forms 86 to 88 us against
+// 207 (one node per thread) and 120 (TMA-staged), 1024^2 FP32 7.7 against 12.3. Measured and
 // not kept: T = 3 at 12 or 16 warps per SM (81 / 102 us), T = 4 at 14 warps per SM
 // (100: spills), T = 2 (130), scalar instead of paired arithmetic (84).
 #pragma once
