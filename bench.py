@@ -275,7 +275,7 @@ def time_steps(s, steps, warmup, label=None):
 def copy_rate_same_size(nbytes: int, reps: int = 20):
     """Read + write GB/s of a device-to-device copy of nbytes (torch copy_),
     best of reps: the copy peak at the size of one step's state, beside the
-    driver's 2 GiB figure in the denominator."""
+    measured 2 GiB copy in the denominator."""
     import torch
 
     a = torch.empty(nbytes // 4, dtype=torch.float32, device="cuda")
